@@ -66,11 +66,10 @@ struct alignas(8) Limbs {
 };
 
 QAOA_HD Limbs split(long long x) {
-  const int l = (int)(unsigned int)(unsigned long long)x;
-  const int h = (int)((x - (long long)l) >> 32);
+  const unsigned int l = (unsigned int)(unsigned long long)x;
   Limbs r;
-  r.h = h;
-  r.l = l;
+  r.l = (int)l;
+  r.h = (int)((unsigned int)((unsigned long long)x >> 32) + (l >> 31));  // a negative l borrows one from h
   return r;
 }
 
@@ -100,14 +99,24 @@ QAOA_HD long long dot2_q62(Limbs a, Limbs b, Limbs c, Limbs d, int e) {
   return (P + ((T + (1ll << (29 + e))) >> 32)) >> (e - 2);
 }
 
+// (a b + c d + half 2^32) / 2^64 rounded down, without the products of the low limbs: half
+// starts the middle sum and the middle sum's high word starts the high sum, so rounding and
+// carrying cost no additions of their own (a 64-bit add occupies the integer pipes as long as
+// a product does; the complex multiplies of the sweeps lose 16 of their 32 add and shift
+// instructions this way)
+QAOA_HD long long dot2_hi64(Limbs a, Limbs b, Limbs c, Limbs d, long long half) {
+  const long long T = madw(c.l, d.h, madw(c.h, d.l, madw(a.l, b.h, madw(a.h, b.l, half))));
+  return madw(c.h, d.h, madw(a.h, b.h, T >> 32));
+}
+
 // dot2_q62 without the products of the low limbs: they add at most 2^(1 - e) result units,
 // so for e >= 3 the result is within one unit of exact rounding (two fewer 32 x 32-bit
 // products per call)
 QAOA_HD long long dot2_q62_hi(Limbs a, Limbs b, Limbs c, Limbs d, int e) {
+  if (e > 2) return dot2_hi64(a, b, c, d, 1ll << (29 + e)) >> (e - 2);
   const long long P = madw(c.h, d.h, madw(a.h, b.h, 0));
-  const long long T = madw(c.l, d.h, madw(c.h, d.l, madw(a.l, b.h, madw(a.h, b.l, 0))));
-  if (e <= 2) return (long long)((unsigned long long)P << (2 - e)) + ((T + (1ll << (29 + e))) >> (30 + e));
-  return (P + ((T + (1ll << (29 + e))) >> 32)) >> (e - 2);
+  const long long T = madw(c.l, d.h, madw(c.h, d.l, madw(a.l, b.h, madw(a.h, b.l, 1ll << (29 + e)))));
+  return (long long)((unsigned long long)P << (2 - e)) + (T >> (30 + e));
 }
 
 // Exact 128-bit products from four 32 x 32-bit limb products each (fused multiply-add-wide
@@ -196,6 +205,74 @@ QAOA_HD C64 cmul_factor(long long xr, long long xi, const Factor& f, int e) {
   }
   return o;
 }
+
+// cmul_factor<false, false> for e >= 3, on limbs the caller has split
+QAOA_HD C64 cmul_big(Limbs r, Limbs i, const Factor& f, int e) {
+  C64 o;
+  o.x = dot2_hi64(r, f.r, i, f.ni, 1ll << (29 + e)) >> (e - 2);
+  o.y = dot2_hi64(r, f.i, i, f.r, 1ll << (29 + e)) >> (e - 2);
+  return o;
+}
+
+// x * u / 2^62 (conj(u) when CONJ) for |re x|, |im x| < 2^59: the operand is scaled by 4 first,
+// so the rounded sum is the high word pair itself (no shift after the products) and the
+// dropped low x low products stay below half a unit: within one unit of exact rounding.
+template <bool CONJ>
+QAOA_HD C64 cmul_unit(long long xr, long long xi, const Factor& f) {
+  const Limbs r = split((long long)((unsigned long long)xr << 2)), i = split((long long)((unsigned long long)xi << 2));
+  const Limbs& ui = CONJ ? f.ni : f.i;
+  const Limbs& nui = CONJ ? f.i : f.ni;
+  C64 o;
+  o.x = dot2_hi64(r, f.r, i, nui, 1ll << 31);
+  o.y = dot2_hi64(r, ui, i, f.r, 1ll << 31);
+  return o;
+}
+
+// Running sums of Im(conj(w) v) = w.x v.y - w.y v.x by limb weight: value = P 2^64 + M 2^32 +
+// L 2^4.  One multiply-add-wide per limb product and no carries between products (an exact
+// 128-bit product and sum per term took ~80 instructions per amplitude, this ~15); the four
+// lowest bits of w are left out of the low x low products only (2^-73 of a unit product).
+// Sums of up to 8 terms with weights 0..3 fit int64 when the 2-norms of w and of v over the
+// terms are at most 1.1 x 2^60: |h| norms are then at most 1.1 x 2^28 and each of M's two
+// halves at most that x 2^31 sqrt(2 sum of squared weights <= 48) < 2^62.
+struct ImSum {
+  unsigned long long P = 0, M = 0, L = 0;
+  QAOA_HD void add(Limbs vx, Limbs vy, Limbs wx, Limbs wy) {
+    const int nwyh = -wy.h, nvxh = -vx.h, wxl = wx.l >> 4, nwyl = -(wy.l >> 4);
+    P = (unsigned long long)madw(nwyh, vx.h, madw(wx.h, vy.h, (long long)P));
+    M = (unsigned long long)madw(wy.l, nvxh, madw(nwyh, vx.l, madw(wx.l, vy.h, madw(wx.h, vy.l, (long long)M))));
+    L = (unsigned long long)madw(nwyl, vx.l, madw(wxl, vy.l, (long long)L));
+  }
+  // this += m s for a small m (modulo 2^64: intermediate sums may wrap)
+  QAOA_HD void add_times(const ImSum& s, int m) {
+    if (m == 0) return;
+    P += s.P * (unsigned long long)(long long)m;
+    M += s.M * (unsigned long long)(long long)m;
+    L += s.L * (unsigned long long)(long long)m;
+  }
+  QAOA_HD i128 value() const {
+    return ((i128)(long long)P << 64) + ((i128)(long long)M << 32) + ((i128)(long long)L << 4);
+  }
+};
+
+// sum of c Im(conj(w) v) for integer c, |c| <= 2^28, and |components| < 2^56 (up to 8 terms):
+// the term is P 2^64 + Q 2^32 with the low products folded into Q, and each word of P and Q is
+// weighted by c with one multiply-add-wide.  value = sum >> 32.
+struct WeightedImSum {
+  long long ph = 0, pl = 0, qh = 0, ql = 0;
+  QAOA_HD void add(long long vx_, long long vy_, long long wx_, long long wy_, int c) {
+    const Limbs vx = split(vx_), vy = split(vy_), wx = split(wx_), wy = split(wy_);
+    const int nwyh = -wy.h, nvxh = -vx.h, wxl = wx.l >> 4, nwyl = -(wy.l >> 4);
+    const long long Lo = madw(nwyl, vx.l, madw(wxl, vy.l, 1ll << 27)) >> 28;
+    const Limbs Q = split(madw(wy.l, nvxh, madw(nwyh, vx.l, madw(wx.l, vy.h, madw(wx.h, vy.l, Lo)))));
+    const Limbs P = split(madw(nwyh, vx.h, madw(wx.h, vy.h, 0)));
+    ph = madw(P.h, c, ph);
+    pl = madw(P.l, c, pl);
+    qh = madw(Q.h, c, qh);
+    ql = madw(Q.l, c, ql);
+  }
+  QAOA_HD i128 value() const { return ((i128)ph << 64) + ((i128)pl << 32) + ((i128)qh << 32) + (i128)ql; }
+};
 
 // float64 of x * 2^-s, correctly rounded (round to nearest, ties to even), assembled from
 // the binary64 layout sign | 11-bit biased exponent | 52-bit fraction.  The result must be

@@ -109,12 +109,12 @@ __device__ __forceinline__ uint64_t local_to_z(const SweepGeom& g, uint64_t base
 using i128 = __int128;
 using fx::round_shift;
 
-// (x * e) / 2^(62 + extra) for a state value x (|re|, |im| < 2^61) and a Q62 unit complex e
-__device__ __forceinline__ longlong2 cmul_fx(longlong2 x, longlong2 e, int extra) {
-  const fx::C64 o = fx::cmul_q62(x.x, x.y, e.x, e.y, extra);
+// x * e / 2^62 for a state value x between mixers (|re|, |im| < 2^59) and a Q62 unit complex e
+__device__ __forceinline__ longlong2 cmul_fx(longlong2 x, longlong2 e) {
+  const fx::C64 o = fx::cmul_unit<false>(x.x, x.y, fx::factor(e.x, e.y));
   return make_longlong2(o.x, o.y);
 }
-// the same with 128-bit products, for operands up to 2^63 (products of two Q62 factors)
+// (x * e) / 2^(62 + extra) with 128-bit products, for operands up to 2^63 (products of two Q62 factors)
 __device__ __forceinline__ longlong2 cmul_fx_wide(longlong2 x, longlong2 e, int extra) {
   const fx::C64 o = fx::cmul_q62_exact(x.x, x.y, e.x, e.y, extra);
   return make_longlong2(o.x, o.y);
@@ -340,7 +340,7 @@ struct Sweeper {
   // ---------------------------------------------------------------- phase
   __device__ __forceinline__ static V vmul(V x, V e) {
     if constexpr (FX) {
-      return cmul_fx(x, e, 0);
+      return cmul_fx(x, e);
     } else {
       return make_float2(x.x * e.x - x.y * e.y, x.x * e.y + x.y * e.x);
     }
@@ -364,7 +364,7 @@ struct Sweeper {
         const uint32_t k = (uint32_t)cost_i(Cs, idx(r)) - (uint32_t)pcmin;
         if (k < (uint32_t)pspan) {
           if constexpr (FX) {
-            const fx::C64 o = fx::cmul_factor<false, INV>(u[r].x, u[r].y, Tf[k], 0);
+            const fx::C64 o = fx::cmul_unit<INV>(u[r].x, u[r].y, Tf[k]);
             u[r] = make_longlong2(o.x, o.y);
           }
         } else {
@@ -414,8 +414,8 @@ struct Sweeper {
         if (k < (uint32_t)pspan) {
           if constexpr (FX) {
             const fx::Factor& f = Tf[k];
-            const fx::C64 o = fx::cmul_factor<false, INV>(v[r].x, v[r].y, f, 0);
-            const fx::C64 q = fx::cmul_factor<false, INV>(w[r].x, w[r].y, f, 0);
+            const fx::C64 o = fx::cmul_unit<INV>(v[r].x, v[r].y, f);
+            const fx::C64 q = fx::cmul_unit<INV>(w[r].x, w[r].y, f);
             v[r] = make_longlong2(o.x, o.y);
             w[r] = make_longlong2(q.x, q.y);
           }
@@ -744,17 +744,27 @@ struct Sweeper {
     const bool f64 = a.cost_dtype == QAOA_COST_F64;
     double e0 = 0.0;
     if constexpr (FX) {
-      i128 sc = 0;
-      double sf = 0.0;
+      if (R <= 8 && !f64 && lam_shift <= 28) {  // |C| <= 2^28: limb sums (fx::WeightedImSum)
+        fx::WeightedImSum sw;
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const uint32_t i = idx(r);
-        if (i >= evalid) continue;
-        const i128 pr = fx::dot2_exact(w[r].x, v[r].y, w[r].y, v[r].x);
-        if (!f64) sc += (pr >> 32) * cost_i(Cs, i);
-        else sf += cost_f(Cs, true, i) * i128_to_double(pr, 2 * a.fx_shift - lam_shift);
+        for (int r = 0; r < R; ++r) {
+          const uint32_t i = idx(r);
+          if (i < evalid) sw.add(v[r].x, v[r].y, w[r].x, w[r].y, cost_i(Cs, i));
+        }
+        e0 = i128_to_double(sw.value(), 2 * a.fx_shift - 32 - lam_shift);
+      } else {
+        i128 sc = 0;
+        double sf = 0.0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const uint32_t i = idx(r);
+          if (i >= evalid) continue;
+          const i128 pr = fx::dot2_exact(w[r].x, v[r].y, w[r].y, v[r].x);
+          if (!f64) sc += (pr >> 32) * cost_i(Cs, i);
+          else sf += cost_f(Cs, true, i) * i128_to_double(pr, 2 * a.fx_shift - lam_shift);
+        }
+        e0 = f64 ? sf : i128_to_double(sc, 2 * a.fx_shift - 32 - lam_shift);
       }
-      e0 = f64 ? sf : i128_to_double(sc, 2 * a.fx_shift - 32 - lam_shift);
     } else {
       float s[4] = {0.f, 0.f, 0.f, 0.f};  // independent partial sums
 #pragma unroll
@@ -1027,13 +1037,44 @@ struct Lean : Sweeper<CF, FX, TWO> {
       fx_back<K - 1>(lam);
     }
   }
-  template <int L, bool BIG>
+  template <int L>
   __device__ __forceinline__ void dmul_l(V (&u)[R], const fx::Factor* Ds, int gl, int t) {
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       const fx::Factor& f = Ds[__popc((ix<L>(r) >> gl) & ((1u << t) - 1))];
-      const fx::C64 o = fx::cmul_factor<!BIG, false>(u[r].x, u[r].y, f, t);
+      const fx::C64 o = fx::cmul_big(fx::split(u[r].x), fx::split(u[r].y), f, t);
       u[r] = make_longlong2(o.x, o.y);
+    }
+  }
+  // D on psi and lambda, with the X-term 2 Im <lam|sum_j X_j|psi> = 2^-t sum_z (t - 2 popcount)
+  // 2 Im conj(lam~) psi~ taken from the same limbs: the popcount of an index is the thread's
+  // part pt plus popcount(r & gm), gm = the register bits that are group bits, so a thread's
+  // sum is (t - 2 pt) S - 2 T with S = sum_r pr_r and T = sum_r popcount(r & gm) pr_r.  T by
+  // summation by parts: walking r downwards, T collects the running S times the step of
+  // popcount(r & gm) to the next r (steps of +-1 at a few places; modulo 2^64, the final
+  // sums fit).
+  template <int L>
+  __device__ __forceinline__ void dmul_xterm(const fx::Factor* Ds, int gl, int t, int xacc) {
+    static_assert(R <= 8, "ImSum: sums of up to 8 terms");
+    const uint32_t gmask = (1u << t) - 1;
+    const int pt = __popc((ix<L>(0) >> gl) & gmask);
+    const uint32_t gm = ((gmask << gl) >> CF::lo(L)) & (uint32_t)(R - 1);
+    fx::ImSum S, T;
+#pragma unroll
+    for (int r = R - 1; r >= 0; --r) {
+      const fx::Limbs vx = fx::split(this->v[r].x), vy = fx::split(this->v[r].y);
+      const fx::Limbs wx = fx::split(this->w[r].x), wy = fx::split(this->w[r].y);
+      S.add(vx, vy, wx, wy);
+      const int pr = __popc(r & gm);
+      if (r > 0) T.add_times(S, pr - __popc((r - 1) & gm));
+      const fx::Factor& f = Ds[pt + pr];
+      const fx::C64 o = fx::cmul_big(vx, vy, f, t), q = fx::cmul_big(wx, wy, f, t);
+      this->v[r] = make_longlong2(o.x, o.y);
+      this->w[r] = make_longlong2(q.x, q.y);
+    }
+    if (xacc >= 0) {
+      const i128 xs = S.value() * (t - 2 * pt) - 2 * T.value();
+      this->block_add(xacc, 2.0 * i128_to_double(xs, 2 * this->a.fx_shift + t - this->lam_shift), 0.0, false);
     }
   }
   // W D W from layout 0 back to layout 0; D at layout L (the last round with group qubits)
@@ -1047,46 +1088,11 @@ struct Lean : Sweeper<CF, FX, TWO> {
     }
     fx_fwd<0, L>(lam);
     if (dpre == nullptr) __syncthreads();
+    // lean sweeps run only on groups of t >= 3 qubits, so the shift form of the multiply applies
     if constexpr (TWO) {
-      if (xacc >= 0) {
-        // sum_r pr_r (t - 2 popcount(group bits of index r)); the index is the thread's
-        // bits OR r << lo(L), so the popcount is the thread's part pt plus popcount(r & gm),
-        // gm = the register bits that are group bits, and the sum is
-        // (t - 2 pt) S - 2 sum_{b in gm} U_b with S = sum_r pr_r, U_b = sum_{r: bit b} pr_r
-        // (exact int128 sums of products below 2^123, shifted once before the weighting)
-        const uint32_t gmask = (1u << t) - 1;
-        const int pt = __popc((ix<L>(0) >> gl) & gmask);
-        const uint32_t gm = (((uint32_t)gmask << gl) >> CF::lo(L)) & (uint32_t)(R - 1);
-        i128 S = 0, U[CF::RB];
-#pragma unroll
-        for (int b = 0; b < CF::RB; ++b) U[b] = 0;
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-          const i128 pr = fx::dot2_exact(this->w[r].x, this->v[r].y, this->w[r].y, this->v[r].x);
-          S += pr;
-#pragma unroll
-          for (int b = 0; b < CF::RB; ++b)
-            if (r & (1 << b)) U[b] += pr;
-        }
-        i128 xs = (S >> 32) * (t - 2 * pt);
-#pragma unroll
-        for (int b = 0; b < CF::RB; ++b)
-          if (gm & (1u << b)) xs -= (U[b] >> 32) * 2;
-        this->block_add(xacc, 2.0 * i128_to_double(xs, 2 * this->a.fx_shift + t - 32 - this->lam_shift), 0.0, false);
-      }
-    }
-    // lean sweeps run only on groups of >= 3 qubits, so the shift form of the multiply
-    // applies; the two-buffer kernels keep the branch (it schedules better there)
-    if constexpr (TWO) {
-      if (t >= 3) {
-        dmul_l<L, true>(this->v, Ds, gl, t);
-        if (lam) dmul_l<L, true>(this->w, Ds, gl, t);
-      } else {
-        dmul_l<L, false>(this->v, Ds, gl, t);
-        if (lam) dmul_l<L, false>(this->w, Ds, gl, t);
-      }
+      dmul_xterm<L>(Ds, gl, t, xacc);
     } else {
-      dmul_l<L, true>(this->v, Ds, gl, t);
+      dmul_l<L>(this->v, Ds, gl, t);
     }
     fx_back<L>(lam);
   }
