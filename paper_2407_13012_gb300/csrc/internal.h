@@ -202,7 +202,7 @@ struct SampleArgs {
   uint64_t* z;
   double* cost;
   double* leaf;     // 2^n / leaf_size leaf sums, then exclusive prefix (+1 total)
-  double* blocksum; // scan scratch
+  double* sub;      // running sums at the eighths of each full 2^10 leaf (8 per leaf)
   int leaf_bits;
 };
 cudaError_t launch_sample(const SampleArgs& a, cudaStream_t s);

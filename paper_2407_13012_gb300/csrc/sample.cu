@@ -2,10 +2,11 @@
 // objective value (Sec. IV-D).
 //
 // The state is cut into leaves of 2^leaf_bits amplitudes.  (1) one read sweep sums
-// |psi|^2 per leaf; (2) an exclusive scan turns the leaf sums into a prefix array
-// whose last entry is the total; (3) one warp per shot draws u_i from the SplitMix64
-// counter stream, finds the leaf holding u_i * total by binary search in the prefix,
-// and scans that leaf with a warp prefix sum to find
+// |psi|^2 per leaf, and notes the running sum at every eighth of a full leaf; (2) an
+// exclusive scan turns the leaf sums into a prefix array whose last entry is the total;
+// (3) one warp per shot draws u_i from the SplitMix64 counter stream, finds the leaf
+// holding u_i * total by a 32-way search in the prefix, the eighth by its running sums, and
+// scans from there with a warp prefix sum to find
 //   z_i = min{z : P(z) > u_i * P_total}.
 // Every sum runs in float64 in a fixed order, so a given seed always yields the same
 // samples on a given device.
@@ -16,6 +17,11 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kChunk = kThreads * 16;  // leaves per scan block
+// running sums kept inside a full 1024-entry leaf, at its eighths (8 slots, the last unused):
+// GB300 retires two float64 additions per SM and clock, and the draw's prefix sums over whole
+// leaves (8 additions per 32 entries, 16 times per shot on average) were bound by them
+constexpr int kSubs = 8;
+constexpr int kSubLen = 1024 / kSubs;
 
 __device__ __forceinline__ uint64_t mix64(uint64_t z) {
   z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
@@ -30,6 +36,11 @@ __device__ __forceinline__ double prob_at(const void* psi, int dtype, uint64_t z
   }
   const float2 v = __ldg((const float2*)psi + z);
   return (double)v.x * v.x + (double)v.y * v.y;
+}
+
+// whether full leaves are summed by 16-byte loads, with running sums at their eighths
+__device__ __forceinline__ bool leaf_vec(const SampleArgs& a) {
+  return a.leaf_bits == 10 && ((uintptr_t)a.psi & 15) == 0;
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -55,6 +66,30 @@ struct F2Sum {
   __device__ __forceinline__ double value() const { return (double)s + (double)c; }
 };
 
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+  s = a + b;
+  const float bp = s - a;
+  e = (a - (s - bp)) + (b - bp);
+}
+
+// Lane sums of x[0..7] over the warp, x[k] ending on lanes with bits 4, 3, 2 = bits 2, 1, 0 of k:
+// each step halves the values a lane still carries (9 additions instead of 40).
+template <class T, class ADD>
+__device__ __forceinline__ T warp_sum8(T (&x)[8], ADD&& add) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int h = 4, o = 16; h >= 1; h >>= 1, o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const T keep = up ? x[k + h] : x[k], give = up ? x[k] : x[k + h];
+      x[k] = add(keep, give, o);
+    }
+  }
+  x[0] = add(x[0], x[0], 2);
+  return add(x[0], x[0], 1);
+}
+
 // (1) one warp per leaf; a.len entries (the last leaf may be partly past the end).  Full
 // leaves of an aligned vector take 16-byte loads, all issued before the sums (complex128:
 // one amplitude per load, two independent float64 FMA chains; complex64: two amplitudes
@@ -65,14 +100,14 @@ __global__ void leaf_sum_kernel(const __grid_constant__ SampleArgs a) {
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const uint32_t L = 1u << a.leaf_bits;
   const int64_t nleaf = (int64_t)((a.len + L - 1) >> a.leaf_bits);
-  const bool vec = a.leaf_bits == 10 && ((uintptr_t)a.psi & 15) == 0;
+  const bool vec = leaf_vec(a);
   for (int64_t li = warp; li < nleaf; li += nwarps) {
     const uint64_t base = (uint64_t)li << a.leaf_bits;
     double s = 0.0;
     if (vec && base + L <= a.len) {
       if (a.dtype == QAOA_C128) {
         const double2* q = (const double2*)a.psi + base + lane;
-        double s0 = 0.0, s1 = 0.0;
+        double s0 = 0.0, s1 = 0.0, run[kSubs];
 #pragma unroll
         for (int m0 = 0; m0 < 32; m0 += 8) {
           double2 v[8];
@@ -82,12 +117,18 @@ __global__ void leaf_sum_kernel(const __grid_constant__ SampleArgs a) {
           for (int m = 0; m < 8; ++m) {
             s0 = fma(v[m].x, v[m].x, s0);
             s1 = fma(v[m].y, v[m].y, s1);
+            if ((m & 3) == 3) run[(m0 + m) >> 2] = s0 + s1;
           }
         }
-        s = s0 + s1;
+        s = run[kSubs - 1];
+        const double t = warp_sum8(run, [](double keep, double give, int o) {
+          return keep + __shfl_xor_sync(0xffffffffu, give, o);
+        });
+        if ((lane & 3) == 0) a.sub[li * kSubs + (lane >> 2)] = t;
       } else {
         const float4* q = (const float4*)a.psi + (base >> 1) + lane;
         F2Sum f0, f1;
+        float2 run[kSubs];
 #pragma unroll
         for (int m0 = 0; m0 < 16; m0 += 8) {
           float4 v[8];
@@ -99,9 +140,22 @@ __global__ void leaf_sum_kernel(const __grid_constant__ SampleArgs a) {
             f1.add_sq(v[m].y);
             f0.add_sq(v[m].z);
             f1.add_sq(v[m].w);
+            if (m & 1) {
+              float2& x = run[(m0 + m) >> 1];
+              two_sum(f0.s, f1.s, x.x, x.y);
+              x.y += f0.c + f1.c;
+            }
           }
         }
         s = f0.value() + f1.value();
+        const float2 t = warp_sum8(run, [](float2 keep, float2 give, int o) {
+          const float gx = __shfl_xor_sync(0xffffffffu, give.x, o), gy = __shfl_xor_sync(0xffffffffu, give.y, o);
+          float2 r;
+          two_sum(keep.x, gx, r.x, r.y);
+          r.y += keep.y + gy;
+          return r;
+        });
+        if ((lane & 3) == 0) a.sub[li * kSubs + (lane >> 2)] = (double)t.x + (double)t.y;
       }
     } else {
       for (uint32_t k = lane; k < L && base + k < a.len; k += 32) s += prob_at(a.psi, a.dtype, base + k);
@@ -180,6 +234,7 @@ __global__ void draw_kernel(const __grid_constant__ SampleArgs a, const double* 
   const uint32_t L = 1u << a.leaf_bits;
   const int64_t nleaf = (int64_t)((a.len + L - 1) >> a.leaf_bits);
   const double total = prefix[nleaf];
+  const bool vec = leaf_vec(a);
   const uint64_t sbase = mix64(mix64(a.seed) ^ 0x5f5f656c706d6173ull);
   for (int64_t i = warp; i < a.shots; i += nwarps) {
     const uint64_t x = mix64(sbase + (uint64_t)(i + 1) * 0x9E3779B97F4A7C15ull);
@@ -187,9 +242,11 @@ __global__ void draw_kernel(const __grid_constant__ SampleArgs a, const double* 
     const double target = u * total;
     // largest leaf li with prefix[li] <= target and positive mass; all lanes agree
     int64_t lo = 0, hi = nleaf;  // invariant: prefix[lo] <= target, answer in [lo, hi)
-    while (hi - lo > 1) {
-      const int64_t mid = (lo + hi) >> 1;
-      if (prefix[mid] <= target) lo = mid; else hi = mid;
+    while (hi - lo > 1) {  // the lanes probe 32 places of the range at once
+      const int64_t step = (hi - lo + 31) >> 5, at = lo + lane * step;
+      const unsigned le = __ballot_sync(0xffffffffu, at < hi && prefix[at] <= target) | 1u;
+      lo += (31 - __clz(le)) * step;
+      if (lo + step < hi) hi = lo + step;
     }
     int64_t li = lo;
     bool past_end = !(target < total);
@@ -202,8 +259,18 @@ __global__ void draw_kernel(const __grid_constant__ SampleArgs a, const double* 
     const uint32_t Lh = a.len - base < L ? (uint32_t)(a.len - base) : L;  // entries in this leaf
     const double rem = target - prefix[li];
     double run = 0.0;
+    uint32_t k1 = 0;  // first entry of the eighth that holds the target (0 without running sums)
+    if (vec && !past_end && Lh == L) {
+      const double r = lane < kSubs - 1 ? __ldg(a.sub + li * kSubs + lane) : 0.0;
+      const unsigned le = __ballot_sync(0xffffffffu, lane < kSubs - 1 && r <= rem);
+      if (le) {
+        const int j = 31 - __clz(le);
+        k1 = (uint32_t)(j + 1) * kSubLen;
+        run = __shfl_sync(0xffffffffu, r, j);
+      }
+    }
     int64_t found = -1, last_nz = -1;
-    for (uint32_t k0 = 0; k0 < Lh && found < 0; k0 += 32) {
+    for (uint32_t k0 = k1; k0 < Lh && found < 0; k0 += 32) {
       const uint32_t k = k0 + lane;
       const double pk = (k < Lh) ? prob_at(a.psi, a.dtype, base + k) : 0.0;
       double incl = pk;
@@ -216,6 +283,11 @@ __global__ void draw_kernel(const __grid_constant__ SampleArgs a, const double* 
       if (nzm) last_nz = k0 + 31 - __clz(nzm);
       if (hit) found = k0 + __ffs(hit) - 1;
       run += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    for (uint32_t k0 = k1; found < 0 && last_nz < 0 && k0 > 0;) {  // rounding left the target past
+      k0 -= 32;                                                       // this leaf's last nonzero entry
+      const unsigned nzm = __ballot_sync(0xffffffffu, prob_at(a.psi, a.dtype, base + k0 + lane) > 0.0);
+      if (nzm) last_nz = k0 + 31 - __clz(nzm);
     }
     if (found < 0) found = (last_nz >= 0 && total > 0.0) ? last_nz : (int64_t)Lh - 1;
     if (lane == 0) {
@@ -239,7 +311,7 @@ size_t sample_ws_bytes_len(uint64_t len) {
   const int lb = leaf_bits_for_len(len);
   const int64_t nleaf = (int64_t)((len + (1ull << lb) - 1) >> lb);
   const int64_t nchunks = (nleaf + kChunk - 1) / kChunk;
-  return (size_t)(nleaf + (nleaf + 1) + (nchunks + 1)) * sizeof(double) + 3 * 256;
+  return (size_t)(nleaf + (nleaf + 1) + (nchunks + 1) + (lb == 10 ? kSubs * nleaf : 0)) * sizeof(double) + 4 * 256;
 }
 
 size_t sample_ws_bytes(int n, int /*dtype*/) { return sample_ws_bytes_len(1ull << n); }
@@ -260,6 +332,7 @@ cudaError_t launch_sample(const SampleArgs& a0, cudaStream_t s) {
   double* leaf = (double*)carve(nleaf * sizeof(double));
   double* prefix = (double*)carve((nleaf + 1) * sizeof(double));
   double* bsum = (double*)carve((nchunks + 1) * sizeof(double));
+  a.sub = (double*)carve((a.leaf_bits == 10 ? kSubs * nleaf : 0) * sizeof(double));
   a.leaf = leaf;
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
