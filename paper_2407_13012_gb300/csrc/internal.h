@@ -137,6 +137,13 @@ struct TableArgs {
   void* turn;    // fixed point: 3 * 1024 entries
 };
 
+// lean sweeps (lean_*.cu) of the sweep's shape, with sm bytes of dynamic shared memory
+void lean_x1(const SweepArgs& a, size_t sm, cudaStream_t s);         // complex128, one buffer
+void lean_x2_mix(const SweepArgs& a, size_t sm, cudaStream_t s);     // complex128, two buffers: one mixer
+void lean_x2_ops(const SweepArgs& a, size_t sm, cudaStream_t s);     // complex128, two buffers: op programs
+void lean_f1(const SweepArgs& a, size_t sm, cudaStream_t s);         // complex64, one buffer
+void lean_f2(const SweepArgs& a, size_t sm, cudaStream_t s);         // complex64, two buffers
+
 // launchers (return a CUDA error code)
 cudaError_t launch_sweep(int dtype, bool two, const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_reduce(const ReducePlan& r, const double* partials, double* out, cudaStream_t s);

@@ -1,0 +1,10 @@
+// Lean sweeps of complex128 (fixed-point) psi and lambda: op programs.
+#include "lean_kernel.cuh"
+
+namespace qaoa {
+
+void lean_x2_ops(const SweepArgs& a, size_t sm, cudaStream_t s) {
+  lean_launch_last<CfgX2, true, true, true>(a, sm, s);
+}
+
+}  // namespace qaoa

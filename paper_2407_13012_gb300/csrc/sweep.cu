@@ -1,111 +1,11 @@
 // Layer sweeps: phase separator, mixer, lambda = C psi and the fused reductions of <C>,
 // the norm and the adjoint-gradient terms (Eq. 1; Sec. II-B, IV-B, IV-C, IV-D); the tile
 // machinery and the arithmetic are described in sweeper.cuh.
-#include "sweeper.cuh"
+#include "lean_kernel.cuh"
 
 namespace qaoa {
 namespace {
 
-
-// One layer's phase table (the sweeper's graph's) in shared memory: float32 factors as they
-// are, fixed-point factors prepared for the limb multiply (fx::Factor, 24 bytes per entry).
-// Callers synchronise.
-template <bool FX, class S>
-__device__ __forceinline__ void stage_table(S& s, const SweepArgs& a, void* dst, int nt) {
-  using V = typename S::V;
-  const V* src = (const V*)s.ptab + (long long)a.smem_table_layer * s.pspan;
-  if constexpr (FX) {
-    fx::Factor* tf = (fx::Factor*)dst;
-    for (int k = threadIdx.x; k < s.pspan; k += nt) {
-      const longlong2 e = __ldg((const longlong2*)src + k);
-      tf[k] = fx::factor(e.x, e.y);
-    }
-    s.Tf = tf;
-  } else {
-    V* ts = (V*)dst;
-    for (int k = threadIdx.x; k < s.pspan; k += nt) ts[k] = __ldg(src + k);
-    s.Ts = ts;
-  }
-  s.ts_layer = a.smem_table_layer;
-}
-
-// Lean sweeps: full tiles, affine layout-0 addresses, state loaded in the internal format
-// or created as |+>, stored in the internal or the caller's format (complex64: the same).
-template <class CF, bool FX, bool TWO, bool OPS, int LAST>
-__global__ void __launch_bounds__(CF::NT, CF::MINB) lean_kernel(const __grid_constant__ SweepArgs a) {
-  using S = Lean<CF, FX, TWO>;
-  using V = typename S::V;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* X = (V*)smem_raw;  // exchange area: 2^B slots, twice that for two-buffer sweeps
-  void* Cs = smem_raw + ((sizeof(V) << CF::B) << (TWO ? 1 : 0));
-  const bool cost = OPS && a.needs_cost;
-  V* Tsm = (V*)((unsigned char*)Cs + (cost ? ((a.cost_dtype == QAOA_COST_F64 ? 8 : 4) << CF::B) : 0));
-  constexpr int NW = CF::NT / 32;
-  __shared__ double wacc[kLeanAcc * NW];
-  __shared__ fx::Factor dpre[FX ? kLeanMix * 16 : 1];
-  for (int r = threadIdx.x; r < kLeanAcc * NW; r += CF::NT) wacc[r] = 0.0;
-  S s(a, X, Cs, nullptr, nullptr);
-  s.wacc = wacc;
-  // grouped sweeps: this block's graph and its share of the graph's tiles
-  int64_t t0 = blockIdx.x, tstep = gridDim.x;
-  if (a.gslot != nullptr) {
-    const GroupSlot& gsl = a.gslot[blockIdx.x / a.gbpg];
-    s.zoff = gsl.zoff;
-    s.ptab = gsl.phase_table;
-    s.pcmin = gsl.cmin;
-    s.pspan = gsl.span;
-    s.trig = gsl.trig;
-    s.dtab = gsl.d_table;
-    t0 = blockIdx.x % a.gbpg;
-    tstep = a.gbpg;
-  }
-  if constexpr (FX) {  // every mixer's diagonal exp(-i beta (t - 2k)), k = 0..t, as prepared factors
-    const int t = a.g.t;
-    int m = 0;
-    for (int k = 0; k < (OPS ? a.nops : 1) && m < kLeanMix; ++k) {
-      const uint32_t op = a.ops[k];
-      if ((op & 0xff) != OP_MIX) continue;
-      if (threadIdx.x <= (uint32_t)t) {
-        const longlong2 e = __ldg((const longlong2*)s.dtab + ((long long)((op >> 16) & 0xff) * 14 + t) * 14 + threadIdx.x);
-        dpre[16 * m + threadIdx.x] = fx::factor(e.x, (op & F_SIGN) ? -e.y : e.y);
-      }
-      ++m;
-    }
-    s.dpre = dpre;
-  }
-  if (OPS && a.smem_table_layer >= 0) {
-    stage_table<FX>(s, a, Tsm, CF::NT);
-  }
-  if (TWO && a.stage) {  // staging area after the phase table, 16-byte aligned
-    const size_t tb = FX ? sizeof(fx::Factor) : sizeof(V);
-    const size_t off = (size_t)((unsigned char*)Tsm - smem_raw) + (OPS && a.smem_table_layer >= 0 ? tb * a.span : 0);
-    s.Ps = (V*)(smem_raw + ((off + 15) & ~(size_t)15));
-  }
-  s.evalid = 1u << CF::B;
-  if constexpr (FX && TWO) {
-    if (a.gslot != nullptr) {
-      s.lam_shift = a.gslot[blockIdx.x / a.gbpg].lam_shift;
-    } else if (a.cmax_dev != nullptr) {
-      const unsigned long long b = *a.cmax_dev;
-      const int ex = (int)((b >> 52) & 0x7FF);
-      const int k = ex == 0 ? 0 : ex - 1023 + ((b & ((1ull << 52) - 1)) != 0 ? 1 : 0);
-      s.lam_shift = k < 0 ? 0 : k;
-    }
-  }
-  __syncthreads();
-  bool have = false;  // this tile's psi is in the staging area
-  for (int64_t tile = t0; tile < a.g.tiles; tile += tstep) {
-    const int64_t next = tile + tstep < a.g.tiles ? tile + tstep : -1;
-    lean_tile<CF, FX, TWO, OPS, LAST, false>(s, a, tile, Cs, next, have);
-    have = s.Ps != nullptr && next >= 0;
-  }
-  __syncthreads();
-  for (int r = threadIdx.x; r < a.nred; r += CF::NT) {
-    double v = 0.0;
-    for (int w = 0; w < NW; ++w) v += wacc[r * NW + w];
-    a.partials[(int64_t)a.red_slot[r] * a.grid + blockIdx.x] = v;
-  }
-}
 
 template <class CF, bool FX, bool TWO>
 __global__ void __launch_bounds__(CF::NT, CF::MINB) sweep_kernel(const __grid_constant__ SweepArgs a) {
@@ -302,13 +202,6 @@ int num_sms() {
   return cached;
 }
 
-template <class CF, bool FX, bool TWO>
-size_t smem_bytes(int cost_bytes, int table_entries = 0) {
-  const size_t vb = FX ? sizeof(longlong2) : sizeof(float2);
-  const size_t tb = FX ? sizeof(fx::Factor) : sizeof(float2);  // staged phase-table entry
-  return ((vb << CF::B) << (TWO ? 1 : 0)) + ((size_t)cost_bytes << CF::B) + tb * table_entries;
-}
-
 // blocks per SM for a configuration with a cost tile of cost_bytes per amplitude (0, 4, 8)
 template <class CF, bool FX, bool TWO>
 int blocks_per_sm(int cost_bytes) {
@@ -329,49 +222,13 @@ int blocks_per_sm(int cost_bytes) {
   return cached[slot];
 }
 
-// dynamic shared memory a lean kernel may take on this device: the opt-in limit less its
-// static shared memory (two-buffer kernels, which may add the psi staging area), else the
-// largest exchange + cost + table layout
+// the lean kernels of this configuration (translation units lean_*.cu)
 template <class CF, bool FX, bool TWO>
-size_t lean_smem_cap() {
-  static size_t cached[64] = {};
-  static std::mutex mu;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  std::lock_guard<std::mutex> lk(mu);
-  size_t& c = cached[dev & 63];
-  if (c == 0) {
-    c = smem_bytes<CF, FX, TWO>(8, kSmemTable);
-    if (TWO) {
-      int optin = 0;
-      cudaFuncAttributes fa;
-      if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
-          cudaFuncGetAttributes(&fa, lean_kernel<CF, FX, TWO, true, 0>) == cudaSuccess &&
-          (size_t)optin > fa.sharedSizeBytes + 1024)
-        c = std::max(c, (size_t)optin - fa.sharedSizeBytes - 1024);
-    }
-  }
-  return c;
-}
-
-template <class CF, bool FX, bool TWO, bool OPS, int LAST>
-void lean_launch_l(const SweepArgs& a, size_t sm, cudaStream_t s) {
-  static std::mutex mu;
-  static uint64_t done = 0;
-  once_per_device(mu, done, [] {
-    cudaFuncSetAttribute(lean_kernel<CF, FX, TWO, OPS, LAST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)lean_smem_cap<CF, FX, TWO>());
-  });
-  lean_kernel<CF, FX, TWO, OPS, LAST><<<a.grid, CF::NT, sm, s>>>(a);
-}
-template <class CF, bool FX, bool TWO, bool OPS>
-void lean_launch(const SweepArgs& a, int last, size_t sm, cudaStream_t s) {
-  switch (last) {
-    case 0: lean_launch_l<CF, FX, TWO, OPS, 0>(a, sm, s); break;
-    case 1: lean_launch_l<CF, FX, TWO, OPS, 1>(a, sm, s); break;
-    case 2: lean_launch_l<CF, FX, TWO, OPS, 2>(a, sm, s); break;
-    default: lean_launch_l<CF, FX, TWO, OPS, (CF::NR > 3 ? 3 : 2)>(a, sm, s); break;
-  }
+void lean_launch_cfg(const SweepArgs& a, size_t sm, cudaStream_t s) {
+  if constexpr (FX && !TWO) lean_x1(a, sm, s);
+  else if constexpr (FX) a.kind == SWEEP_LEAN_OPS ? lean_x2_ops(a, sm, s) : lean_x2_mix(a, sm, s);
+  else if constexpr (!TWO) lean_f1(a, sm, s);
+  else lean_f2(a, sm, s);
 }
 
 template <class CF, bool FX, bool TWO>
@@ -381,12 +238,6 @@ void launch_t(const SweepArgs& a, cudaStream_t s) {
   const int te = a.smem_table_layer >= 0 ? (int)a.span : 0;
   const size_t sm = smem_bytes<CF, FX, TWO>(cb, te);
   if (a.kind == SWEEP_LEAN_MIX || a.kind == SWEEP_LEAN_OPS) {
-    // last round holding group qubits selects the instance
-    int last = 0;
-    for (int k = 0; k < CF::NR; ++k) {
-      const int lo = std::max(0, CF::B - CF::RB * (k + 1)), hi = k == 0 ? CF::B : std::max(0, CF::B - CF::RB * k);
-      if (hi > a.g.c && lo < a.g.c + a.g.t) last = k;
-    }
     // complex128 two-buffer sweeps that load psi stage the next tile's psi when shared
     // memory allows (complex64: measured no gain)
     SweepArgs b = a;
@@ -395,13 +246,11 @@ void launch_t(const SweepArgs& a, cudaStream_t s) {
       const size_t st = ((sm + 15) & ~(size_t)15) + ((FX ? sizeof(longlong2) : sizeof(float2)) << CF::B);
       if (st <= lean_smem_cap<CF, FX, TWO>()) {
         b.stage = 1;
-        if (a.kind == SWEEP_LEAN_OPS) lean_launch<CF, FX, TWO, true>(b, last, st, s);
-        else lean_launch<CF, FX, TWO, false>(b, last, st, s);
+        lean_launch_cfg<CF, FX, TWO>(b, st, s);
         return;
       }
     }
-    if (a.kind == SWEEP_LEAN_OPS) lean_launch<CF, FX, TWO, true>(b, last, sm, s);
-    else lean_launch<CF, FX, TWO, false>(b, last, sm, s);
+    lean_launch_cfg<CF, FX, TWO>(b, sm, s);
     return;
   }
   sweep_kernel<CF, FX, TWO><<<a.grid, CF::NT, sm, s>>>(a);

@@ -947,12 +947,19 @@ __device__ __forceinline__ void sweep_tile(Sweeper<CF, FX, TWO>& s, const SweepA
 // checks the tile shape, the formats and the affine layout-0 addresses before choosing
 // them.
 
-template <class CF, bool FX, bool TWO>
+//
+// With C >= 0 the carried bits are fixed too (c = C, group bits [C, B)): the group bits of
+// every round and the popcount class of every register are then constants, and the kernel
+// holds no branches on them.  C = -1 takes them from the sweep.
+
+template <class CF, bool FX, bool TWO, int C = -1>
 struct Lean : Sweeper<CF, FX, TWO> {
   using B = Sweeper<CF, FX, TWO>;
   using V = typename B::V;
   static constexpr int R = CF::R, NR = CF::NR;
   using B::B;
+  __device__ __forceinline__ int gc() const { return C >= 0 ? C : this->a.g.c; }
+  __device__ __forceinline__ int gt() const { return C >= 0 ? CF::B - C : this->a.g.t; }
   // mixer diagonals of the launch's mixers, staged once in shared memory ([kLeanMix][16]),
   // or nullptr: each mixer then stages its own between block barriers
   const fx::Factor* dpre = nullptr;
@@ -960,7 +967,7 @@ struct Lean : Sweeper<CF, FX, TWO> {
   // group-qubit register bits of round K (relative to lo(K)), uniform
   template <int K>
   __device__ __forceinline__ unsigned gmask() const {
-    const int gl = this->a.g.c, gh = this->a.g.c + this->a.g.t;
+    const int gl = gc(), gh = gl + gt();
     unsigned m = 0;
 #pragma unroll
     for (int rb = 0; rb < CF::RB; ++rb) {
@@ -1080,7 +1087,7 @@ struct Lean : Sweeper<CF, FX, TWO> {
   // W D W from layout 0 back to layout 0; D at layout L (the last round with group qubits)
   template <int L>
   __device__ __forceinline__ void fx_mixer(int layer, bool inverse, bool lam, int xacc, int mix) {
-    const int gl = this->a.g.c, t = this->a.g.t;
+    const int gl = gc(), t = gt();
     const fx::Factor* Ds = dpre != nullptr ? dpre + 16 * mix : this->Ds;
     if (dpre == nullptr) {
       __syncthreads();
@@ -1151,7 +1158,7 @@ struct Lean : Sweeper<CF, FX, TWO> {
       const bool xt = TWO && xacc >= 0;
       float xs = 0.f, w2 = 1.f;
       f32_fwd<0, L>(tanf, tu, m * m, xt, xs, w2);
-      const float2 f = B::round_factor(tanf, m, this->a.g.t);
+      const float2 f = B::round_factor(tanf, m, gt());
       this->scale_f32(this->v, f);
       if constexpr (TWO) this->scale_f32(this->w, f);
       if (xt) this->block_add(xacc, 2.0 * (double)xs, 0.0, false);
@@ -1214,10 +1221,10 @@ struct Lean : Sweeper<CF, FX, TWO> {
 // layout-0 slots, so the staging needs no barrier, only waits for the thread's own copy
 // groups; the cost tile's group is committed after the prefetch of this tile's psi and before
 // the prefetch of the next one.
-template <class CF, bool FX, bool TWO, bool OPS, int LAST, bool COHERENT>
-__device__ __forceinline__ void lean_tile(Lean<CF, FX, TWO>& s, const SweepArgs& a, int64_t tile, void* Cs,
+template <class CF, bool FX, bool TWO, bool OPS, int LAST, bool COHERENT, int C = -1>
+__device__ __forceinline__ void lean_tile(Lean<CF, FX, TWO, C>& s, const SweepArgs& a, int64_t tile, void* Cs,
                                           int64_t next = -1, bool have = false) {
-  using V = typename Lean<CF, FX, TWO>::V;
+  using V = typename Lean<CF, FX, TWO, C>::V;
   constexpr int R = CF::R;
   V (&v)[R] = s.v;
   V (&w)[R] = s.w;
@@ -1226,7 +1233,7 @@ __device__ __forceinline__ void lean_tile(Lean<CF, FX, TWO>& s, const SweepArgs&
   const bool cf64 = a.cost_dtype == QAOA_COST_F64;
   const bool cost = OPS && a.needs_cost;
   const uint32_t tb0 = CF::idx(0, tid, 0);
-  const uint64_t zs = 1ull << (CF::lo(0) - g.c + g.j0);
+  const uint64_t zs = 1ull << (CF::lo(0) - s.gc() + g.j0);
   const bool init = OPS && a.load_fmt == 2;
   const bool ld_lam = TWO && (!OPS || a.load_lam), st_lam = TWO && (!OPS || a.store_lam);
   const int st_fmt = OPS ? a.store_fmt : 0;
@@ -1293,6 +1300,14 @@ __device__ __forceinline__ void lean_tile(Lean<CF, FX, TWO>& s, const SweepArgs&
     }
     if (st_lam) ((V*)a.lam)[z] = w[r];
   }
+}
+
+// dynamic shared memory of a sweep: exchange area, cost tile, staged phase table
+template <class CF, bool FX, bool TWO>
+size_t smem_bytes(int cost_bytes, int table_entries = 0) {
+  const size_t vb = FX ? sizeof(longlong2) : sizeof(float2);
+  const size_t tb = FX ? sizeof(fx::Factor) : sizeof(float2);  // staged phase-table entry
+  return ((vb << CF::B) << (TWO ? 1 : 0)) + ((size_t)cost_bytes << CF::B) + tb * table_entries;
 }
 
 }  // namespace
