@@ -228,6 +228,12 @@ QAOA_HD C64 cmul_unit(long long xr, long long xi, const Factor& f) {
   return o;
 }
 
+// x c / 2^62 for |x| < 2^59 and a Q62 c with |c| <= 2^62, by cmul_unit's rounding (within one unit)
+QAOA_HD long long mul_unit(long long x, Limbs c) {
+  const Limbs a = split((long long)((unsigned long long)x << 2));
+  return madw(a.h, c.h, madw(a.l, c.h, madw(a.h, c.l, 1ll << 31)) >> 32);
+}
+
 // Running sums of Im(conj(w) v) = w.x v.y - w.y v.x by limb weight: value = P 2^64 + M 2^32 +
 // L 2^4.  One multiply-add-wide per limb product and no carries between products (an exact
 // 128-bit product and sum per term took ~80 instructions per amplitude, this ~15); the four

@@ -44,7 +44,9 @@ constexpr int lean_last(int c) {
 // static shared memory of a lean kernel: per-warp accumulators and staged diagonals
 template <class CF, bool FX>
 constexpr size_t lean_static_smem() {
-  return sizeof(double) * kLeanAcc * (CF::NT / 32) + sizeof(fx::Factor) * (FX ? kLeanMix * 16 : 1);
+  const size_t slots = (size_t)kLeanAcc * (CF::NT / 32);
+  return sizeof(double) * slots + (FX ? (sizeof(__int128) * slots + sizeof(fx::Factor) * kLeanMix * 16) : sizeof(float2) * slots) +
+         sizeof(int) * kLeanAcc + sizeof(F32Mix) * kLeanMix + 256;
 }
 
 // dynamic shared memory a lean kernel may take on this device: the opt-in limit less its
@@ -85,9 +87,24 @@ __global__ void __launch_bounds__(CF::NT, CF::MINB) lean_kernel(const __grid_con
   constexpr int NW = CF::NT / 32;
   __shared__ double wacc[kLeanAcc * NW];
   __shared__ fx::Factor dpre[FX ? kLeanMix * 16 : 1];
-  for (int r = threadIdx.x; r < kLeanAcc * NW; r += CF::NT) wacc[r] = 0.0;
+  __shared__ __int128 iacc[FX ? kLeanAcc * NW : 1];
+  __shared__ int ishift[kLeanAcc];
+  __shared__ float2 facc[FX ? 1 : kLeanAcc * NW];
+  __shared__ F32Mix fpre[kLeanMix];
+  for (int r = threadIdx.x; r < kLeanAcc * NW; r += CF::NT) {
+    wacc[r] = 0.0;
+    if constexpr (FX) iacc[r] = 0;
+    else facc[r] = make_float2(0.f, 0.f);
+    if (r < kLeanAcc) ishift[r] = 0;
+  }
   S s(a, X, Cs, nullptr, nullptr);
   s.wacc = wacc;
+  if constexpr (FX) {
+    s.iacc = iacc;
+    s.ishift = ishift;
+  } else {
+    s.facc = facc;
+  }
   // grouped sweeps: this block's graph and its share of the graph's tiles
   int64_t t0 = blockIdx.x, tstep = gridDim.x;
   if (a.gslot != nullptr) {
@@ -114,6 +131,16 @@ __global__ void __launch_bounds__(CF::NT, CF::MINB) lean_kernel(const __grid_con
       ++m;
     }
     s.dpre = dpre;
+  }
+  if constexpr (!FX) {
+    int m = 0;
+    for (int k = 0; k < (OPS ? a.nops : 1) && m < kLeanMix; ++k) {
+      const uint32_t op = a.ops[k];
+      if ((op & 0xff) != OP_MIX) continue;
+      if (threadIdx.x == (uint32_t)m) fpre[m] = f32_mix(a, s.trig, (op >> 16) & 0xff, op & F_SIGN, s.gt());
+      ++m;
+    }
+    s.fpre = fpre;
   }
   if (OPS && a.smem_table_layer >= 0) {
     stage_table<FX>(s, a, Tsm, CF::NT);
@@ -145,6 +172,13 @@ __global__ void __launch_bounds__(CF::NT, CF::MINB) lean_kernel(const __grid_con
   for (int r = threadIdx.x; r < a.nred; r += CF::NT) {
     double v = 0.0;
     for (int w = 0; w < NW; ++w) v += wacc[r * NW + w];
+    if constexpr (FX) {
+      __int128 t = 0;
+      for (int w = 0; w < NW; ++w) t += iacc[r * NW + w];
+      v += i128_to_double(t, ishift[r]);
+    } else {
+      for (int w = 0; w < NW; ++w) v += (double)facc[r * NW + w].x + (double)facc[r * NW + w].y;
+    }
     a.partials[(int64_t)a.red_slot[r] * a.grid + blockIdx.x] = v;
   }
 }

@@ -124,6 +124,13 @@ __device__ __forceinline__ double i128_to_double(i128 v, int s) { return fx::i12
 __device__ __forceinline__ long long double_to_fx(double d, int s) { return fx::from_double(d, s); }
 __device__ __forceinline__ unsigned long long frac_turns(double d) { return fx::frac_turns(d); }
 
+// a + b = s + e exactly (Knuth)
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+  const float t = a + b, bp = t - a;
+  e = (a - (t - bp)) + (b - bp);
+  s = t;
+}
+
 // exp(-2 pi i th) in float32 for a turn count th (the rare path of float costs or costs
 // outside the table); kept out of line so it does not raise the register budget of the
 // common path
@@ -173,6 +180,10 @@ __device__ __forceinline__ double arg_sinb(const SweepArgs& a, const double* tri
 __device__ __forceinline__ double cost_f(const void* Cs, bool f64, uint32_t i) {
   return f64 ? ((const double*)Cs)[phys_cost(i, true)] : (double)((const int*)Cs)[phys_cost(i, false)];
 }
+// in float32, integer costs without the float64 conversions
+__device__ __forceinline__ float cost_f32(const void* Cs, bool f64, uint32_t i) {
+  return f64 ? (float)((const double*)Cs)[phys_cost(i, true)] : (float)((const int*)Cs)[phys_cost(i, false)];
+}
 __device__ __forceinline__ int cost_i(const void* Cs, uint32_t i) { return ((const int*)Cs)[phys_cost(i, false)]; }
 
 template <class CF, bool FX, bool TWO>
@@ -192,6 +203,13 @@ struct Sweeper {
   int ts_layer;  // layer whose table Ts holds (-1: none)
   double* blk;   // block accumulators
   double* wacc = nullptr;  // per-warp accumulators [kLeanAcc][NT / 32], if set (lean sweeps)
+  // Lean sweeps sum what is not float64 by itself without the float64 pipe (two lanes per SM and
+  // clock: the ten warp-wide additions of one reduction took it 640 cycles per warp, and every
+  // warp of a block comes to a reduction at the same time): fixed-point terms as 128-bit integers
+  // (exact; value = sum 2^-ishift), float32 terms in double-float.  Per-warp slots as wacc's.
+  __int128* iacc = nullptr;
+  int* ishift = nullptr;
+  float2* facc = nullptr;
   double* red;   // reduction scratch [2][NT/32]
   int cur;       // current layout
   int lam_shift;  // lambda scale exponent (fixed point)
@@ -334,6 +352,43 @@ struct Sweeper {
       }
       blk[r] += s0;
       if (pair) blk[r + 1] += s1;
+    }
+  }
+
+  // add the block's sum of v 2^-shift to accumulator r
+  __device__ __forceinline__ void block_add_fx(int r, i128 v, int shift) {
+    if (iacc == nullptr) {
+      block_add(r, i128_to_double(v, shift), 0.0, false);
+      return;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long lo = __shfl_down_sync(0xffffffffu, (unsigned long long)v, o);
+      const unsigned long long hi = __shfl_down_sync(0xffffffffu, (unsigned long long)((unsigned __int128)v >> 64), o);
+      v = (i128)((unsigned __int128)v + (((unsigned __int128)hi << 64) | lo));
+    }
+    if ((tid & 31) == 0) iacc[r * (CF::NT / 32) + (tid >> 5)] += v;
+    if (tid == 0) ishift[r] = shift;
+  }
+  // add the block's sum of the float32 v to accumulator r
+  __device__ __forceinline__ void block_add_f32(int r, float v) {
+    if (facc == nullptr) {
+      block_add(r, (double)v, 0.0, false);
+      return;
+    }
+    float c = 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float y = __shfl_down_sync(0xffffffffu, v, o), yc = __shfl_down_sync(0xffffffffu, c, o);
+      float e;
+      two_sum(v, y, v, e);
+      c += yc + e;
+    }
+    if ((tid & 31) == 0) {
+      float2& t = facc[r * (CF::NT / 32) + (tid >> 5)];
+      float e;
+      two_sum(t.x, v, t.x, e);
+      t.y += c + e;
     }
   }
 
@@ -578,7 +633,7 @@ struct Sweeper {
       if (on_psi) scale_f32(v, f);
       if (TWO && on_lam) scale_f32(w, f);
     }
-    if (xt) block_add(xacc, 2.0 * (double)xs, 0.0, false);
+    if (xt) block_add_f32(xacc, 2.f * xs);
   }
 
   // ---------------------------------------------------------------- mixer, fixed point: W D W
@@ -701,7 +756,7 @@ struct Sweeper {
           w[r] = make_longlong2(round_shift((i128)v[r].x * cq, 62), round_shift((i128)v[r].y * cq, 62));
         }
       } else {
-        const float c = (float)cost_f(Cs, f64, i);
+        const float c = cost_f32(Cs, f64, i);
         w[r] = make_float2(c * v[r].x, c * v[r].y);
       }
     }
@@ -709,7 +764,6 @@ struct Sweeper {
 
   __device__ __forceinline__ void op_expect(int acc) {
     const bool f64 = a.cost_dtype == QAOA_COST_F64;
-    double e0 = 0.0, e1 = 0.0;
     if constexpr (FX) {
       i128 sc = 0, sn = 0;
       double sf = 0.0;
@@ -722,8 +776,9 @@ struct Sweeper {
         if (!f64) sc += (p2 >> 32) * cost_i(Cs, i);
         else sf += cost_f(Cs, true, i) * i128_to_double(p2, 2 * a.fx_shift);
       }
-      e1 = i128_to_double(sn, 2 * (a.fx_shift - in_shift) - 16);
-      e0 = f64 ? ldexp(sf, 2 * in_shift) : i128_to_double(sc, 2 * (a.fx_shift - in_shift) - 32);
+      if (f64) block_add(acc, ldexp(sf, 2 * in_shift), 0.0, false);
+      else block_add_fx(acc, sc, 2 * (a.fx_shift - in_shift) - 32);
+      block_add_fx(acc + 1, sn, 2 * (a.fx_shift - in_shift) - 16);
     } else {
       float s0[4] = {0.f, 0.f, 0.f, 0.f}, s1[4] = {0.f, 0.f, 0.f, 0.f};  // independent partial sums
 #pragma unroll
@@ -731,27 +786,38 @@ struct Sweeper {
         const uint32_t i = idx(r);
         if (i >= evalid) continue;
         const float p2 = v[r].x * v[r].x + v[r].y * v[r].y;
-        s0[r & 3] += (float)cost_f(Cs, f64, i) * p2;
+        s0[r & 3] += cost_f32(Cs, f64, i) * p2;
         s1[r & 3] += p2;
       }
-      e0 = (double)((s0[0] + s0[1]) + (s0[2] + s0[3]));
-      e1 = (double)((s1[0] + s1[1]) + (s1[2] + s1[3]));
+      block_add_f32(acc, (s0[0] + s0[1]) + (s0[2] + s0[3]));
+      block_add_f32(acc + 1, (s1[0] + s1[1]) + (s1[2] + s1[3]));
     }
-    block_add(acc, e0, e1, true);
   }
 
   __device__ __forceinline__ void op_cterm(int acc) {
     const bool f64 = a.cost_dtype == QAOA_COST_F64;
-    double e0 = 0.0;
     if constexpr (FX) {
-      if (R <= 8 && !f64 && lam_shift <= 28) {  // |C| <= 2^28: limb sums (fx::WeightedImSum)
+      if (R <= 8 && f64) {
+        // C psi / 2^lam_shift rounded to the state's resolution (as lambda holds it), then exact
+        // limb sums against lambda / 2^lam_shift
+        fx::ImSum sw;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const uint32_t i = idx(r);
+          if (i >= evalid) continue;
+          const fx::Limbs c = fx::split(double_to_fx(cost_f(Cs, true, i), 62 - lam_shift));
+          sw.add(fx::split(fx::mul_unit(v[r].x, c)), fx::split(fx::mul_unit(v[r].y, c)), fx::split(w[r].x),
+                 fx::split(w[r].y));
+        }
+        block_add_fx(acc, sw.value(), 2 * a.fx_shift - 2 * lam_shift - 1);
+      } else if (R <= 8 && lam_shift <= 28) {  // |C| <= 2^28: limb sums (fx::WeightedImSum)
         fx::WeightedImSum sw;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           const uint32_t i = idx(r);
           if (i < evalid) sw.add(v[r].x, v[r].y, w[r].x, w[r].y, cost_i(Cs, i));
         }
-        e0 = i128_to_double(sw.value(), 2 * a.fx_shift - 32 - lam_shift);
+        block_add_fx(acc, sw.value(), 2 * a.fx_shift - 32 - lam_shift - 1);
       } else {
         i128 sc = 0;
         double sf = 0.0;
@@ -763,7 +829,8 @@ struct Sweeper {
           if (!f64) sc += (pr >> 32) * cost_i(Cs, i);
           else sf += cost_f(Cs, true, i) * i128_to_double(pr, 2 * a.fx_shift - lam_shift);
         }
-        e0 = f64 ? sf : i128_to_double(sc, 2 * a.fx_shift - 32 - lam_shift);
+        if (f64) block_add(acc, 2.0 * sf, 0.0, false);
+        else block_add_fx(acc, sc, 2 * a.fx_shift - 32 - lam_shift - 1);
       }
     } else {
       float s[4] = {0.f, 0.f, 0.f, 0.f};  // independent partial sums
@@ -771,11 +838,10 @@ struct Sweeper {
       for (int r = 0; r < R; ++r) {
         const uint32_t i = idx(r);
         if (i >= evalid) continue;
-        s[r & 3] += (float)cost_f(Cs, f64, i) * (w[r].x * v[r].y - w[r].y * v[r].x);
+        s[r & 3] += cost_f32(Cs, f64, i) * (w[r].x * v[r].y - w[r].y * v[r].x);
       }
-      e0 = (double)((s[0] + s[1]) + (s[2] + s[3]));
+      block_add_f32(acc, 2.f * ((s[0] + s[1]) + (s[2] + s[3])));
     }
-    block_add(acc, 2.0 * e0, 0.0, false);
   }
 };
 
@@ -952,6 +1018,25 @@ __device__ __forceinline__ void sweep_tile(Sweeper<CF, FX, TWO>& s, const SweepA
 // every round and the popcount class of every register are then constants, and the kernel
 // holds no branches on them.  C = -1 takes them from the sweep.
 
+// A float32 mixer on t qubits: RX(2 beta) = m (I - i tu X) per qubit (tanf) or -i m (X + i tu I),
+// and the factor m^t or (-i m)^t of the group, which is f or i f.
+struct F32Mix {
+  float tu, m, f;
+  bool tanf, real;
+};
+__device__ __forceinline__ F32Mix f32_mix(const SweepArgs& a, const double* trig, int layer, bool inverse, int t) {
+  const double c = arg_cosb(a, trig, layer), s = inverse ? -arg_sinb(a, trig, layer) : arg_sinb(a, trig, layer);
+  F32Mix q;
+  q.tanf = fabs(c) >= fabs(s);
+  q.tu = q.tanf ? (float)(s / c) : (float)(c / s);
+  q.m = q.tanf ? (float)c : (float)s;
+  float f = 1.f;
+  for (int j = 0; j < t; ++j) f *= q.m;
+  q.real = q.tanf || (t & 1) == 0;
+  q.f = !q.tanf && ((t & 3) == 1 || (t & 3) == 2) ? -f : f;  // (-i)^t = 1, -i, -1, i
+  return q;
+}
+
 template <class CF, bool FX, bool TWO, int C = -1>
 struct Lean : Sweeper<CF, FX, TWO> {
   using B = Sweeper<CF, FX, TWO>;
@@ -963,6 +1048,7 @@ struct Lean : Sweeper<CF, FX, TWO> {
   // mixer diagonals of the launch's mixers, staged once in shared memory ([kLeanMix][16]),
   // or nullptr: each mixer then stages its own between block barriers
   const fx::Factor* dpre = nullptr;
+  const F32Mix* fpre = nullptr;  // float32: the mixers' coefficients, staged likewise
 
   // group-qubit register bits of round K (relative to lo(K)), uniform
   template <int K>
@@ -1081,7 +1167,7 @@ struct Lean : Sweeper<CF, FX, TWO> {
     }
     if (xacc >= 0) {
       const i128 xs = S.value() * (t - 2 * pt) - 2 * T.value();
-      this->block_add(xacc, 2.0 * i128_to_double(xs, 2 * this->a.fx_shift + t - this->lam_shift), 0.0, false);
+      this->block_add_fx(xacc, xs, 2 * this->a.fx_shift + t - this->lam_shift - 1);
     }
   }
   // W D W from layout 0 back to layout 0; D at layout L (the last round with group qubits)
@@ -1107,6 +1193,8 @@ struct Lean : Sweeper<CF, FX, TWO> {
   // ---- float32: RX(2 beta) = m (I - i u X) per qubit in tangent or cotangent form, as
   // unit-free butterflies round by round through layouts 0..L; the factors m (or -i m) of
   // all t qubits are applied once at the end, then one exchange returns to layout 0.
+  // (the coefficients are staged once per launch: their float64 division took every thread of
+  // every tile through the float64 pipe).
   // X-terms (adjoint pass): psi and lambda carry the same factor c of the qubits already
   // done, so Im conj(lambda) X_j psi of the unscaled buffers is |c|^2 = m^(2 done) times the
   // true value; X_j commutes with every RX_i, so each round's terms may be taken just before
@@ -1147,28 +1235,35 @@ struct Lean : Sweeper<CF, FX, TWO> {
     f32_round<K>(tanf, tu, m2, xt, xs, w2);
     if constexpr (K < L) f32_fwd<K + 1, L>(tanf, tu, m2, xt, xs, w2);
   }
-  template <int L>
-  __device__ __forceinline__ void f32_mixer(int layer, bool inverse, int xacc) {
+  // every amplitude times f (real) or i f
+  __device__ __forceinline__ void scale_axis(V (&u)[R], float f, bool real) {
     if constexpr (!FX) {
-      const double cbd = arg_cosb(this->a, this->trig, layer);
-      const double sbd = inverse ? -arg_sinb(this->a, this->trig, layer) : arg_sinb(this->a, this->trig, layer);
-      const bool tanf = fabs(cbd) >= fabs(sbd);
-      const float tu = tanf ? (float)(sbd / cbd) : (float)(cbd / sbd);
-      const float m = tanf ? (float)cbd : (float)sbd;
+      if (real) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) u[r] = make_float2(u[r].x * f, u[r].y * f);
+      } else {
+#pragma unroll
+        for (int r = 0; r < R; ++r) u[r] = make_float2(-(u[r].y * f), u[r].x * f);
+      }
+    }
+  }
+  template <int L>
+  __device__ __forceinline__ void f32_mixer(int layer, bool inverse, int xacc, int mix) {
+    if constexpr (!FX) {
+      const F32Mix q = fpre != nullptr ? fpre[mix] : f32_mix(this->a, this->trig, layer, inverse, gt());
       const bool xt = TWO && xacc >= 0;
       float xs = 0.f, w2 = 1.f;
-      f32_fwd<0, L>(tanf, tu, m * m, xt, xs, w2);
-      const float2 f = B::round_factor(tanf, m, gt());
-      this->scale_f32(this->v, f);
-      if constexpr (TWO) this->scale_f32(this->w, f);
-      if (xt) this->block_add(xacc, 2.0 * (double)xs, 0.0, false);
+      f32_fwd<0, L>(q.tanf, q.tu, q.m * q.m, xt, xs, w2);
+      scale_axis(this->v, q.f, q.real);
+      if constexpr (TWO) scale_axis(this->w, q.f, q.real);
+      if (xt) this->block_add_f32(xacc, 2.f * xs);
       if constexpr (L > 0) exb<L, 0>();
     }
   }
   template <int L>
   __device__ __forceinline__ void mixer(int layer, bool inverse, int xacc, int mix) {
     if constexpr (FX) fx_mixer<L>(layer, inverse, TWO, xacc, mix);
-    else f32_mixer<L>(layer, inverse, xacc);
+    else f32_mixer<L>(layer, inverse, xacc, mix);
   }
 
   // ---- the sweep: one mixer (OPS = false), or the sweep's op program (OPS = true) with
