@@ -84,6 +84,10 @@ __device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(gmem) : "memory");
 }
+__device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(sa), "l"(gmem) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 // all but the newest N committed groups of this thread are complete
 template <int N>
@@ -1337,14 +1341,19 @@ __device__ __forceinline__ void lean_tile(Lean<CF, FX, TWO, C>& s, const SweepAr
   const uint64_t base = tile_base(g, tile);
   s.base = base;
   s.cur = 0;
-  if (cost) {  // cost tile, 16-byte asynchronous copies
+  if (cost) {  // cost tile, asynchronous copies of the longest runs up to 16 bytes that are contiguous
     __syncthreads();
-    const int per = cf64 ? 2 : 4;
-    const uint32_t nch = (1u << CF::B) / per;
+    const int eb = cf64 ? 3 : 2;  // log2 of an entry's bytes
+    const int pb = g.j0 == 0 ? 4 - eb : min(4 - eb, s.gc());  // log2 of the entries per copy
+    const uint32_t nch = 1u << (CF::B - pb);
     for (uint32_t ch = tid; ch < nch; ch += CF::NT) {
-      const uint32_t i = ch * per;
+      const uint32_t i = ch << pb;
       const uint64_t z = local_to_z(g, base, i);
-      cp_async16((char*)Cs + (size_t)phys_cost(i, cf64) * (cf64 ? 8 : 4), (const char*)a.C + (s.zoff + z) * (cf64 ? 8 : 4));
+      char* dst = (char*)Cs + ((size_t)phys_cost(i, cf64) << eb);
+      const char* src = (const char*)a.C + ((s.zoff + z) << eb);
+      if (pb + eb == 4) cp_async16(dst, src);
+      else if (pb + eb == 3) cp_async8(dst, src);
+      else cp_async4(dst, src);
     }
     if (stage) cp_async_commit();
   }
