@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(kPrepThreads) batch_prep_kernel(const __grid_c
     return;
   }
   if (fx)
-    for (int j = tid; j < 3 * 1024; j += kPrepThreads) ((longlong2*)b.turn)[j] = turn_entry(j);
+    for (int j = tid; j < kTurnEntries; j += kPrepThreads) ((longlong2*)b.turn)[j] = turn_entry(j);
 }
 
 // The persistent kernel: graphs [first, first + count) of the processing order, taken from

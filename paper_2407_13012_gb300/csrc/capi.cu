@@ -125,7 +125,7 @@ static size_t phase_table_bytes(int dtype, int p, int64_t span) {
 }
 static size_t fx_table_bytes(int dtype, int p) {
   if (dtype != QAOA_C128) return 0;
-  return round256((size_t)p * 196 * 16) + round256(3072 * 16);
+  return round256((size_t)p * 196 * 16) + round256(kTurnEntries * 16);
 }
 // workspace of the optimiser beyond the gradient's: Adam moments (4p), step counter,
 // gradient output (2p + 2)
@@ -200,7 +200,10 @@ static int run_sweeps(const Ctx& c, std::vector<Sweep>& sw, const std::vector<Gr
     any_user_load |= s.load_user;
   }
   for (const Group& g : gs) tmax = std::max(tmax, g.t);
-  const int cost_bytes = c.cost->C_dev == nullptr ? 0 : (c.cost->dtype == QAOA_COST_I32 ? 4 : 8);
+  // (complex64 sweeps stage no float64 costs)
+  const int cost_bytes = c.cost->C_dev == nullptr || (!fx && c.cost->dtype != QAOA_COST_I32) ? 0
+                         : c.cost->dtype == QAOA_COST_I32                                    ? 4
+                                                                                             : 8;
   // one grid (the partials' stride) for all sweeps: sized for the single-buffer kernels;
   // two-buffer kernels with fewer resident blocks per SM run it in waves
   int grid = sweep_grid(c.dtype, false, tile_bits, cost_bytes, max_tiles);
@@ -1164,7 +1167,7 @@ int batch_layout(int dtype, int p, int ngraphs, const qaoa_graph_t* gs, const do
   L.off_C = take((L.cost_f64 ? 8 : 4) * std::max<int64_t>(amps, 1));
   L.off_phase = take(vs * std::max<int64_t>(tab, 1));
   L.off_dtab = take(fx ? (size_t)16 * p * 196 * std::max(ngraphs, 1) : 0);
-  L.off_turn = take(fx ? (size_t)16 * 3072 : 0);
+  L.off_turn = take(fx ? (size_t)16 * kTurnEntries : 0);
   L.off_gslot = take(sizeof(GroupSlot) * std::max(L.n_grouped, 1));
   L.off_grow = take(sizeof(int) * std::max(L.n_grouped, 1));
   L.off_gpart = take(std::max<size_t>(gpart, 8));

@@ -347,5 +347,29 @@ QAOA_HD unsigned long long frac_turns(double d) {
   return (bits >> 63) ? (0ull - t) : t;
 }
 
+// exp(-2 pi i t / 2^64) in Q62: two 256-entry tables (tt[k] = exp(-2 pi i k / 2^8), tt[256 + k] =
+// exp(-2 pi i k / 2^16)) take the turn's nearest multiple of 2^-16, and the residual angle rho
+// (below 2^-13.3) enters as (1 - rho^2/2) - i (rho - rho^3/6), to 2^-57 (the next term is
+// rho^4/24).  The tables are 8 KB, so a sweep holds them in shared memory beside its cost tile;
+// three 1024-entry tables with a first-order residual (to 2^-55) took three reads from L2 and two
+// 128-bit complex products per amplitude.
+template <class E>
+QAOA_HD C64 turn_phase(unsigned long long t, const E* tt) {
+  const unsigned k = (unsigned)((t + (1ull << 47)) >> 48);                  // modulo 2^16
+  const long long r = (long long)(t - ((unsigned long long)k << 48));       // [-2^47, 2^47)
+  const E a = tt[(k >> 8) & 255], b = tt[256 + (k & 255)];
+  const Limbs ax = split(a.x), ay = split(a.y), bx = split(b.x), by = split(b.y), nby = split(-b.y);
+  const long long ex = dot2_q62_hi(ax, bx, ay, nby, 0), ey = dot2_q62_hi(ax, by, ay, bx, 0);
+  const long long rho = mul_unit(2 * r, split(3622009729038561421ll));      // 2 pi r 2^-64: pi/4 in Q62
+  const int x = (int)(rho >> 18);
+  const int h4 = (int)(madw(x, x, 0) >> 31);                                // rho^2 / 2, 2^-58 units
+  const long long s = rho - (madw(x, h4 / 3, 0) >> 40);                     // rho - rho^3 / 6
+  const Limbs X = split(ex), Y = split(ey);
+  C64 o;
+  o.x = ex - (madw(X.h, h4, 0) >> 26) + mul_unit(s, Y);
+  o.y = ey - (madw(Y.h, h4, 0) >> 26) - mul_unit(s, X);
+  return o;
+}
+
 }  // namespace fx
 }  // namespace qaoa

@@ -44,6 +44,7 @@ constexpr int kGridCap = 2048;               // most blocks a reduction writes p
 // qaoa_expectation_host lets the device write the result before copying it out
 constexpr size_t kExpectPartialBytes = 2 * (size_t)kMaxContrib * kGridCap * sizeof(double);
 constexpr size_t kHostResultBytes = 256;
+constexpr int kTurnEntries = 512;            // entries of the two turn tables (computed phases)
 constexpr int kSmemTable = 1024;             // phase-table entries a sweep may keep in shared memory
 
 struct SweepGeom {
@@ -97,11 +98,12 @@ struct SweepArgs {
   double cosb[QAOA_MAX_P];
   double sinb[QAOA_MAX_P];
   // tables (workspace): integer-cost phases exp(-i gamma_l c) at [l * span + (c - cmin)];
-  // fixed point also mixer diagonals [(l * 14 + t) * 14 + k] and turn tables [3 * 1024]
+  // fixed point also mixer diagonals [(l * 14 + t) * 14 + k] and turn tables [kTurnEntries]
   const void* phase_table;
   int64_t cmin;
   int64_t span;
   int smem_table_layer;  // layer whose table the kernel copies to shared memory (-1: none)
+  int smem_turns;        // lean fixed-point sweeps: the turn tables are copied to shared memory
   const void* d_table;
   const void* turn_table;
   // reductions: accumulator r is written to partials[red_slot[r] * grid + block],
@@ -134,7 +136,7 @@ struct TableArgs {
   double beta[QAOA_MAX_P];
   void* phase;   // p * span entries
   void* dtab;    // fixed point: p * 14 * 14 entries
-  void* turn;    // fixed point: 3 * 1024 entries
+  void* turn;    // fixed point: kTurnEntries entries
 };
 
 // lean sweeps (lean_*.cu) of the sweep's shape, with sm bytes of dynamic shared memory

@@ -90,7 +90,7 @@ __global__ void group_reduce_kernel(const __grid_constant__ ReducePlan r, int ng
 __global__ void tables_kernel(const __grid_constant__ TableArgs ta) {
   const int64_t nphase = (int64_t)ta.p * ta.span;
   const int64_t nd = ta.fx ? (int64_t)ta.p * 14 * 14 : 0;
-  const int64_t nt = ta.fx ? 3 * 1024 : 0;
+  const int64_t nt = ta.fx ? kTurnEntries : 0;
   const int64_t total = nphase + nd + nt;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
     if (i < nphase) {
@@ -236,12 +236,17 @@ void launch_t(const SweepArgs& a, cudaStream_t s) {
   blocks_per_sm<CF, FX, TWO>(8);
   const int cb = a.needs_cost ? (a.cost_dtype == QAOA_COST_F64 ? 8 : 4) : 0;
   const int te = a.smem_table_layer >= 0 ? (int)a.span : 0;
-  const size_t sm = smem_bytes<CF, FX, TWO>(cb, te);
+  size_t sm = smem_bytes<CF, FX, TWO>(cb, te);
   if (a.kind == SWEEP_LEAN_MIX || a.kind == SWEEP_LEAN_OPS) {
     // complex128 two-buffer sweeps that load psi stage the next tile's psi when shared
     // memory allows (complex64: measured no gain)
     SweepArgs b = a;
     b.stage = 0;
+    if (a.needs_cost) {
+      sm = smem_bytes<CF, FX, TWO>(lean_cost_bytes<FX>(a.cost_dtype), te);
+      b.smem_turns = FX && a.kind == SWEEP_LEAN_OPS && a.cost_dtype == QAOA_COST_F64;
+      if (b.smem_turns) sm += sizeof(longlong2) * kTurnEntries;
+    }
     if (TWO && FX && !(a.kind == SWEEP_LEAN_OPS && a.load_fmt == 2)) {
       const size_t st = ((sm + 15) & ~(size_t)15) + ((FX ? sizeof(longlong2) : sizeof(float2)) << CF::B);
       if (st <= lean_smem_cap<CF, FX, TWO>()) {
@@ -369,7 +374,7 @@ cudaError_t launch_group_reduce(const ReducePlan& r, int ngraphs, int bpg, const
 }
 
 cudaError_t launch_tables(const TableArgs& t, cudaStream_t s) {
-  const int64_t total = (int64_t)t.p * t.span + (t.fx ? (int64_t)t.p * 196 + 3072 : 0);
+  const int64_t total = (int64_t)t.p * t.span + (t.fx ? (int64_t)t.p * 196 + kTurnEntries : 0);
   if (total <= 0) return cudaSuccess;
   const int blocks = (int)((total + 255) / 256 < 1024 ? (total + 255) / 256 : 1024);
   note_launch(3, s, true);

@@ -118,11 +118,6 @@ __device__ __forceinline__ longlong2 cmul_fx(longlong2 x, longlong2 e) {
   const fx::C64 o = fx::cmul_unit<false>(x.x, x.y, fx::factor(e.x, e.y));
   return make_longlong2(o.x, o.y);
 }
-// (x * e) / 2^(62 + extra) with 128-bit products, for operands up to 2^63 (products of two Q62 factors)
-__device__ __forceinline__ longlong2 cmul_fx_wide(longlong2 x, longlong2 e, int extra) {
-  const fx::C64 o = fx::cmul_q62_exact(x.x, x.y, e.x, e.y, extra);
-  return make_longlong2(o.x, o.y);
-}
 __device__ __forceinline__ double fx_to_double(long long x, int s) { return fx::to_double(x, s); }
 __device__ __forceinline__ double i128_to_double(i128 v, int s) { return fx::i128_to_double(v, s); }
 __device__ __forceinline__ long long double_to_fx(double d, int s) { return fx::from_double(d, s); }
@@ -135,13 +130,15 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = t;
 }
 
-// exp(-2 pi i th) in float32 for a turn count th (the rare path of float costs or costs
-// outside the table); kept out of line so it does not raise the register budget of the
-// common path
+// exp(-2 pi i th) in float32 for a turn count th (the path of float costs or costs outside the
+// table); kept out of line so it does not raise the register budget of the common path.  The
+// fraction of the turn comes from the integer bits (its float64 rounding, subtraction and
+// conversion took the float64 pipe three times as long as the product that th is).
 __device__ __noinline__ float2 phase_f32_direct(double th) {
-  const float f = (float)(th - rint(th));
+  const int f = (int)(unsigned)(frac_turns(th) >> 32);  // signed: the turn in [-1/2, 1/2) x 2^32
   float s, c;
-  sincospif(2.0f * f, &s, &c);
+  sincospif((float)f * 0x1.0p-31f, &s, &c);
+  if (((unsigned)__double2hiint(th) & 0x7ff00000u) == 0x7ff00000u) s = c = __int_as_float(0x7fffffff);  // no phase
   return make_float2(c, -s);
 }
 
@@ -152,19 +149,9 @@ __device__ __noinline__ longlong2 phase_fx_direct(double th, const longlong2* __
   return turn_phase(frac_turns(th), tt);
 }
 
-// exp(-2 pi i t / 2^64) in Q62 from three 1024-entry tables and a first-order residual
 __device__ __forceinline__ longlong2 turn_phase(unsigned long long t, const longlong2* __restrict__ tt) {
-  const longlong2 e1 = tt[t >> 54];
-  const longlong2 e2 = tt[1024 + ((t >> 44) & 1023)];
-  const longlong2 e3 = tt[2048 + ((t >> 34) & 1023)];
-  longlong2 e = cmul_fx_wide(e1, e2, 0);
-  e = cmul_fx_wide(e, e3, 0);
-  // residual angle rho = 2 pi r 2^-64 < 2 pi 2^-30; exp(-i rho) = 1 - i rho to 2e-17
-  const unsigned long long r = t & ((1ull << 34) - 1);
-  const long long rho = (long long)(((r >> 2) * 3373259426ull) >> 29);  // rho * 2^62, 3373259426 = round(pi/2 2^31)
-  const long long dre = round_shift((i128)rho * e.y, 62);
-  const long long dim = round_shift((i128)rho * e.x, 62);
-  return make_longlong2(e.x + dre, e.y - dim);
+  const fx::C64 e = fx::turn_phase(t, tt);
+  return make_longlong2(e.x, e.y);
 }
 
 // ------------------------------------------------------------------ kernel
@@ -205,6 +192,7 @@ struct Sweeper {
   const fx::Factor* Tf;  // the same for fixed-point states, as prepared factors
   fx::Factor* Ds;  // shared-memory mixer diagonal of the current fixed-point mixer (<= 14 entries)
   int ts_layer;  // layer whose table Ts holds (-1: none)
+  const longlong2* turns;  // fixed point: the turn tables (shared memory in lean sweeps of float costs)
   double* blk;   // block accumulators
   double* wacc = nullptr;  // per-warp accumulators [kLeanAcc][NT / 32], if set (lean sweeps)
   // Lean sweeps sum what is not float64 by itself without the float64 pipe (two lanes per SM and
@@ -221,6 +209,10 @@ struct Sweeper {
   uint32_t evalid;
   uint64_t base;
   const uint32_t tid;
+  // float64 costs read from memory by the ops (layout 0) instead of from a staged tile: this
+  // thread's first entry, and the stride of the register index; nullptr: the tile
+  const double* Cg = nullptr;
+  uint64_t czs = 0;
   // the graph's data: a's, or one graph's of a grouped sweep (lean kernels)
   int64_t zoff;          // element offset of psi, lambda and C
   const void* ptab;      // phase tables
@@ -232,7 +224,9 @@ struct Sweeper {
       : a(a_), X(X_), Cs(Cs_), Ts(nullptr), Tf(nullptr), Ds(nullptr), ts_layer(-1), blk(blk_), red(red_), cur(0),
         lam_shift(0),
         in_shift(0), evalid(0), base(0), tid(threadIdx.x), zoff(0), ptab(a_.phase_table), pcmin(a_.cmin),
-        pspan(a_.span), trig(a_.dev_trig), dtab(a_.d_table) {}
+        pspan(a_.span), trig(a_.dev_trig), dtab(a_.d_table) {
+    turns = (const longlong2*)a_.turn_table;
+  }
 
   __device__ __forceinline__ uint32_t idx(int r) const { return CF::idx(cur, tid, r); }
 
@@ -407,10 +401,41 @@ struct Sweeper {
   // phase factor of cost c computed directly (out of line: only costs outside the table and
   // float costs take it)
   __device__ __forceinline__ V phase_direct(int layer, double c) const {
-    if constexpr (FX) return phase_fx_direct(arg_g2pi(a, trig, layer) * c, (const longlong2*)a.turn_table);
+    if constexpr (FX) return phase_fx_direct(arg_g2pi(a, trig, layer) * c, turns);
     else return phase_f32_direct(arg_g2pi(a, trig, layer) * c);
   }
   // psi (or lambda) *= exp(-i s gamma_l C): table lookups first, the rest out of line
+  // the float64 cost of register r
+  __device__ __forceinline__ double cost_at(bool f64, int r) const {
+    if (!FX && Cg != nullptr) return __ldg(Cg + (uint64_t)r * czs);
+    return cost_f(Cs, f64, idx(r));
+  }
+  __device__ __forceinline__ float cost32_at(bool f64, int r) const {
+    if (!FX && Cg != nullptr) return (float)__ldg(Cg + (uint64_t)r * czs);
+    return cost_f32(Cs, f64, idx(r));
+  }
+  // u (and u2, if TWO_U) *= the directly computed phase factors of the registers in miss; the
+  // costs of eight registers are read at a time, ahead of their out-of-line factors
+  template <bool INV, bool TWO_U>
+  __device__ __forceinline__ void phase_misses(V (&u)[R], V (&u2)[R], int layer, unsigned miss, bool f64) {
+    constexpr int G = R < 8 ? R : 8;
+#pragma unroll
+    for (int r0 = 0; r0 < R; r0 += G) {
+      if (((miss >> r0) & ((1u << G) - 1u)) == 0) continue;
+      double c[G];
+#pragma unroll
+      for (int k = 0; k < G; ++k) c[k] = cost_at(f64, r0 + k);
+#pragma unroll
+      for (int k = 0; k < G; ++k) {
+        const int r = r0 + k;
+        if (!((miss >> r) & 1u)) continue;
+        V e = phase_direct(layer, c[k]);
+        if constexpr (INV) e.y = -e.y;
+        u[r] = vmul(u[r], e);
+        if constexpr (TWO_U) u2[r] = vmul(u2[r], e);
+      }
+    }
+  }
   template <bool INV>
   __device__ __forceinline__ void phase_apply(V (&u)[R], int layer) {
     const bool f64 = a.cost_dtype == QAOA_COST_F64;
@@ -448,15 +473,7 @@ struct Sweeper {
     } else {
       miss = R == 32 ? 0xffffffffu : ((1u << R) - 1);
     }
-    if (miss) {
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        if (!((miss >> r) & 1u)) continue;
-        V e = phase_direct(layer, cost_f(Cs, f64, idx(r)));
-        if constexpr (INV) e.y = -e.y;
-        u[r] = vmul(u[r], e);
-      }
-    }
+    if (miss) phase_misses<INV, false>(u, u, layer, miss, f64);
   }
 
   // the same factors on psi and lambda: looked up (or computed) once per amplitude
@@ -501,16 +518,7 @@ struct Sweeper {
     } else {
       miss = R == 32 ? 0xffffffffu : ((1u << R) - 1);
     }
-    if (miss) {
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        if (!((miss >> r) & 1u)) continue;
-        V e = phase_direct(layer, cost_f(Cs, f64, idx(r)));
-        if constexpr (INV) e.y = -e.y;
-        v[r] = vmul(v[r], e);
-        w[r] = vmul(w[r], e);
-      }
-    }
+    if (miss) phase_misses<INV, true>(v, w, layer, miss, f64);
   }
 
   __device__ __forceinline__ void op_phase(int layer, bool inverse, bool on_psi, bool on_lam) {
@@ -760,7 +768,7 @@ struct Sweeper {
           w[r] = make_longlong2(round_shift((i128)v[r].x * cq, 62), round_shift((i128)v[r].y * cq, 62));
         }
       } else {
-        const float c = cost_f32(Cs, f64, i);
+        const float c = cost32_at(f64, r);
         w[r] = make_float2(c * v[r].x, c * v[r].y);
       }
     }
@@ -790,7 +798,7 @@ struct Sweeper {
         const uint32_t i = idx(r);
         if (i >= evalid) continue;
         const float p2 = v[r].x * v[r].x + v[r].y * v[r].y;
-        s0[r & 3] += cost_f32(Cs, f64, i) * p2;
+        s0[r & 3] += cost32_at(f64, r) * p2;
         s1[r & 3] += p2;
       }
       block_add_f32(acc, (s0[0] + s0[1]) + (s0[2] + s0[3]));
@@ -842,7 +850,7 @@ struct Sweeper {
       for (int r = 0; r < R; ++r) {
         const uint32_t i = idx(r);
         if (i >= evalid) continue;
-        s[r & 3] += cost_f32(Cs, f64, i) * (w[r].x * v[r].y - w[r].y * v[r].x);
+        s[r & 3] += cost32_at(f64, r) * (w[r].x * v[r].y - w[r].y * v[r].x);
       }
       block_add_f32(acc, 2.f * ((s[0] + s[1]) + (s[2] + s[3])));
     }
@@ -853,7 +861,7 @@ struct Sweeper {
 //
 // Integer-cost phase tables hold exp(-i gamma c); fixed-point mixer diagonals hold
 // exp(-i beta (t - 2k)) at [(l * 14 + t) * 14 + k] for t = 1..13, k = 0..t (zero past t);
-// the turn tables hold exp(-2 pi i k / 2^(10 (level + 1))) for level 0..2, k < 1024.
+// the turn tables hold exp(-2 pi i k / 2^(8 (level + 1))) for level 0 and 1, k < 256.
 __device__ __forceinline__ long long q62(double x) { return llrint(ldexp(x, 62)); }
 __device__ __forceinline__ longlong2 unit_q62(double th) {
   double sn, cs;
@@ -871,8 +879,8 @@ __device__ __forceinline__ longlong2 d_entry(double beta, int j) {
   return k <= t ? unit_q62(beta * (double)(t - 2 * k)) : make_longlong2(0, 0);
 }
 __device__ __forceinline__ longlong2 turn_entry(int j) {
-  const int level = j / 1024, k = j % 1024;
-  return unit_q62(2.0 * 3.141592653589793238 * (double)k * ldexp(1.0, -10 * (level + 1)));
+  const int level = j / 256, k = j % 256;
+  return unit_q62(2.0 * 3.141592653589793238 * (double)k * ldexp(1.0, -8 * (level + 1)));
 }
 
 // state loads: through the read-only path, or (COHERENT) through L2 for state that the same
@@ -1330,7 +1338,8 @@ __device__ __forceinline__ void lean_tile(Lean<CF, FX, TWO, C>& s, const SweepAr
   const SweepGeom& g = a.g;
   const uint32_t tid = threadIdx.x;
   const bool cf64 = a.cost_dtype == QAOA_COST_F64;
-  const bool cost = OPS && a.needs_cost;
+  const bool direct = !FX && OPS && a.needs_cost && cf64;  // float64 costs, read by the ops
+  const bool cost = OPS && a.needs_cost && !direct;
   const uint32_t tb0 = CF::idx(0, tid, 0);
   const uint64_t zs = 1ull << (CF::lo(0) - s.gc() + g.j0);
   const bool init = OPS && a.load_fmt == 2;
@@ -1362,6 +1371,10 @@ __device__ __forceinline__ void lean_tile(Lean<CF, FX, TWO, C>& s, const SweepAr
     else cp_async_wait<0>();
   }
   const uint64_t z0 = local_to_z(g, base, tb0);
+  if (direct) {
+    s.Cg = (const double*)a.C + s.zoff + z0;
+    s.czs = zs;
+  }
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const uint64_t z = z0 + (uint64_t)r * zs;
