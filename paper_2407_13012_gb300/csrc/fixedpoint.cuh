@@ -214,7 +214,7 @@ QAOA_HD C64 cmul_big(Limbs r, Limbs i, const Factor& f, int e) {
   return o;
 }
 
-// x * u / 2^62 (conj(u) when CONJ) for |re x|, |im x| < 2^59: the operand is scaled by 4 first,
+// x * u / 2^62 (conj(u) when CONJ) for |re x|, |im x| <= 2^60: the operand is scaled by 4 first,
 // so the rounded sum is the high word pair itself (no shift after the products) and the
 // dropped low x low products stay below half a unit: within one unit of exact rounding.
 template <bool CONJ>

@@ -18,11 +18,8 @@
 //
 // A pair gate on (a, b), a < b, pairs z (z_a = 1, z_b = 0) with z' = z ^ 2^a ^ 2^b, the
 // same state with that set bit moved from a up to b (z' > z); states with z_a = z_b are
-// unchanged.  The thread owning z updates both amplitudes, so a launch touches every
-// amplitude at most once.  For adjacent qubits (b = a + 1) the moved bit keeps its index
-// j + 1 among the set bits (j = set bits below a), so
-//   rank(z') - rank(z) = binom(a + 1, j + 1) - binom(a, j + 1) = binom(a, j);
-// the closing pair (0, n-1) ranks z' directly.
+// unchanged.  A launch applies the pairs of a window of adjacent qubits to tiles in shared
+// memory (xy_window.cuh), or the closing pair (0, n-1), and touches every amplitude at most once.
 #include "fixedpoint.cuh"
 #include "internal.h"
 #include "xy_window.cuh"
@@ -60,6 +57,20 @@ struct XYCostArgs {
   long long ew[QAOA_XY_MAX_EDGES];  // integer or fixed-point weights
 };
 
+// Pascal's triangle in device memory: the window kernels copy the rows they need
+struct Pascal {
+  unsigned long long v[kBN][kBN];
+};
+constexpr Pascal make_pascal() {
+  Pascal p = {};
+  for (int c = 0; c < kBN; ++c) {
+    p.v[c][0] = 1;
+    for (int i = 1; i <= c; ++i) p.v[c][i] = p.v[c - 1][i - 1] + p.v[c - 1][i];
+  }
+  return p;
+}
+__device__ const Pascal g_pascal = make_pascal();
+
 __device__ __forceinline__ void load_binom(unsigned long long (*B)[kBN], const XYShape& s) {
   for (int i = threadIdx.x; i < kBN * kBN; i += blockDim.x) B[i / kBN][i % kBN] = s.binom[i / kBN][i % kBN];
   __syncthreads();
@@ -80,15 +91,6 @@ __device__ __forceinline__ unsigned long long xy_unrank(unsigned long long r, in
   return z;
 }
 
-__device__ __forceinline__ unsigned long long xy_rank(unsigned long long z, const unsigned long long (*B)[kBN]) {
-  unsigned long long r = 0;
-  for (int i = 1; z != 0; ++i) {
-    r += B[__ffsll((long long)z) - 1][i];
-    z &= z - 1;
-  }
-  return r;
-}
-
 // next larger integer with the same popcount (Gosper); z != 0
 __device__ __forceinline__ unsigned long long xy_next(unsigned long long z) {
   const unsigned long long t = z | (z - 1);
@@ -105,38 +107,6 @@ template <>
 struct Real<float2> {
   using type = float;
 };
-
-template <typename T>
-__global__ void __launch_bounds__(kXYThreads)
-    xy_gate_kernel(const __grid_constant__ XYShape s, T* __restrict__ psi, int qa, int qb,
-                   typename Real<T>::type cb, typename Real<T>::type sb) {
-  __shared__ unsigned long long B[kBN][kBN];
-  load_binom(B, s);
-  const unsigned long long D = s.D, nch = (D + kXYChunk - 1) / kXYChunk;
-  const unsigned long long ma = 1ull << qa, mb = 1ull << qb, below = ma - 1;
-  const bool adjacent = qb == qa + 1;
-  for (unsigned long long ch = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; ch < nch;
-       ch += (unsigned long long)gridDim.x * blockDim.x) {
-    const unsigned long long r0 = ch * kXYChunk, r1 = r0 + kXYChunk < D ? r0 + kXYChunk : D;
-    unsigned long long z = xy_unrank(r0, s.n, s.k, B);
-    for (unsigned long long r = r0; r < r1; ++r) {
-      if ((z & ma) && !(z & mb)) {
-        const unsigned long long rp = adjacent ? r + B[qa][__popcll(z & below)] : xy_rank(z ^ ma ^ mb, B);
-        if (rp < D) {
-          const T x = psi[r], y = psi[rp];
-          T u, v;
-          u.x = cb * x.x + sb * y.y;  // cos(beta) x - i sin(beta) y
-          u.y = cb * x.y - sb * y.x;
-          v.x = cb * y.x + sb * x.y;  // cos(beta) y - i sin(beta) x
-          v.y = cb * y.y - sb * x.x;
-          psi[r] = u;
-          psi[rp] = v;
-        }
-      }
-      if (r + 1 < r1) z = xy_next(z);
-    }
-  }
-}
 
 __global__ void __launch_bounds__(kXYThreads) xy_cost_kernel(const __grid_constant__ XYCostArgs a) {
   __shared__ unsigned long long B[kBN][kBN];
@@ -241,9 +211,33 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   __syncthreads();
   double t = 0.0;
   if (threadIdx.x == 0)
-    for (int w = 0; w < kXYThreads / 32; ++w) t += red[w];
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
   return t;  // valid in thread 0
 }
+
+// Sums of products of a state's components.  Float32 states: the exact product (as a product
+// and its FMA residual) into a double-float sum, ~2^-44 relative, all on the float32 pipe: a
+// float64 product and sum per term (with its conversions) takes GB300's float64 pipe, two lanes
+// per SM and clock, a dozen times as long as the rest of a subspace gate.
+template <typename T>
+struct Acc {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double a, double b) { s += a * b; }
+  __device__ __forceinline__ void sub(double a, double b) { s -= a * b; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <>
+struct Acc<float2> {
+  float s = 0.f, c = 0.f;
+  __device__ __forceinline__ void add(float a, float b) {
+    const float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p);
+    const float t = __fadd_rn(s, p), bp = __fsub_rn(t, s);
+    c = __fadd_rn(c, __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, bp)), __fsub_rn(p, bp))));
+    s = t;
+  }
+  __device__ __forceinline__ void sub(float a, float b) { add(-a, b); }
+  __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+};
 
 // lambda = C psi, with block partials of [sum C |psi|^2, sum |psi|^2] (E = Re <psi|lambda>)
 template <typename T>
@@ -251,72 +245,137 @@ __global__ void __launch_bounds__(kXYThreads)
     xy_lambda_kernel(const T* __restrict__ psi, T* __restrict__ lam, const void* __restrict__ C, int cost_dtype,
                      unsigned long long D, double* __restrict__ pe, double* __restrict__ pn) {
   __shared__ double red[kXYThreads / 32];
-  double e = 0.0, nn = 0.0;
+  using R = typename Real<T>::type;
+  Acc<T> e, nn;
   for (unsigned long long r = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; r < D;
        r += (unsigned long long)gridDim.x * blockDim.x) {
     const T x = psi[r];
-    const double c = cost_dtype == QAOA_COST_I32 ? (double)((const int*)C)[r] : ((const double*)C)[r];
+    const R c = cost_dtype == QAOA_COST_I32 ? (R)((const int*)C)[r] : (R)((const double*)C)[r];
     T y;
-    y.x = (typename Real<T>::type)c * x.x;
-    y.y = (typename Real<T>::type)c * x.y;
+    y.x = c * x.x;
+    y.y = c * x.y;
     lam[r] = y;
-    const double pr = (double)x.x * (double)x.x + (double)x.y * (double)x.y;
-    e += c * pr;
-    nn += pr;
+    e.add(c, x.x * x.x + x.y * x.y);
+    nn.add(x.x, x.x);
+    nn.add(x.y, x.y);
   }
-  const double se = block_sum(e, red);
+  const double se = block_sum(e.value(), red);
   __syncthreads();
-  const double sn = block_sum(nn, red);
+  const double sn = block_sum(nn.value(), red);
   if (threadIdx.x == 0) {
     pe[blockIdx.x] = se;
     pn[blockIdx.x] = sn;
   }
 }
 
-// one pair gate backwards: the block partial of 2 Im <lambda|K_ab|psi>, then G_ab(-beta) on
-// both buffers (cb = cos beta, sb = -sin beta in the forward gate's formula)
 template <typename T>
+__device__ __forceinline__ void xy_rotate(T& x, T& y, typename Real<T>::type cb, typename Real<T>::type sb) {
+  T u, v;
+  u.x = cb * x.x + sb * y.y;  // cos(beta) x - i sin(beta) y
+  u.y = cb * x.y - sb * y.x;
+  v.x = cb * y.x + sb * x.y;  // cos(beta) y - i sin(beta) x
+  v.y = cb * y.y - sb * x.x;
+  x = u;
+  y = v;
+}
+
+// The closing pair (0, n - 1).  Its gate pairs z (bit 0 set, bit n - 1 clear) with z' (bit 0 clear,
+// bit n - 1 set) over the same middle bits y = bits 1 .. n - 2, popcount(y) = k - 1.  With y's i-th
+// set bit (i = 1, 2, ...) at qubit c_i, rank(z) = sum_i binom(c_i, i + 1) and
+// rank(z') = sum_i binom(c_i, i) + binom(n - 1, k).  The low `lb` bits of y (popcount kl) give the
+// sums' first parts, u16 tables over all their patterns (sorted by kl); the high bits give a pair
+// of bases per column.  So a pair costs two table reads and two additions, with consecutive
+// threads on consecutive patterns; walking all ranks took 250 instructions per amplitude with a
+// quarter of the lanes on a pair (463 us at n = 28, k = 14 complex128, a tenth of a layer).
+constexpr int kCloseBits = 10;   // most low bits: both parts are below binom(11, 5) + ... < 2^16
+constexpr int kCloseCols = 256;  // columns per tile
+constexpr int kClosePairs = 2048;
+struct XYClosing {
+  int n, k, lb, nh, ncls;
+  unsigned long long tiles;
+  struct Cls {
+    unsigned long long first_tile, ncols;
+    int kl, rows, start, m;
+  } cls[kCloseBits + 1];
+};
+
+// TWO: backwards on psi and lambda, taking the gate's term 2 Im <lambda|K|psi> first (one partial
+// per block)
+template <typename T, bool TWO>
 __global__ void __launch_bounds__(kXYThreads)
-    xy_gate_adjoint_kernel(const __grid_constant__ XYShape s, T* __restrict__ psi, T* __restrict__ lam, int qa,
-                           int qb, typename Real<T>::type cb, typename Real<T>::type sb, double* __restrict__ part) {
+    xy_closing_kernel(const __grid_constant__ XYClosing W, T* __restrict__ psi, T* __restrict__ lam,
+                      typename Real<T>::type cb, typename Real<T>::type sb, double* __restrict__ part) {
   __shared__ unsigned long long B[kBN][kBN];
+  __shared__ unsigned short r1[1 << kCloseBits], r0[1 << kCloseBits];
+  __shared__ unsigned long long b1[kCloseCols], b0[kCloseCols];
   __shared__ double red[kXYThreads / 32];
-  load_binom(B, s);
-  const unsigned long long D = s.D, nch = (D + kXYChunk - 1) / kXYChunk;
-  const unsigned long long ma = 1ull << qa, mb = 1ull << qb, below = ma - 1;
-  const bool adjacent = qb == qa + 1;
-  double acc = 0.0;
-  for (unsigned long long ch = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; ch < nch;
-       ch += (unsigned long long)gridDim.x * blockDim.x) {
-    const unsigned long long r0 = ch * kXYChunk, r1 = r0 + kXYChunk < D ? r0 + kXYChunk : D;
-    unsigned long long z = xy_unrank(r0, s.n, s.k, B);
-    for (unsigned long long r = r0; r < r1; ++r) {
-      if ((z & ma) && !(z & mb)) {
-        const unsigned long long rp = adjacent ? r + B[qa][__popcll(z & below)] : xy_rank(z ^ ma ^ mb, B);
-        if (rp < D) {
-          const T x = psi[r], y = psi[rp], lx = lam[r], ly = lam[rp];
-          // Im(conj(lam_z) psi_z' + conj(lam_z') psi_z)
-          acc += (double)lx.x * y.y - (double)lx.y * y.x + (double)ly.x * x.y - (double)ly.y * x.x;
-          T u, v;
-          u.x = cb * x.x + sb * y.y;
-          u.y = cb * x.y - sb * y.x;
-          v.x = cb * y.x + sb * x.y;
-          v.y = cb * y.y - sb * x.x;
-          psi[r] = u;
-          psi[rp] = v;
-          u.x = cb * lx.x + sb * ly.y;
-          u.y = cb * lx.y - sb * ly.x;
-          v.x = cb * ly.x + sb * lx.y;
-          v.y = cb * ly.y - sb * lx.x;
-          lam[r] = u;
-          lam[rp] = v;
-        }
+  const int tid = threadIdx.x;
+  for (int i = tid; i < (W.n + 1) * kBN; i += kXYThreads) (&B[0][0])[i] = (&g_pascal.v[0][0])[i];
+  __syncthreads();
+  for (unsigned x = tid; x < (1u << W.lb); x += kXYThreads) {
+    // place of x among the patterns by popcount, then value; the low parts of both ranks
+    const int kl = __popc(x);
+    unsigned at = 0, u1 = 0, u0 = 0;
+    for (int j = 0; j < kl; ++j) at += (unsigned)B[W.lb][j];
+    unsigned y = x;
+    for (int i = 1; y != 0; ++i) {
+      const int q = __ffs((int)y) - 1;
+      at += (unsigned)B[q][i];
+      u1 += (unsigned)B[q + 1][i + 1];
+      u0 += (unsigned)B[q + 1][i];
+      y &= y - 1;
+    }
+    r1[at] = (unsigned short)u1;
+    r0[at] = (unsigned short)u0;
+  }
+  Acc<T> acc;
+  const unsigned long long t0 = W.tiles * blockIdx.x / gridDim.x, t1 = W.tiles * (blockIdx.x + 1ull) / gridDim.x;
+  int ci = 0;
+  for (unsigned long long tile = t0; tile < t1; ++tile) {
+    while (ci + 1 < W.ncls && W.cls[ci + 1].first_tile <= tile) ++ci;
+    const XYClosing::Cls& C = W.cls[ci];
+    const unsigned long long col0 = (tile - C.first_tile) * (unsigned long long)C.m;
+    const int ncol = (int)(C.ncols - col0 < (unsigned long long)C.m ? C.ncols - col0 : (unsigned long long)C.m);
+    __syncthreads();  // the tables are in; the previous tile is done with the bases
+    for (int c = tid; c < ncol; c += kXYThreads) {
+      unsigned long long h = xyw::unrank_bits(col0 + c, W.nh, W.k - 1 - C.kl, B);
+      unsigned long long s1 = 0, s0 = B[W.n - 1][W.k];
+      for (int i = C.kl + 1; h != 0; ++i) {
+        const int q = W.lb + 1 + __ffsll((long long)h) - 1;
+        s1 += B[q][i + 1];
+        s0 += B[q][i];
+        h &= h - 1;
       }
-      if (r + 1 < r1) z = xy_next(z);
+      b1[c] = s1;
+      b0[c] = s0;
+    }
+    __syncthreads();
+    const int items = C.rows * ncol;
+    const unsigned mg = xyw::div_magic((unsigned)C.rows);
+#pragma unroll 4
+    for (int e = tid; e < items; e += kXYThreads) {
+      const int c = (int)xyw::div_small((unsigned)e, mg), r = e - c * C.rows + C.start;
+      const unsigned long long rz = b1[c] + r1[r], rp = b0[c] + r0[r];
+      T x = psi[rz], y = psi[rp];
+      if constexpr (TWO) {
+        T lx = lam[rz], ly = lam[rp];
+        acc.add(lx.x, y.y);  // Im(conj(lam_z) psi_z' + conj(lam_z') psi_z)
+        acc.sub(lx.y, y.x);
+        acc.add(ly.x, x.y);
+        acc.sub(ly.y, x.x);
+        xy_rotate(lx, ly, cb, sb);
+        lam[rz] = lx;
+        lam[rp] = ly;
+      }
+      xy_rotate(x, y, cb, sb);
+      psi[rz] = x;
+      psi[rp] = y;
     }
   }
-  const double t = block_sum(acc, red);
-  if (threadIdx.x == 0) part[blockIdx.x] = 2.0 * t;
+  if constexpr (TWO) {
+    const double t = block_sum(acc.value(), red);
+    if (tid == 0) part[blockIdx.x] = 2.0 * t;
+  }
 }
 
 // the cost unitary backwards: the block partial of 2 Im <lambda|C|psi>, then both buffers
@@ -375,26 +434,20 @@ __global__ void __launch_bounds__(kXYThreads)
 static_assert(xyw::kMaxN == QAOA_XY_MAX_N, "window tables sized for QAOA_XY_MAX_N");
 static_assert(xyw::kMaxRows <= 128, "tile scale headroom assumes columns of <= 128 rows");
 
-template <typename T>
-__device__ __forceinline__ void xy_rotate(T& x, T& y, typename Real<T>::type cb, typename Real<T>::type sb) {
-  T u, v;
-  u.x = cb * x.x + sb * y.y;  // cos(beta) x - i sin(beta) y
-  u.y = cb * x.y - sb * y.x;
-  v.x = cb * y.x + sb * x.y;  // cos(beta) y - i sin(beta) x
-  v.y = cb * y.y - sb * x.x;
-  x = u;
-  y = v;
-}
-
 // Q62 of |d| <= 1 (from a 2^-61 rounding, so that d = +-1 stays inside from_double's range)
 __device__ __forceinline__ long long xy_q62(double d) { return fx::from_double(d, 61) * 2; }
 
+__device__ __forceinline__ fx::Limbs xy_split4(long long x) {
+  return fx::split((long long)((unsigned long long)x << 2));
+}
 // the same rotation in fixed point: cb, sb as Q62 limbs (nsb = -sb); each part from six limb
-// products (the two low x low ones dropped: within three units of exact rounding)
+// products (the two low x low ones dropped) of operands scaled by 4 (below 2^62), so that the
+// sums need no shift afterwards: within one unit of exact rounding
 __device__ __forceinline__ void xy_rotate_fx(longlong2& x, longlong2& y, fx::Limbs cb, fx::Limbs sb, fx::Limbs nsb) {
-  const fx::Limbs xr = fx::split(x.x), xi = fx::split(x.y), yr = fx::split(y.x), yi = fx::split(y.y);
-  x = make_longlong2(fx::dot2_q62_hi(xr, cb, yi, sb, 0), fx::dot2_q62_hi(xi, cb, yr, nsb, 0));
-  y = make_longlong2(fx::dot2_q62_hi(yr, cb, xi, sb, 0), fx::dot2_q62_hi(yi, cb, xr, nsb, 0));
+  const fx::Limbs xr = xy_split4(x.x), xi = xy_split4(x.y), yr = xy_split4(y.x), yi = xy_split4(y.y);
+  const long long half = 1ll << 31;
+  x = make_longlong2(fx::dot2_hi64(xr, cb, yi, sb, half), fx::dot2_hi64(xi, cb, yr, nsb, half));
+  y = make_longlong2(fx::dot2_hi64(yr, cb, xi, sb, half), fx::dot2_hi64(yi, cb, xr, nsb, half));
 }
 
 // The layer's cost unitary fused into the first window's pass (PH): forward, each amplitude
@@ -411,16 +464,28 @@ struct XYPhaseArgs {
   double* cpart;  // backward: the block partials of the gamma term
 };
 
+// the cost entry of rank r, as both forms the passes use (integer costs: exact in c and ci)
 template <typename T>
-__device__ __forceinline__ T xy_phase_factor(const XYPhaseArgs<T>& ph, unsigned long long r, double& c) {
+__device__ __forceinline__ void xy_cost_at(const XYPhaseArgs<T>& ph, unsigned long long r, double& c, int& ci) {
+  if (ph.cost_dtype == QAOA_COST_I32) ci = __ldg((const int*)ph.C + r);
+  else c = __ldg((const double*)ph.C + r);
+}
+// exp(-i gamma c) of that entry; complex128: in Q62, which is how its table holds the factors
+__device__ __forceinline__ float2 xy_phase_factor(const XYPhaseArgs<float2>& ph, double c, int ci) {
   if (ph.cost_dtype == QAOA_COST_I32) {
-    const long long ci = ((const int*)ph.C)[r];
-    const long long i = ci - ph.cmin;
-    c = (double)ci;
-    return (ph.tab != nullptr && i >= 0 && i < ph.span) ? ph.tab[i] : phase_of(ph.gamma * c, (T*)nullptr);
+    const long long i = (long long)ci - ph.cmin;
+    return (ph.tab != nullptr && i >= 0 && i < ph.span) ? __ldg(ph.tab + i) : phase_of(ph.gamma * ci, (float2*)nullptr);
   }
-  c = ((const double*)ph.C)[r];
-  return phase_of(ph.gamma * c, (T*)nullptr);
+  return phase_of(ph.gamma * c, (float2*)nullptr);
+}
+__device__ __forceinline__ longlong2 xy_phase_factor(const XYPhaseArgs<double2>& ph, double c, int ci) {
+  if (ph.cost_dtype == QAOA_COST_I32) {
+    const long long i = (long long)ci - ph.cmin;
+    if (ph.tab != nullptr && i >= 0 && i < ph.span) return __ldg((const longlong2*)ph.tab + i);
+    c = (double)ci;
+  }
+  const double2 f = phase_of(ph.gamma * c, (double2*)nullptr);
+  return make_longlong2(xy_q62(f.x), xy_q62(f.y));
 }
 
 template <typename T>
@@ -431,67 +496,114 @@ __device__ __forceinline__ T xy_cmul(T x, T f) {
   return y;
 }
 
-// float64 components of a fixed-point tile slot (raw bits while the tile's scale is open)
-__device__ __forceinline__ longlong2 xy_fx_load(const longlong2 raw, int fs) {
-  return make_longlong2(fx::from_double(fx::bits_to_double((unsigned long long)raw.x), fs),
-                        fx::from_double(fx::bits_to_double((unsigned long long)raw.y), fs));
+// Fixed-point tile components from float64 bits and back, for a tile whose largest biased exponent
+// is ep: value = integer x 2^-fs with fs = 56 - (ep - 1022).  Branch-free integer code, since
+// GB300's float64 <-> int64 conversions run on the float64 pipe (64 cycles per warp each).
+// In: round half away from zero, as fx::from_double; |result| < 2^56.
+__device__ __forceinline__ long long xy_fx_in(long long raw, int ep) {
+  const unsigned long long bits = (unsigned long long)raw;
+  const int ex = (int)(bits >> 52) & 0x7FF;
+  const int d = ex == 0 ? 63 : min(ep - ex, 63);  // zero and subnormals: below every resolution
+  const unsigned long long m = ((bits & ((1ull << 52) - 1)) | (1ull << 52)) << 3;
+  const long long r = (long long)((m + ((1ull << d) >> 1)) >> d);
+  const long long s = raw >> 63;
+  return (r ^ s) - s;
+}
+// Out: float64 nearest to x 2^-fs (halves away from zero); x != 0 lies in float64's normal range.
+__device__ __forceinline__ double xy_fx_out(long long x, int fs) {
+  const long long s = x >> 63;
+  const unsigned long long a = (unsigned long long)((x ^ s) - s);
+  const int lz = __clzll((long long)a);
+  const unsigned long long m = a << (lz & 63);  // leading one at bit 63
+  const unsigned long long keep = (m >> 11) + ((m >> 10) & 1ull);  // 53 bits; a carry moves to the exponent
+  // biased exponent of the leading one, less the one that keep's top bit adds
+  const unsigned long long b = ((unsigned long long)(unsigned)(63 - lz - fs + 1022) << 52) + keep;
+  return a == 0 ? 0.0 : __longlong_as_double((long long)(b | ((unsigned long long)s << 63)));
 }
 __device__ __forceinline__ unsigned xy_exp_bits(double2 v) {
   const unsigned long long bx = fx::double_to_bits(v.x), by = fx::double_to_bits(v.y);
   return max((unsigned)(bx >> 52) & 0x7FFu, (unsigned)(by >> 52) & 0x7FFu);
 }
-// x * f (conj(f) when CONJ) for a fixed-point x and a unit float64 factor f, as Q62 limbs
+// x * f (conj(f) when CONJ) for a fixed-point x below 2^59 and a Q62 unit factor f
 template <bool CONJ>
-__device__ __forceinline__ longlong2 xy_fx_phase(longlong2 x, double2 f) {
-  const long long fre = xy_q62(f.x), fim = xy_q62(CONJ ? -f.y : f.y);
-  const fx::Limbs fr = fx::split(fre), fi = fx::split(fim), nfi = fx::split(-fim);
-  const fx::Limbs xr = fx::split(x.x), xi = fx::split(x.y);
-  return make_longlong2(fx::dot2_q62_hi(xr, fr, xi, nfi, 0), fx::dot2_q62_hi(xr, fi, xi, fr, 0));
+__device__ __forceinline__ longlong2 xy_fx_phase(longlong2 x, longlong2 f) {
+  const fx::C64 o = fx::cmul_unit<CONJ>(x.x, x.y, fx::factor(f.x, f.y));
+  return make_longlong2(o.x, o.y);
 }
 
+constexpr int xy_window_threads(bool two) { return two ? 512 : 256; }
+// amplitudes per tile and buffer: a class of 126 (70, 36, 9) rows takes 16 (32, 64, 256) columns
+// of complex128; column-major tiles pad each row by one slot
+template <typename T>
+constexpr int xy_tile_elems() {
+  return 36864 / (int)sizeof(T);
+}
+template <typename T>
+constexpr size_t xy_buffer_bytes() {
+  return (size_t)(xy_tile_elems<T>() + xyw::kMaxRows + 2) * sizeof(T);
+}
+// dynamic shared memory: the binomials up to n, then the tiles
+__host__ __device__ inline size_t xy_binom_bytes(int n) {
+  return ((size_t)(n + 1) * xyw::kBN * sizeof(unsigned long long) + 15) & ~(size_t)15;
+}
+
+// A block walks consecutive tiles (mostly of one class, whose row tables it then keeps).  A
+// tile's rows stay row-major in shared memory, columns fastest, so in every gate consecutive
+// threads take consecutive columns of one pair of rows: no bank conflicts, and the pair comes
+// from the item index by a shift.  Tiles whose columns are runs of consecutive ranks (len = 1)
+// are read and written column by column and only stored row-major, rows padded by one slot.
+// With the closing pair's pass above: n = 30, k = 15, p = 3 layers 57.4 -> 47.4 ms complex128,
+// n = 27, k = 12, p = 2 gradient 10.4 -> 4.0 ms complex64.  Bound: the per-tile work (rotations and
+// conversions) and its latency at four blocks per SM, not memory.
 template <typename T, bool TWO, bool PH>
-__global__ void __launch_bounds__(kXYThreads)
+__global__ void __launch_bounds__(xy_window_threads(TWO), TWO ? 2 : 4)
     xy_window_kernel(const __grid_constant__ xyw::Window W, T* __restrict__ psi, T* __restrict__ lam,
-                     typename Real<T>::type cb, typename Real<T>::type sb, double* __restrict__ part,
+                     typename Real<T>::type cb, typename Real<T>::type sb, double* __restrict__ part, int part_cols,
                      const __grid_constant__ XYPhaseArgs<T> ph) {
   constexpr bool FXR = std::is_same<T, double2>::value;  // complex128: fixed-point tiles
   using S = typename std::conditional<FXR, longlong2, T>::type;
-  __shared__ unsigned long long B[xyw::kBN][xyw::kBN];
+  constexpr int NT = xy_window_threads(TWO);
   __shared__ unsigned long long rowoff[xyw::kMaxRows];
   __shared__ unsigned long long colbase[xyw::kMaxCols];
   __shared__ unsigned short rowpat[xyw::kMaxRows];
-  __shared__ unsigned char pr0[xyw::kMaxGates][xyw::kMaxPairs], pr1[xyw::kMaxGates][xyw::kMaxPairs];
+  __shared__ unsigned prow[xyw::kMaxGates][xyw::kMaxPairs];  // row slots of each gate's pairs: low | high << 16
   __shared__ int npr[xyw::kMaxGates];
-  __shared__ double red[kXYThreads / 32];
+  __shared__ double red[NT / 32];
   __shared__ unsigned tile_ex[2];  // fixed-point tiles: largest biased float64 exponent of psi, lambda
   extern __shared__ __align__(16) unsigned char xy_win_smem[];
-  S* tp = (S*)xy_win_smem;     // psi tile
-  S* tl = tp + W.tile_elems;   // lambda tile (TWO)
+  unsigned long long(*B)[xyw::kBN] = (unsigned long long(*)[xyw::kBN])xy_win_smem;
+  S* tp = (S*)(xy_win_smem + xy_binom_bytes(W.n));           // psi tile
+  S* tl = (S*)((unsigned char*)tp + xy_buffer_bytes<T>());   // lambda tile (TWO)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int c = tid; c < xyw::kBN; c += kXYThreads) xyw::binom_row(B, c);
+  for (int i = tid; i < (W.n + 1) * xyw::kBN; i += NT) (&B[0][0])[i] = (&g_pascal.v[0][0])[i];
   fx::Limbs qc = {0, 0}, qs = {0, 0}, qns = {0, 0};
   if constexpr (FXR) {
     qc = fx::split(xy_q62((double)cb));
     qs = fx::split(xy_q62((double)sb));
     qns = fx::split(-xy_q62((double)sb));
   }
-  double acc = 0.0, cacc = 0.0;
+  Acc<T> acc, cacc;
+  double cacc_d = 0.0;
   int cur = -1;  // class whose row tables are in shared memory (the same in every thread)
-  for (unsigned long long tile = blockIdx.x; tile < W.tiles; tile += gridDim.x) {
-    const int ci = xyw::find_class(W, tile);
+  const unsigned long long t0 = W.tiles * blockIdx.x / gridDim.x, t1 = W.tiles * (blockIdx.x + 1ull) / gridDim.x;
+  int ci = t0 < t1 ? xyw::find_class(W, t0) : 0;
+  for (unsigned long long tile = t0; tile < t1; ++tile) {
+    while (ci + 1 < W.ncls && W.cls[ci + 1].first_tile <= tile) ++ci;
     const xyw::Class& C = W.cls[ci];
-    const int rows = C.rows;
-    const unsigned long long col0 = (tile - C.first_tile) * (unsigned long long)C.m;
-    const int ncol = (int)(C.ncols - col0 < (unsigned long long)C.m ? C.ncols - col0 : (unsigned long long)C.m);
-    __syncthreads();  // Pascal's triangle is ready; the previous tile is stored
+    const int rows = C.rows, mb = C.mb, m = 1 << mb;
+    const unsigned long long col0 = (tile - C.first_tile) << mb;
+    const int ncol = (int)(C.ncols - col0 < (unsigned long long)m ? C.ncols - col0 : (unsigned long long)m);
+    const bool cm = C.len == 1;  // a column's rows are consecutive ranks
+    const int stride = cm ? m + 1 : m;
+    __syncthreads();  // the binomials are in; the previous tile is stored
     if (ci != cur) {  // row patterns, their rank parts, and each gate's moved rows
-      for (int r = tid; r < rows; r += kXYThreads) {
+      for (int r = tid; r < rows; r += NT) {
         const unsigned long long P = xyw::unrank_bits((unsigned long long)r, W.w, C.kw, B);
         rowpat[r] = (unsigned short)P;
         rowoff[r] = xyw::rank_part(P, W.lo, C.kL, B);
       }
       __syncthreads();
-      for (int g = warp; g < W.ngates; g += kXYThreads / 32) {
+      for (int g = warp; g < W.ngates; g += NT / 32) {
         const int ga = W.ga[g];
         int cnt = 0;
         for (int base = 0; base < rows; base += 32) {
@@ -499,52 +611,48 @@ __global__ void __launch_bounds__(kXYThreads)
           const unsigned P = r < rows ? rowpat[r] : 0u;
           const bool mv = r < rows && ((P >> ga) & 3u) == 1u;
           const unsigned bal = __ballot_sync(0xffffffffu, mv);
-          if (mv) {
-            const int q = cnt + __popc(bal & ((1u << lane) - 1u));
-            pr0[g][q] = (unsigned char)r;
-            pr1[g][q] = (unsigned char)xyw::partner_row(r, P, ga, B);
-          }
+          if (mv)
+            prow[g][cnt + __popc(bal & ((1u << lane) - 1u))] =
+                (unsigned)(r * stride) | (unsigned)(xyw::partner_row(r, P, ga, B) * stride) << 16;
           cnt += __popc(bal);
         }
         if (lane == 0) npr[g] = cnt;
       }
       cur = ci;
     }
-    for (int c = tid; c < ncol; c += kXYThreads) colbase[c] = xyw::col_base(W, C, col0 + c, B);
+    for (int c = tid; c < ncol; c += NT) colbase[c] = xyw::col_base(W, C, col0 + c, B);
     if (FXR && tid == 0) tile_ex[0] = tile_ex[1] = 0;
     __syncthreads();
-    // element e of the tile: column-major when a column's rows are consecutive ranks (len = 1),
-    // otherwise row-major, so consecutive threads touch consecutive ranks
-    const bool cm = C.len == 1;
-    const unsigned inner = cm ? (unsigned)rows : (unsigned)ncol;  // < 2^16
-    const unsigned mg = xyw::div_magic(inner);
-    const int ne = rows * ncol;
+    // element e of the tile in memory order; slots past the last column are skipped
+    const int ns = cm ? rows * ncol : rows << mb;
+    const unsigned mg = xyw::div_magic((unsigned)rows);
+    auto place = [&](int e, int& r, int& c) {
+      if (cm) {
+        c = (int)xyw::div_small((unsigned)e, mg);
+        r = e - c * rows;
+      } else {
+        r = e >> mb;
+        c = e & (m - 1);
+      }
+      return c < ncol;
+    };
     unsigned exp_psi = 0, exp_lam = 0;
-    for (int e = tid; e < ne; e += kXYThreads) {
-      const unsigned o = xyw::div_small((unsigned)e, mg), i = (unsigned)e - o * inner;
-      const int r = cm ? (int)i : (int)o, c = cm ? (int)o : (int)i;
-      const unsigned long long rk = rowoff[r] + colbase[c];
-      const T x = psi[rk];
-      if constexpr (FXR) {  // raw bits for now; the exponents give the tile's scales
+    int fs = 0, fl = 0;  // fixed-point tiles: psi value = integer x 2^-fs, lambda 2^-fl
+    if constexpr (FXR) {
+#pragma unroll 2
+      for (int e = tid; e < ns; e += NT) {
+        int r, c;
+        if (!place(e, r, c)) continue;
+        const unsigned long long rk = rowoff[r] + colbase[c];
+        const T x = psi[rk];  // raw bits for now; the exponents give the tile's scales
         exp_psi = max(exp_psi, xy_exp_bits(x));
-        tp[e] = make_longlong2((long long)fx::double_to_bits(x.x), (long long)fx::double_to_bits(x.y));
+        tp[r * stride + c] = make_longlong2((long long)fx::double_to_bits(x.x), (long long)fx::double_to_bits(x.y));
         if constexpr (TWO) {
           const T l = lam[rk];
           exp_lam = max(exp_lam, xy_exp_bits(l));
-          tl[e] = make_longlong2((long long)fx::double_to_bits(l.x), (long long)fx::double_to_bits(l.y));
+          tl[r * stride + c] = make_longlong2((long long)fx::double_to_bits(l.x), (long long)fx::double_to_bits(l.y));
         }
-      } else {
-        T v = x;
-        if constexpr (PH && !TWO) {
-          double cv;
-          v = xy_cmul(v, xy_phase_factor(ph, rk, cv));
-        }
-        tp[e] = v;
-        if constexpr (TWO) tl[e] = lam[rk];
       }
-    }
-    int fs = 0, fl = 0;  // fixed-point tiles: psi value = integer x 2^-fs, lambda 2^-fl
-    if constexpr (FXR) {
       exp_psi = __reduce_max_sync(0xffffffffu, exp_psi);
       if (lane == 0) atomicMax(&tile_ex[0], exp_psi);
       if constexpr (TWO) {
@@ -552,37 +660,52 @@ __global__ void __launch_bounds__(kXYThreads)
         if (lane == 0) atomicMax(&tile_ex[1], exp_lam);
       }
       __syncthreads();
-      fs = 56 - ((int)tile_ex[0] - 1022);  // every component is below 2^(tile_ex - 1022)
-      fl = 56 - ((int)tile_ex[1] - 1022);
-      for (int e = tid; e < ne; e += kXYThreads) {  // the slots this thread loaded
-        longlong2 X = xy_fx_load(tp[e], fs);
+      const int ep = (int)tile_ex[0], el = (int)tile_ex[1];
+      fs = 56 - (ep - 1022);  // every component is below 2^(ep - 1022)
+      fl = 56 - (el - 1022);
+#pragma unroll 2
+      for (int e = tid; e < ns; e += NT) {  // the slots this thread loaded
+        int r, c;
+        if (!place(e, r, c)) continue;
+        const int at = r * stride + c;
+        longlong2 X = make_longlong2(xy_fx_in(tp[at].x, ep), xy_fx_in(tp[at].y, ep));
         if constexpr (PH && !TWO) {  // the layer's cost unitary; a unit factor keeps the bound
-          const unsigned o = xyw::div_small((unsigned)e, mg), i = (unsigned)e - o * inner;
-          const int r = cm ? (int)i : (int)o, c = cm ? (int)o : (int)i;
-          double cv;
-          X = xy_fx_phase<false>(X, xy_phase_factor(ph, rowoff[r] + colbase[c], cv));
+          double cf = 0.0;
+          int cI = 0;
+          xy_cost_at(ph, rowoff[r] + colbase[c], cf, cI);
+          X = xy_fx_phase<false>(X, xy_phase_factor(ph, cf, cI));
         }
-        tp[e] = X;
-        if constexpr (TWO) tl[e] = xy_fx_load(tl[e], fl);
+        tp[at] = X;
+        if constexpr (TWO) tl[at] = make_longlong2(xy_fx_in(tl[at].x, el), xy_fx_in(tl[at].y, el));
+      }
+    } else {
+#pragma unroll 6
+      for (int e = tid; e < ns; e += NT) {
+        int r, c;
+        if (!place(e, r, c)) continue;
+        const unsigned long long rk = rowoff[r] + colbase[c];
+        T v = psi[rk];
+        if constexpr (PH && !TWO) {
+          double cf = 0.0;
+          int cI = 0;
+          xy_cost_at(ph, rk, cf, cI);
+          v = xy_cmul(v, xy_phase_factor(ph, cf, cI));
+        }
+        tp[r * stride + c] = v;
+        if constexpr (TWO) tl[r * stride + c] = lam[rk];
       }
     }
     __syncthreads();
-    // gates one after another, each gate's (pair, column) items spread over the block:
-    // consecutive threads take consecutive columns (row-major tiles) or consecutive pairs of
-    // one column (column-major tiles), so shared-memory accesses stay conflict-free
+    // gates one after another, each gate's (pair, column) items spread over the block
     fx::i128 tacc = 0;  // fixed point: this thread's gate terms of the tile, x 2^-(fs + fl - 4)
     for (int gi = 0; gi < W.ngates; ++gi) {
       const int g = TWO ? W.ngates - 1 - gi : gi;
-      const int np = npr[g];
-      const int items = np * ncol;
-      const unsigned in2 = cm ? (unsigned)np : (unsigned)ncol;
-      const unsigned m2 = xyw::div_magic(in2);
-      for (int it = tid; it < items; it += kXYThreads) {
-        const unsigned o = xyw::div_small((unsigned)it, m2), i = (unsigned)it - o * in2;
-        const int q = cm ? (int)i : (int)o, c = cm ? (int)o : (int)i;
-        const int r0 = pr0[g][q], r1 = pr1[g][q];
-        const int s0 = cm ? c * rows + r0 : r0 * ncol + c;
-        const int s1 = cm ? c * rows + r1 : r1 * ncol + c;
+      const int items = npr[g] << mb;
+      for (int it = tid; it < items; it += NT) {
+        const int c = it & (m - 1);
+        if (c >= ncol) continue;
+        const unsigned pr = prow[g][it >> mb];
+        const int s0 = (int)(pr & 0xffffu) + c, s1 = (int)(pr >> 16) + c;
         S x = tp[s0], y = tp[s1];
         if constexpr (TWO) {
           S lx = tl[s0], ly = tl[s1];
@@ -590,7 +713,10 @@ __global__ void __launch_bounds__(kXYThreads)
             tacc += (fx::dot2_exact(lx.x, y.y, lx.y, y.x) + fx::dot2_exact(ly.x, x.y, ly.y, x.x)) >> 4;
             xy_rotate_fx(lx, ly, qc, qs, qns);
           } else {
-            acc += (double)lx.x * y.y - (double)lx.y * y.x + (double)ly.x * x.y - (double)ly.y * x.x;
+            acc.add(lx.x, y.y);
+            acc.sub(lx.y, y.x);
+            acc.add(ly.x, x.y);
+            acc.sub(ly.y, x.x);
             xy_rotate(lx, ly, cb, sb);
           }
           tl[s0] = lx;
@@ -603,53 +729,59 @@ __global__ void __launch_bounds__(kXYThreads)
       }
       __syncthreads();
     }
-    if constexpr (FXR && TWO) acc += fx::i128_to_double(tacc, fs + fl - 4);
+    if constexpr (FXR && TWO) acc.s += fx::i128_to_double(tacc, fs + fl - 4);
     fx::i128 cacc_i = 0;  // fixed point, integer costs: sum of c (conj(lambda) psi products >> 32)
-    for (int e = tid; e < ne; e += kXYThreads) {
-      const unsigned o = xyw::div_small((unsigned)e, mg), i = (unsigned)e - o * inner;
-      const int r = cm ? (int)i : (int)o, c = cm ? (int)o : (int)i;
+#pragma unroll 3
+    for (int e = tid; e < ns; e += NT) {
+      int r, c;
+      if (!place(e, r, c)) continue;
       const unsigned long long rk = rowoff[r] + colbase[c];
-      if constexpr (FXR) {
-        longlong2 X = tp[e];
-        if constexpr (TWO) {
-          longlong2 L = tl[e];
-          if constexpr (PH) {  // the gamma term at the state right after the cost unitary, then undo it
-            double cv;
-            const T f = xy_phase_factor(ph, rk, cv);
-            const fx::i128 pr = fx::dot2_exact(L.x, X.y, L.y, X.x);  // Im(conj(lambda) psi)
-            if (ph.cost_dtype == QAOA_COST_I32) cacc_i += (pr >> 32) * (long long)cv;
-            else cacc += cv * fx::i128_to_double(pr, fs + fl);
-            X = xy_fx_phase<true>(X, f);
-            L = xy_fx_phase<true>(L, f);
+      S X = tp[r * stride + c], L;
+      if constexpr (TWO) L = tl[r * stride + c];
+      if constexpr (TWO && PH) {  // the gamma term at the state right after the cost unitary, then undo it
+        double cf = 0.0;
+        int cI = 0;
+        xy_cost_at(ph, rk, cf, cI);
+        if constexpr (FXR) {
+          const longlong2 f = xy_phase_factor(ph, cf, cI);
+          const fx::i128 pr = fx::dot2_exact(L.x, X.y, L.y, X.x);  // Im(conj(lambda) psi)
+          if (ph.cost_dtype == QAOA_COST_I32) cacc_i += (pr >> 32) * (long long)cI;
+          else cacc_d += cf * fx::i128_to_double(pr, fs + fl);
+          X = xy_fx_phase<true>(X, f);
+          L = xy_fx_phase<true>(L, f);
+        } else {
+          T f = xy_phase_factor(ph, cf, cI);
+          if (ph.cost_dtype == QAOA_COST_I32 && abs((long long)cI) <= (1 << 24)) {  // c exact in float32
+            cacc.add((float)cI * L.x, X.y);
+            cacc.sub((float)cI * L.y, X.x);
+          } else {
+            const double cv = ph.cost_dtype == QAOA_COST_I32 ? (double)cI : cf;
+            cacc_d += cv * ((double)L.x * X.y - (double)L.y * X.x);
           }
-          lam[rk] = make_double2(fx::to_double(L.x, fl), fx::to_double(L.y, fl));
-        }
-        psi[rk] = make_double2(fx::to_double(X.x, fs), fx::to_double(X.y, fs));
-      } else if constexpr (TWO) {
-        T x = tp[e], l = tl[e];
-        if constexpr (PH) {
-          double cv;
-          T f = xy_phase_factor(ph, rk, cv);
-          cacc += cv * ((double)l.x * x.y - (double)l.y * x.x);
           f.y = -f.y;  // exp(+i gamma c)
-          x = xy_cmul(x, f);
-          l = xy_cmul(l, f);
+          X = xy_cmul(X, f);
+          L = xy_cmul(L, f);
         }
-        psi[rk] = x;
-        lam[rk] = l;
+      }
+      if constexpr (FXR) {
+        psi[rk] = make_double2(xy_fx_out(X.x, fs), xy_fx_out(X.y, fs));
+        if constexpr (TWO) lam[rk] = make_double2(xy_fx_out(L.x, fl), xy_fx_out(L.y, fl));
       } else {
-        psi[rk] = tp[e];
+        psi[rk] = X;
+        if constexpr (TWO) lam[rk] = L;
       }
     }
-    if constexpr (FXR && TWO && PH) cacc += fx::i128_to_double(cacc_i, fs + fl - 32);
+    if constexpr (FXR && TWO && PH) cacc_d += fx::i128_to_double(cacc_i, fs + fl - 32);
   }
-  if constexpr (TWO) {
-    const double t = block_sum(acc, red);
-    if (tid == 0) part[blockIdx.x] = 2.0 * t;
+  if constexpr (TWO) {  // one partial per block; the row's slots past the grid are zero
+    const double t = block_sum(acc.value(), red);
+    if (tid == 0)
+      for (int j = blockIdx.x; j < part_cols; j += gridDim.x) part[j] = j == (int)blockIdx.x ? 2.0 * t : 0.0;
     if constexpr (PH) {
       __syncthreads();
-      const double tc = block_sum(cacc, red);
-      if (tid == 0) ph.cpart[blockIdx.x] = 2.0 * tc;
+      const double tc = block_sum(cacc.value() + cacc_d, red);
+      if (tid == 0)
+        for (int j = blockIdx.x; j < part_cols; j += gridDim.x) ph.cpart[j] = j == (int)blockIdx.x ? 2.0 * tc : 0.0;
     }
   }
 }
@@ -757,6 +889,7 @@ __global__ void __launch_bounds__(kXYThreads) xy_finish_kernel(const double* __r
 struct XYTableArgs {
   double gam[QAOA_MAX_P];
   int p;
+  int q62;  // complex128: Q62 entries (the window passes) instead of float64 ones
   long long cmin, span;
   void* tab;
 };
@@ -767,7 +900,9 @@ __global__ void xy_tables_kernel(const __grid_constant__ XYTableArgs a) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
     const int l = (int)(i / a.span);
-    ((T*)a.tab)[i] = phase_of(a.gam[l] * (double)(a.cmin + i % a.span), (T*)nullptr);
+    const T f = phase_of(a.gam[l] * (double)(a.cmin + i % a.span), (T*)nullptr);
+    if (std::is_same<T, double2>::value && a.q62) ((longlong2*)a.tab)[i] = make_longlong2(xy_q62(f.x), xy_q62(f.y));
+    else ((T*)a.tab)[i] = f;
   }
 }
 
@@ -876,7 +1011,7 @@ int expectation_t(const XYShape& s, const T* psi, const qaoa_cost_t* cost, doubl
   return status_of(cudaGetLastError());
 }
 
-// The windows of the ring mixer for (n, k), 0 < k < n, n >= 2: tiles of 32 KB of amplitudes
+// The windows of the ring mixer for (n, k), 0 < k < n, n >= 2: tiles of 36 KB of amplitudes
 // per buffer; the first window visits every amplitude, since the layer's cost unitary rides
 // on its pass; the closing pair (0, n - 1) (n >= 3) is a per-gate pass after the windows.
 struct XYMixPlan {
@@ -891,49 +1026,73 @@ XYMixPlan* make_mix_plan(const XYShape& s) {
   int lo[xyw::kMaxWindows + 1], w[xyw::kMaxWindows + 1];
   mp->nwin = xyw::plan_ring_windows(s.n, lo, w);
   for (int i = 0; i < mp->nwin; ++i)
-    xyw::plan_window(mp->win[i], s.n, s.k, lo[i], w[i], (int)(32768 / sizeof(T)), s.binom, i == 0);
+    xyw::plan_window(mp->win[i], s.n, s.k, lo[i], w[i], xy_tile_elems<T>(), s.binom, i == 0);
   mp->closing = s.n >= 3;
   return mp;
 }
 
-template <typename T, bool TWO>
-size_t window_smem(const xyw::Window& W) {
-  return (size_t)W.tile_elems * sizeof(T) * (TWO ? 2 : 1);
-}
-
-// one windowed pass; grid = 0 takes every SM's resident blocks (forward), the gradient passes
-// its partial-row grid
+// one windowed pass on every SM's resident blocks; part_cols: the partial slots of a row (backward)
 template <typename T, bool TWO, bool PH>
 cudaError_t launch_window(const xyw::Window& W, T* psi, T* lam, typename Real<T>::type cb,
-                          typename Real<T>::type sb, double* part, const XYPhaseArgs<T>& ph, unsigned grid,
+                          typename Real<T>::type sb, double* part, int part_cols, const XYPhaseArgs<T>& ph,
                           cudaStream_t st) {
   static std::mutex mu;
   static unsigned long long done = 0;
-  static int per_sm = 1;
-  const size_t max_smem = (size_t)32768 * (TWO ? 2 : 1);  // tiles hold <= 32 KB of amplitudes per buffer
+  static int per_sm[64] = {};
+  constexpr int NT = xy_window_threads(TWO);
+  const size_t smem = xy_binom_bytes(W.n) + xy_buffer_bytes<T>() * (TWO ? 2 : 1);
+  int dev = 0;
+  cudaGetDevice(&dev);
+  int resident;
   {
-    int dev = 0;
-    cudaGetDevice(&dev);
     std::lock_guard<std::mutex> lk(mu);
     if (!(done & (1ull << (dev & 63)))) {
-      cudaFuncSetAttribute(xy_window_kernel<T, TWO, PH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xy_window_kernel<T, TWO, PH>, kXYThreads, max_smem);
-      if (per_sm < 1) per_sm = 1;
+      const size_t most = xy_binom_bytes(xyw::kMaxN) + xy_buffer_bytes<T>() * (TWO ? 2 : 1);
+      cudaFuncSetAttribute(xy_window_kernel<T, TWO, PH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[dev & 63], xy_window_kernel<T, TWO, PH>, NT,
+                                                    xy_binom_bytes(32) + xy_buffer_bytes<T>() * (TWO ? 2 : 1));
+      if (per_sm[dev & 63] < 1) per_sm[dev & 63] = 1;
       done |= 1ull << (dev & 63);
     }
+    resident = per_sm[dev & 63];
   }
   if (W.tiles == 0) return cudaSuccess;
-  if (window_smem<T, TWO>(W) > max_smem) return cudaErrorInvalidValue;
-  if (grid == 0) {
-    const unsigned long long g = (unsigned long long)sm_count() * per_sm;
-    grid = (unsigned)(W.tiles < g ? W.tiles : g);
-  }
+  if (W.tile_elems > xy_tile_elems<T>()) return cudaErrorInvalidValue;
+  unsigned long long g = (unsigned long long)sm_count() * resident;
+  if (TWO && g > (unsigned long long)part_cols) g = part_cols;
+  const unsigned grid = (unsigned)(W.tiles < g ? W.tiles : g);
   const double cb_bytes = PH ? (double)W.elems * cost_bytes(ph.cost_dtype) : 0.0;
   const double bytes = (double)W.elems * sizeof(T) * 2 * (TWO ? 2 : 1) + cb_bytes;
   note_launch(0, st, true);
-  xy_window_kernel<T, TWO, PH><<<grid, kXYThreads, window_smem<T, TWO>(W), st>>>(W, psi, lam, cb, sb, part, ph);
+  xy_window_kernel<T, TWO, PH><<<grid, NT, smem, st>>>(W, psi, lam, cb, sb, part, part_cols, ph);
   note_launch(0, st, false, bytes);
   return cudaGetLastError();
+}
+
+// the closing pair's classes and tiles (n >= 3, 0 < k < n)
+XYClosing make_closing(const XYShape& s) {
+  XYClosing W;
+  std::memset(&W, 0, sizeof(W));
+  W.n = s.n;
+  W.k = s.k;
+  W.lb = std::max(0, std::min(kCloseBits, s.n - 2));
+  W.nh = std::max(0, s.n - 2 - W.lb);
+  int start = 0;
+  for (int kl = 0; kl <= W.lb; ++kl) {
+    const int rows = (int)s.binom[W.lb][kl], kh = s.k - 1 - kl;
+    if (kh >= 0 && kh <= W.nh) {
+      XYClosing::Cls& C = W.cls[W.ncls++];
+      C.kl = kl;
+      C.rows = rows;
+      C.start = start;
+      C.ncols = s.binom[W.nh][kh];
+      C.m = std::max(1, std::min(kCloseCols, kClosePairs / rows));
+      C.first_tile = W.tiles;
+      W.tiles += (C.ncols + C.m - 1) / C.m;
+    }
+    start += rows;
+  }
+  return W;
 }
 
 template <typename T>
@@ -957,6 +1116,7 @@ int layers_t(const XYShape& s, T* psi, const qaoa_cost_t* cost, const double* ga
     ta.p = p;
     ta.cmin = cost->cmin;
     ta.span = span;
+    ta.q62 = s.k > 0 && s.k < s.n && s.n >= 2;
     ta.tab = tab;
     note_launch(3, st, true);
     xy_tables_kernel<T><<<grid_for((unsigned long long)p * span, sms), kXYThreads, 0, st>>>(ta);
@@ -965,7 +1125,8 @@ int layers_t(const XYShape& s, T* psi, const qaoa_cost_t* cost, const double* ga
   const bool mixes = s.k > 0 && s.k < s.n && s.n >= 2;
   XYMixPlan* mp = mixes && p > 0 ? make_mix_plan<T>(s) : nullptr;
   const unsigned long long moved = s.n >= 2 && s.k >= 1 && s.k <= s.n - 1 ? 2 * s.binom[s.n - 2][s.k - 1] : 0;
-  const unsigned long long nch = (s.D + kXYChunk - 1) / kXYChunk;
+  const XYClosing cw = make_closing(s);
+  const unsigned cgrid = (unsigned)std::max<unsigned long long>(1, std::min<unsigned long long>(cw.tiles, (unsigned)sms * 6u));
   for (int l = 0; l < p; ++l) {
     const XYPhaseArgs<T> ph = {cost->C_dev, cost->dtype, tab ? tab + (size_t)l * span : nullptr, cost->cmin, span,
                                gamma[l], nullptr};
@@ -979,8 +1140,8 @@ int layers_t(const XYShape& s, T* psi, const qaoa_cost_t* cost, const double* ga
     if (mp != nullptr) {  // the cost unitary on the first window's pass, the ring mixer, the closing pair
       for (int i = 0; i < mp->nwin; ++i) {
         const cudaError_t e =
-            i == 0 ? launch_window<T, false, true>(mp->win[i], psi, nullptr, cb, snb, nullptr, ph, 0, st)
-                   : launch_window<T, false, false>(mp->win[i], psi, nullptr, cb, snb, nullptr, ph, 0, st);
+            i == 0 ? launch_window<T, false, true>(mp->win[i], psi, nullptr, cb, snb, nullptr, 0, ph, st)
+                   : launch_window<T, false, false>(mp->win[i], psi, nullptr, cb, snb, nullptr, 0, ph, st);
         if (e != cudaSuccess) {
           delete mp;
           return QAOA_ERR_CUDA;
@@ -988,7 +1149,7 @@ int layers_t(const XYShape& s, T* psi, const qaoa_cost_t* cost, const double* ga
       }
       if (mp->closing) {
         note_launch(0, st, true);
-        xy_gate_kernel<T><<<grid_for(nch, sms), kXYThreads, 0, st>>>(s, psi, 0, s.n - 1, cb, snb);
+        xy_closing_kernel<T, false><<<cgrid, kXYThreads, 0, st>>>(cw, psi, nullptr, cb, snb, nullptr);
         note_launch(0, st, false, (double)moved * 2 * sb);
       }
     }
@@ -1032,9 +1193,9 @@ int gradient_t(const XYShape& s, T* psi, T* lam, const qaoa_cost_t* cost, const 
   note_launch(0, st, true);
   xy_lambda_kernel<T><<<gr, kXYThreads, 0, st>>>(psi, lam, cost->C_dev, cost->dtype, s.D, part, part + kXYPartStride);
   note_launch(0, st, false, (double)s.D * (2 * sb + cost_bytes(cost->dtype)));
-  // beta rows of layer l: one per window and one for the closing pair (at most np of them),
-  // every row written by a launch of gg blocks
+  // beta rows of layer l: one per window and one for the closing pair (at most np of them), every row's gg slots written
   XYMixPlan* mp = np > 0 && p > 0 ? make_mix_plan<T>(s) : nullptr;
+  const XYClosing cw = make_closing(s);
   const int brows = mp != nullptr ? mp->nwin + (mp->closing ? 1 : 0) : 0;
   const bool fused = mp != nullptr;  // gamma terms from the first window's pass (gg blocks)
   for (int l = p - 1; l >= 0; --l) {
@@ -1043,8 +1204,8 @@ int gradient_t(const XYShape& s, T* psi, T* lam, const qaoa_cost_t* cost, const 
     if (mp != nullptr) {
       if (mp->closing) {  // applied last in the layer, undone first
         note_launch(0, st, true);
-        xy_gate_adjoint_kernel<T><<<gg, kXYThreads, 0, st>>>(s, psi, lam, 0, s.n - 1, cb, snb,
-                                                              rows + (size_t)mp->nwin * kXYPartStride);
+        xy_closing_kernel<T, true><<<gg, kXYThreads, 0, st>>>(cw, psi, lam, cb, snb,
+                                                               rows + (size_t)mp->nwin * kXYPartStride);
         note_launch(0, st, false, (double)moved * 4 * sb);
       }
       // the first window's pass also takes the gamma term and undoes the cost unitary
@@ -1052,8 +1213,8 @@ int gradient_t(const XYShape& s, T* psi, T* lam, const qaoa_cost_t* cost, const 
                                  span, gamma[l], part + (size_t)(2 + l) * kXYPartStride};
       for (int i = mp->nwin - 1; i >= 0; --i) {
         double* row = rows + (size_t)i * kXYPartStride;
-        const cudaError_t e = i == 0 ? launch_window<T, true, true>(mp->win[i], psi, lam, cb, snb, row, ph, gg, st)
-                                     : launch_window<T, true, false>(mp->win[i], psi, lam, cb, snb, row, ph, gg, st);
+        const cudaError_t e = i == 0 ? launch_window<T, true, true>(mp->win[i], psi, lam, cb, snb, row, (int)gg, ph, st)
+                                     : launch_window<T, true, false>(mp->win[i], psi, lam, cb, snb, row, (int)gg, ph, st);
         if (e != cudaSuccess) {
           delete mp;
           return QAOA_ERR_CUDA;

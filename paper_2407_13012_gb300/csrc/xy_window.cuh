@@ -56,7 +56,7 @@ struct Class {
   u64 ncols;       // binom(nh, h) * len
   u64 len;         // binom(lo, kL): ranks per row run of one H
   int h, kw, kL;   // popcounts above, inside and below the window
-  int rows, m;     // binom(w, kw); columns per tile
+  int rows, m, mb; // binom(w, kw); columns per tile, a power of two: m = 2^mb
 };
 
 struct Window {
@@ -200,10 +200,12 @@ inline void plan_window(Window& W, int n, int k, int lo, int w, int target, cons
       C.rows = (int)B[w][kw];
       C.len = B[lo][kL];
       C.ncols = B[W.nh][h] * C.len;
-      u64 m = (u64)(target / C.rows);
-      if (m < 1) m = 1;
-      if (m > (u64)kMaxCols) m = kMaxCols;
-      if (m > C.ncols) m = C.ncols;
+      u64 m = 1;  // the most columns of a power of two in the target, no more than the class needs
+      C.mb = 0;
+      while (2 * m * (u64)C.rows <= (u64)target && 2 * m <= (u64)kMaxCols && m < C.ncols) {
+        m *= 2;
+        ++C.mb;
+      }
       C.m = (int)m;
       C.first_tile = W.tiles;
       W.tiles += (C.ncols + m - 1) / m;

@@ -29,8 +29,8 @@ int main() {
     if (it % 97 == 0) ur = 0, ui = -(1ll << 62);
     if (it % 89 == 0) ur = 1ll << 62, ui = 0;
     const Factor f = factor(ur, ui);
-    const int b1 = 1 + (int)(rng() % 59);
-    const long long x = below(b1), y = it % 53 ? below(b1) : (1ll << 59) - 1;
+    const int b1 = 1 + (int)(rng() % 60);
+    const long long x = below(b1), y = it % 53 ? below(b1) : 1ll << 60;
     const C64 a = cmul_unit<false>(x, y, f), c = cmul_unit<true>(x, y, f);
     const C64 wa = cmul_q62_exact(x, y, ur, ui, 0), wc = cmul_q62_exact(x, y, ur, -ui, 0);
     if (far(a.x, wa.x, 1) || far(a.y, wa.y, 1) || far(c.x, wc.x, 1) || far(c.y, wc.y, 1)) bad("cmul_unit", it);
