@@ -509,13 +509,15 @@ __device__ __forceinline__ long long xy_fx_in(long long raw, int ep) {
   const long long s = raw >> 63;
   return (r ^ s) - s;
 }
-// Out: float64 nearest to x 2^-fs (halves away from zero); x != 0 lies in float64's normal range.
+// Out: float64 nearest to x 2^-fs, ties to even (a component keeps up to 56 bits here, so one in
+// eight of the large ones is a tie); x != 0 lies in float64's normal range.
 __device__ __forceinline__ double xy_fx_out(long long x, int fs) {
   const long long s = x >> 63;
   const unsigned long long a = (unsigned long long)((x ^ s) - s);
   const int lz = __clzll((long long)a);
   const unsigned long long m = a << (lz & 63);  // leading one at bit 63
-  const unsigned long long keep = (m >> 11) + ((m >> 10) & 1ull);  // 53 bits; a carry moves to the exponent
+  const unsigned up = ((unsigned)m & 0x7FFu) + (((unsigned)m >> 11) & 1u) > 0x400u;
+  const unsigned long long keep = (m >> 11) + up;  // 53 bits; a carry moves to the exponent
   // biased exponent of the leading one, less the one that keep's top bit adds
   const unsigned long long b = ((unsigned long long)(unsigned)(63 - lz - fs + 1022) << 52) + keep;
   return a == 0 ? 0.0 : __longlong_as_double((long long)(b | ((unsigned long long)s << 63)));
