@@ -160,7 +160,7 @@ static int cuda_status(cudaError_t e) { return e == cudaSuccess ? QAOA_OK : QAOA
 // before, the n = 24, p = 10 gradient with U(0, 1) weights took 27.8 instead of 24.1 ms.
 static int lean_kind(const Sweep& s, const Group& g, int tile_bits, int dtype) {
   const bool fx = dtype == QAOA_C128;
-  const int rb = fx ? (s.two ? 3 : 4) : (s.two ? 4 : 5);
+  const int rb = fx ? (tile_bits < 12 ? 2 : s.two ? 3 : 4) : (s.two ? 4 : 5);
   if (g.t + g.c != tile_bits || g.c > tile_bits - rb || g.t < 3) return SWEEP_GENERIC;
   if (fx && s.load_user) return SWEEP_GENERIC;
   if ((int)s.red_slot.size() > kLeanAcc) return SWEEP_GENERIC;
@@ -659,7 +659,7 @@ int qaoa_apply_layers(int n, int dtype, void* psi_dev, const qaoa_cost_t* cost, 
   size_t need = 0;
   qaoa_workspace_size(n, dtype, QAOA_OP_LAYERS, p, 0, span, &need);
   if (need > 0 && (ws_dev == nullptr || ws_bytes < need)) return QAOA_ERR_WORKSPACE;
-  const int B = sweep_tile_bits(dtype, false);
+  const int B = sweep_tile_bits(dtype, n);
   const std::vector<Group> gs = plan_groups(n, B);
   std::vector<Sweep> sw;
   plan_forward((int)gs.size(), p, init != 0, sw);
@@ -785,7 +785,7 @@ static int gradient_impl(int n, int dtype, void* psi_dev, void* lambda_dev, cons
   size_t need = 0;
   qaoa_workspace_size(n, dtype, QAOA_OP_GRADIENT, p, 0, span, &need);
   if (ws_dev == nullptr || ws_bytes < need) return QAOA_ERR_WORKSPACE;
-  const int B = sweep_tile_bits(dtype, true);
+  const int B = sweep_tile_bits(dtype, n);
   const std::vector<Group> gs = plan_groups(n, B);
   const int k = (int)gs.size();
   std::vector<Sweep> sw;
@@ -1027,7 +1027,7 @@ struct GroupPlan {
 
 static bool group_plan(int n, int dtype, int p, GroupPlan& G) {
   if (n < kGroupMinN) return false;
-  G.B = sweep_tile_bits(dtype, true);
+  G.B = sweep_tile_bits(dtype, QAOA_MAX_N);
   G.gs = plan_groups(n, G.B);
   G.sw.clear();
   G.nout = 2 * p + 2;

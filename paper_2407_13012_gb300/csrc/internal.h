@@ -143,6 +143,8 @@ struct TableArgs {
 void lean_x1(const SweepArgs& a, size_t sm, cudaStream_t s);         // complex128, one buffer
 void lean_x2_mix(const SweepArgs& a, size_t sm, cudaStream_t s);     // complex128, two buffers: one mixer
 void lean_x2_ops(const SweepArgs& a, size_t sm, cudaStream_t s);     // complex128, two buffers: op programs
+void lean_xt1(const SweepArgs& a, size_t sm, cudaStream_t s);        // complex128, small tiles, one buffer
+void lean_xt2(const SweepArgs& a, size_t sm, cudaStream_t s);        // complex128, small tiles, two buffers
 void lean_f1(const SweepArgs& a, size_t sm, cudaStream_t s);         // complex64, one buffer
 void lean_f2(const SweepArgs& a, size_t sm, cudaStream_t s);         // complex64, two buffers
 
@@ -166,7 +168,7 @@ cudaError_t launch_lbfgs_resume(double* ang, const double* st, int p, cudaStream
 cudaError_t launch_lbfgs_finish(double* ang, const double* st, int p, double* info, cudaStream_t s);
 cudaError_t launch_expect(int dtype, const void* psi, const void* C, int cost_dtype, int n, double* partials,
                           int grid, cudaStream_t s);
-int sweep_tile_bits(int dtype, bool two);     // B of the kernel a sweep uses
+int sweep_tile_bits(int dtype, int n);        // B of the kernels a one-graph sweep of n qubits uses
 // persistent grid size for a sweep (cost_bytes: 0, 4 or 8 bytes of cost tile per amplitude)
 int sweep_grid(int dtype, bool two, int tile_bits, int cost_bytes, int64_t tiles);
 int fx_shift_for(int tmax);                   // fixed-point scale for groups of <= tmax qubits

@@ -225,7 +225,8 @@ int blocks_per_sm(int cost_bytes) {
 // the lean kernels of this configuration (translation units lean_*.cu)
 template <class CF, bool FX, bool TWO>
 void lean_launch_cfg(const SweepArgs& a, size_t sm, cudaStream_t s) {
-  if constexpr (FX && !TWO) lean_x1(a, sm, s);
+  if constexpr (CF::B == CfgXT::B) TWO ? lean_xt2(a, sm, s) : lean_xt1(a, sm, s);
+  else if constexpr (FX && !TWO) lean_x1(a, sm, s);
   else if constexpr (FX) a.kind == SWEEP_LEAN_OPS ? lean_x2_ops(a, sm, s) : lean_x2_mix(a, sm, s);
   else if constexpr (!TWO) lean_f1(a, sm, s);
   else lean_f2(a, sm, s);
@@ -309,8 +310,15 @@ __global__ void expect_kernel(const void* __restrict__ psi, const void* __restri
 
 }  // namespace
 
-int sweep_tile_bits(int dtype, bool /*two*/) {
-  return dtype == QAOA_C128 ? 12 : 13;
+// complex128 sweeps of up to kSmallTileN qubits run on 512-amplitude tiles (two groups, so the
+// same number of sweeps as on 4096-amplitude tiles): they fill the chip better while the large
+// tiles of such a state are fewer than its SMs.  Measured, 4096- -> 512-amplitude tiles: n = 14, p = 4,
+// 50 Adam steps 12.4 -> 5.5 ms; n = 16 and 18, p = 6 gradients 353 -> 175 and 366 -> 266 us; n = 17,
+// p = 6 layers 151 -> 88 us.
+constexpr int kSmallTileN = 18;
+
+int sweep_tile_bits(int dtype, int n) {
+  return dtype == QAOA_C128 ? (n <= kSmallTileN ? CfgXT::B : CfgX1::B) : CfgF1::B;
 }
 
 // values stay below 2^61 through a group's Walsh-Hadamard transform (growth 2^(t/2)) for
@@ -319,7 +327,9 @@ int fx_shift_for(int tmax) { return 62 - (tmax + 1) / 2 - 2; }
 
 int sweep_grid(int dtype, bool two, int tile_bits, int cost_bytes, int64_t tiles) {
   int per_sm;
-  if (dtype == QAOA_C128) {
+  if (dtype == QAOA_C128 && tile_bits == CfgXT::B) {
+    per_sm = two ? blocks_per_sm<CfgXT, true, true>(cost_bytes) : blocks_per_sm<CfgXT, true, false>(cost_bytes);
+  } else if (dtype == QAOA_C128) {
     per_sm = two ? blocks_per_sm<CfgX2, true, true>(cost_bytes) : blocks_per_sm<CfgX1, true, false>(cost_bytes);
   } else if (two) {
     per_sm = blocks_per_sm<CfgF3, false, true>(cost_bytes);
@@ -332,7 +342,10 @@ int sweep_grid(int dtype, bool two, int tile_bits, int cost_bytes, int64_t tiles
 
 cudaError_t launch_sweep(int dtype, bool two, const SweepArgs& a, cudaStream_t s) {
   note_launch(0, s, true);
-  if (dtype == QAOA_C128) {
+  if (dtype == QAOA_C128 && a.tile_bits == CfgXT::B) {
+    if (two) launch_t<CfgXT, true, true>(a, s);
+    else launch_t<CfgXT, true, false>(a, s);
+  } else if (dtype == QAOA_C128) {
     if (two) launch_t<CfgX2, true, true>(a, s);
     else launch_t<CfgX1, true, false>(a, s);
   } else {

@@ -67,6 +67,12 @@ using CfgX1 = Cfg<12, 4, 4, 3, 2>;
 // complex128 fixed point two buffers: 4096-amplitude tiles, 8 per thread per buffer, 512 threads
 using CfgX2 = Cfg<12, 3, 3, 3, 1>;
 
+// complex128 at small n, one or two buffers: 512-amplitude tiles, 4 per thread per buffer.  At
+// n = 14 a sweep of 4096-amplitude tiles keeps 4 of 152 SMs busy for a whole tile's latency
+// (~25 us, whatever the rest of the chip does); 512-amplitude tiles spread it over 32 SMs with an
+// eighth of the work per SM quarter.
+using CfgXT = Cfg<9, 2, 2, 3, 4>;
+
 // cost-tile slot of local index i; the XOR leaves the bits inside a 16-byte chunk alone so
 // the tile can be fetched with 16-byte asynchronous copies
 __device__ __forceinline__ uint32_t phys_cost(uint32_t i, bool f64) {
@@ -182,6 +188,7 @@ struct Sweeper {
   using V = typename std::conditional<FX, longlong2, float2>::type;
   static constexpr int R = CF::R;
 
+  static_assert(CF::NR <= 5, "exchanges between run-time layouts: five at most");
   const SweepArgs& a;
   V v[R];        // register tile of psi (layout cur)
   V w[R];        // register tile of lambda (two-buffer sweeps)
@@ -266,7 +273,8 @@ struct Sweeper {
       case 0: ex<F, 0>(u); break;
       case 1: if constexpr (CF::NR > 1) ex<F, (CF::NR > 1 ? 1 : 0)>(u); break;
       case 2: if constexpr (CF::NR > 2) ex<F, (CF::NR > 2 ? 2 : 0)>(u); break;
-      default: if constexpr (CF::NR > 3) ex<F, (CF::NR > 3 ? 3 : 0)>(u); break;
+      case 3: if constexpr (CF::NR > 3) ex<F, (CF::NR > 3 ? 3 : 0)>(u); break;
+      default: if constexpr (CF::NR > 4) ex<F, (CF::NR > 4 ? 4 : 0)>(u); break;
     }
   }
   __device__ __forceinline__ void exchange_one(V (&u)[R], int to) {
@@ -274,7 +282,8 @@ struct Sweeper {
       case 0: ex_from<0>(u, to); break;
       case 1: if constexpr (CF::NR > 1) ex_from<(CF::NR > 1 ? 1 : 0)>(u, to); break;
       case 2: if constexpr (CF::NR > 2) ex_from<(CF::NR > 2 ? 2 : 0)>(u, to); break;
-      default: if constexpr (CF::NR > 3) ex_from<(CF::NR > 3 ? 3 : 0)>(u, to); break;
+      case 3: if constexpr (CF::NR > 3) ex_from<(CF::NR > 3 ? 3 : 0)>(u, to); break;
+      default: if constexpr (CF::NR > 4) ex_from<(CF::NR > 4 ? 4 : 0)>(u, to); break;
     }
   }
   // both buffers at once: psi through X, lambda through the second half X + 2^B, so one
@@ -299,7 +308,8 @@ struct Sweeper {
       case 0: ex2<F, 0>(); break;
       case 1: if constexpr (CF::NR > 1) ex2<F, (CF::NR > 1 ? 1 : 0)>(); break;
       case 2: if constexpr (CF::NR > 2) ex2<F, (CF::NR > 2 ? 2 : 0)>(); break;
-      default: if constexpr (CF::NR > 3) ex2<F, (CF::NR > 3 ? 3 : 0)>(); break;
+      case 3: if constexpr (CF::NR > 3) ex2<F, (CF::NR > 3 ? 3 : 0)>(); break;
+      default: if constexpr (CF::NR > 4) ex2<F, (CF::NR > 4 ? 4 : 0)>(); break;
     }
   }
   __device__ __forceinline__ void exchange_both(int to) {
@@ -307,7 +317,8 @@ struct Sweeper {
       case 0: ex2_from<0>(to); break;
       case 1: if constexpr (CF::NR > 1) ex2_from<(CF::NR > 1 ? 1 : 0)>(to); break;
       case 2: if constexpr (CF::NR > 2) ex2_from<(CF::NR > 2 ? 2 : 0)>(to); break;
-      default: if constexpr (CF::NR > 3) ex2_from<(CF::NR > 3 ? 3 : 0)>(to); break;
+      case 3: if constexpr (CF::NR > 3) ex2_from<(CF::NR > 3 ? 3 : 0)>(to); break;
+      default: if constexpr (CF::NR > 4) ex2_from<(CF::NR > 4 ? 4 : 0)>(to); break;
     }
   }
   // both buffers always share one layout; two-buffer kernels own an exchange area of 2 x 2^B
