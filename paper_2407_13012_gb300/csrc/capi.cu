@@ -147,6 +147,7 @@ struct Ctx {
   cudaStream_t s;
   char* ws;
   size_t ws_bytes;
+  bool bound_ready = false;  // the workspace already holds max |C| (a later step of an optimiser loop)
 };
 
 static int cuda_status(cudaError_t e) { return e == cudaSuccess ? QAOA_OK : QAOA_ERR_CUDA; }
@@ -236,7 +237,7 @@ static int run_sweeps(const Ctx& c, std::vector<Sweep>& sw, const std::vector<Gr
   p_ws += fx_table_bytes(c.dtype, p);
   if ((size_t)(p_ws - c.ws) > c.ws_bytes) return QAOA_ERR_WORKSPACE;
 
-  if (p > 0 && (span > 0 || fx)) {
+  if (p > 0 && (span > 0 || fx || ang_dev != nullptr)) {
     TableArgs t;
     std::memset(&t, 0, sizeof(t));
     t.fx = fx;
@@ -245,6 +246,7 @@ static int run_sweeps(const Ctx& c, std::vector<Sweep>& sw, const std::vector<Gr
     t.span = span;
     if (ang_dev != nullptr) {
       t.dev_angles = ang_dev;
+      t.trig = trig;
     } else {
       for (int l = 0; l < p; ++l) {
         t.gamma[l] = gamma[l];
@@ -270,13 +272,8 @@ static int run_sweeps(const Ctx& c, std::vector<Sweep>& sw, const std::vector<Gr
     rc = cuda_status(launch_reduce(r, norm_part, norm2, c.s));
     if (rc) return rc;
   }
-  if (fx && any_two) {  // lambda scale from max |C|
+  if (fx && any_two && !c.bound_ready) {  // lambda scale from max |C|
     int rc = cuda_status(launch_cost_bound(c.cost->C_dev, c.cost->dtype == QAOA_COST_F64, c.n, cmax_bits, c.s));
-    if (rc) return rc;
-  }
-
-  if (ang_dev != nullptr && p > 0) {
-    int rc = cuda_status(launch_angle_prep(ang_dev, p, trig, c.s));
     if (rc) return rc;
   }
   const double amp0 = std::pow(2.0, -0.5 * c.n);
@@ -775,7 +772,7 @@ int qaoa_sample_host(int n, int dtype, const void* psi_dev, const qaoa_cost_t* c
 // (ang_dev = [gamma p | beta p]).
 static int gradient_impl(int n, int dtype, void* psi_dev, void* lambda_dev, const qaoa_cost_t* cost,
                          const double* gamma, const double* beta, const double* ang_dev, int p, double* out_dev,
-                         void* ws_dev, size_t ws_bytes, void* stream) {
+                         void* ws_dev, size_t ws_bytes, void* stream, bool bound_ready = false) {
   if (n < 1 || n > QAOA_MAX_N || !valid_dtype(dtype) || psi_dev == nullptr || lambda_dev == nullptr ||
       out_dev == nullptr || !valid_cost(cost) || p < 1 || p > QAOA_MAX_P)
     return QAOA_ERR_INVALID_ARG;
@@ -805,7 +802,7 @@ static int gradient_impl(int n, int dtype, void* psi_dev, void* lambda_dev, cons
     if (ncontrib[o] > kMaxContrib) return QAOA_ERR_UNSUPPORTED;
   for (const Sweep& s : sw)
     if ((int)s.red_slot.size() > 255) return QAOA_ERR_UNSUPPORTED;
-  Ctx c{n, dtype, cost, (cudaStream_t)stream, (char*)ws_dev, ws_bytes};
+  Ctx c{n, dtype, cost, (cudaStream_t)stream, (char*)ws_dev, ws_bytes, bound_ready};
   return run_sweeps(c, sw, gs, B, psi_dev, lambda_dev, gamma, beta, ang_dev, p, nout, ncontrib, out_dev);
 }
 
@@ -860,9 +857,12 @@ int qaoa_optimize_adam(int n, int dtype, void* psi_dev, void* lambda_dev, const 
   } else if (cudaMemsetAsync(state, 0, (4 * p + 1) * sizeof(double), s) != cudaSuccess) {
     return QAOA_ERR_CUDA;
   }
+  bool first = true;
   return replay_steps(s, steps, [&](cudaStream_t cur) {
+    // the first step leaves max |C| in the workspace for the captured ones
     int r = gradient_impl(n, dtype, psi_dev, lambda_dev, cost, nullptr, nullptr, angles_dev, p, gout, ws_dev, gbytes,
-                          (void*)cur);
+                          (void*)cur, !first);
+    first = false;
     if (r) return r;
     return cuda_status(
         launch_adam(angles_dev, gout, state, counter, p, lr, beta1, beta2, eps, history_dev, row0, steps, cur));
@@ -900,9 +900,12 @@ int qaoa_optimize_lbfgs(int n, int dtype, void* psi_dev, void* lambda_dev, const
   } else if (cudaMemsetAsync(state, 0, nstate * sizeof(double), s) != cudaSuccess) {
     return QAOA_ERR_CUDA;
   }
+  bool first = true;
   rc = replay_steps(s, max_evals, [&](cudaStream_t cur) {
+    // the first step leaves max |C| in the workspace for the captured ones
     int r = gradient_impl(n, dtype, psi_dev, lambda_dev, cost, nullptr, nullptr, angles_dev, p, gout, ws_dev, gbytes,
-                          (void*)cur);
+                          (void*)cur, !first);
+    first = false;
     if (r) return r;
     return cuda_status(launch_lbfgs(angles_dev, gout, state, p, m, gtol, 1e-4, history_dev, row0, max_evals, cur));
   }, state + 7, 16);

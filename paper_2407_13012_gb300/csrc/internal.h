@@ -137,6 +137,7 @@ struct TableArgs {
   void* phase;   // p * span entries
   void* dtab;    // fixed point: p * 14 * 14 entries
   void* turn;    // fixed point: kTurnEntries entries
+  double* trig;  // with dev_angles: [g2pi p | cos p | sin p], or nullptr
 };
 
 // lean sweeps (lean_*.cu) of the sweep's shape, with sm bytes of dynamic shared memory
@@ -158,7 +159,6 @@ cudaError_t launch_group_reduce(const ReducePlan& r, int ngraphs, int bpg, const
 cudaError_t launch_tables(const TableArgs& t, cudaStream_t s);
 cudaError_t launch_cost_bound(const void* C, int f64, int n, unsigned long long* out, cudaStream_t s);
 cudaError_t launch_norm(const void* psi, int dtype, int n, double* partials, int* nblocks, cudaStream_t s);
-cudaError_t launch_angle_prep(const double* ang, int p, double* trig, cudaStream_t s);
 cudaError_t launch_adam(double* ang, const double* g, double* state, long long* step, int p, double lr, double b1,
                         double b2, double eps, double* history, long long row0, long long max_rows, cudaStream_t s);
 size_t lbfgs_state_doubles(int p, int m);

@@ -91,9 +91,16 @@ __global__ void tables_kernel(const __grid_constant__ TableArgs ta) {
   const int64_t nphase = (int64_t)ta.p * ta.span;
   const int64_t nd = ta.fx ? (int64_t)ta.p * 14 * 14 : 0;
   const int64_t nt = ta.fx ? kTurnEntries : 0;
-  const int64_t total = nphase + nd + nt;
+  const int64_t total = nphase + nd + nt + (ta.trig != nullptr ? ta.p : 0);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    if (i < nphase) {
+    if (i >= nphase + nd + nt) {  // [g2pi p | cos(beta) p | sin(beta) p] from device angles [gamma p | beta p]
+      const int l = (int)(i - nphase - nd - nt);
+      ta.trig[l] = ta.dev_angles[l] / (2.0 * 3.141592653589793238);
+      double sn, cs;
+      sincos(ta.dev_angles[ta.p + l], &sn, &cs);
+      ta.trig[ta.p + l] = cs;
+      ta.trig[2 * ta.p + l] = sn;
+    } else if (i < nphase) {
       const int l = (int)(i / ta.span);
       const int64_t c = ta.cmin + (i - (int64_t)l * ta.span);
       const double th = (ta.dev_angles ? ta.dev_angles[l] : ta.gamma[l]) * (double)c;
@@ -106,18 +113,6 @@ __global__ void tables_kernel(const __grid_constant__ TableArgs ta) {
     } else {
       ((longlong2*)ta.turn)[i - nphase - nd] = turn_entry((int)(i - nphase - nd));
     }
-  }
-}
-
-// [g2pi p | cos(beta) p | sin(beta) p] from device angles [gamma p | beta p]
-__global__ void angle_prep_kernel(const double* __restrict__ ang, int p, double* __restrict__ trig) {
-  const int l = threadIdx.x;
-  if (l < p) {
-    trig[l] = ang[l] / (2.0 * 3.141592653589793238);
-    double sn, cs;
-    sincos(ang[p + l], &sn, &cs);
-    trig[p + l] = cs;
-    trig[2 * p + l] = sn;
   }
 }
 
@@ -387,11 +382,15 @@ cudaError_t launch_group_reduce(const ReducePlan& r, int ngraphs, int bpg, const
 }
 
 cudaError_t launch_tables(const TableArgs& t, cudaStream_t s) {
-  const int64_t total = (int64_t)t.p * t.span + (t.fx ? (int64_t)t.p * 196 + kTurnEntries : 0);
+  const int64_t total =
+      (int64_t)t.p * t.span + (t.fx ? (int64_t)t.p * 196 + kTurnEntries : 0) + (t.trig != nullptr ? t.p : 0);
   if (total <= 0) return cudaSuccess;
-  const int blocks = (int)((total + 255) / 256 < 1024 ? (total + 255) / 256 : 1024);
+  // an entry is a float64 sincos, ~100 operations of which an SM quarter retires one per 64 cycles
+  // and warp: one warp per block spreads them over the chip (with the angle terms in the same launch
+  // and max |C| read once per run, 50 Adam steps at n = 14, p = 4 went from 5.5 to 5.05 ms)
+  const int64_t blocks = std::min<int64_t>((total + 31) / 32, 4096);
   note_launch(3, s, true);
-  tables_kernel<<<blocks, 256, 0, s>>>(t);
+  tables_kernel<<<(int)blocks, 32, 0, s>>>(t);
   note_launch(3, s, false);
   return cudaGetLastError();
 }
@@ -404,13 +403,6 @@ cudaError_t launch_cost_bound(const void* C, int f64, int n, unsigned long long*
   if (blocks > (int64_t)num_sms() * 8) blocks = (int64_t)num_sms() * 8;
   cost_bound_kernel<<<(int)blocks, 256, 0, s>>>(C, f64, count, out);
   note_launch(3, s, false, (double)(1ull << n) * (f64 ? 8.0 : 4.0));
-  return cudaGetLastError();
-}
-
-cudaError_t launch_angle_prep(const double* ang, int p, double* trig, cudaStream_t s) {
-  note_launch(3, s, true);
-  angle_prep_kernel<<<1, 64, 0, s>>>(ang, p, trig);
-  note_launch(3, s, false);
   return cudaGetLastError();
 }
 

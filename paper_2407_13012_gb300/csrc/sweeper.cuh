@@ -163,7 +163,7 @@ __device__ __forceinline__ longlong2 turn_phase(unsigned long long t, const long
 // ------------------------------------------------------------------ kernel
 
 // per-layer angle terms: kernel parameters, or device memory ([g2pi p | cos p | sin p],
-// written by angle_prep_kernel) when the angles live on the device
+// written by tables_kernel) when the angles live on the device
 __device__ __forceinline__ double arg_g2pi(const SweepArgs& a, const double* trig, int l) {
   return trig ? trig[l] : a.g2pi[l];
 }
