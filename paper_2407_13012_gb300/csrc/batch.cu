@@ -26,6 +26,89 @@ constexpr int kMaxBatchEdges = 512;
 static_assert(QAOA_BATCH_MAX_EDGES <= kMaxBatchEdges, "edge staging holds every edge of a graph");
 static_assert(QAOA_BATCH_MAX_N < 32, "cost-vector indices in 32 bits");
 
+// The costs of one block's 2^12 entries z = (h, y, x), y and x six bits each, h fixed:
+//   C(z) = Q0[x] + T1[y] + sum_{u < 6} x_u a_u[y],
+// Q0 the edges inside x, T1 those inside y, between y and h and inside h, and
+// a_u[y] = sum_{v >= 6} w_uv (1 - 2 z_v), which together with the cut edges' constant w z_v (part of
+// T1) gives the edges leaving x.  The tables take a few operations per thread; an entry is then
+// three additions (summing every edge per entry took 9.8 of the 191 ms of the 4096-graph batch).
+// S: unsigned for integer weights (sums modulo 2^32 give the exact int32 cost), long long for
+// fixed-point ones.  4096-graph batch, complex128: 174.4 -> 167.0 ms.
+constexpr int kHalf = 6;
+template <class S, class OUT>
+__device__ __forceinline__ void batch_costs(int n, const int2* e_s, const S* w_s, int m, uint32_t z0, S* W, S* tab,
+                                            OUT&& put) {
+  constexpr int N = QAOA_BATCH_MAX_N, H = 1 << kHalf;
+  S* Q0 = tab;              // [64]
+  S* T1 = tab + H;          // [64]
+  S* A = tab + 2 * H;       // [6][64]
+  S* lin = tab + 8 * H;     // [12]: bits 0..5: sum over h of w (1 - 2 h_v); bits 6..11: the same
+  S* kh = lin + 2 * kHalf;  // edges inside h, and the constants h_v w of edges into h
+  const int tid = threadIdx.x;
+  for (int i = tid; i < N * N; i += kPrepThreads) W[i] = 0;
+  __syncthreads();
+  for (int k = tid; k < m; k += kPrepThreads) {
+    W[e_s[k].x * N + e_s[k].y] = w_s[k];
+    W[e_s[k].y * N + e_s[k].x] = w_s[k];
+  }
+  __syncthreads();
+  if (tid < 2 * kHalf) {
+    S s = 0;
+    for (int v = 2 * kHalf; v < n; ++v) s += (z0 >> v) & 1u ? -W[tid * N + v] : W[tid * N + v];
+    lin[tid] = s;
+  } else if (tid == 32) {
+    S s = 0;
+    for (int v = 2 * kHalf; v < n; ++v) {
+      if (!((z0 >> v) & 1u)) continue;
+      for (int u = 0; u < n; ++u)  // inside h: pairs with a clear bit; below h: the constant
+        if (u < 2 * kHalf || !((z0 >> u) & 1u)) s += W[v * N + u];
+    }
+    *kh = s;
+  }
+  __syncthreads();
+  for (int i = tid; i < 8 * H; i += kPrepThreads) {
+    const int y = i % H, row = i / H;
+    S s = 0;
+    if (row == 0) {
+      for (int u = 0; u < kHalf; ++u)
+        for (int v = u + 1; v < kHalf; ++v)
+          if (((y >> u) ^ (y >> v)) & 1) s += W[u * N + v];
+    } else if (row == 1) {
+      s = *kh;
+      for (int u = 0; u < kHalf; ++u) {
+        if (!((y >> u) & 1)) continue;
+        s += lin[kHalf + u];
+        for (int v = 0; v < kHalf; ++v)  // inside y: pairs with a clear bit; below y: the constant
+          s += W[(kHalf + u) * N + v] + ((y >> v) & 1 ? 0 : W[(kHalf + u) * N + kHalf + v]);
+      }
+    } else {
+      const int u = row - 2;
+      s = lin[u];
+      for (int v = 0; v < kHalf; ++v) s += (y >> v) & 1 ? -W[u * N + kHalf + v] : W[u * N + kHalf + v];
+    }
+    tab[i] = s;
+  }
+  __syncthreads();
+  // thread: one y, 16 consecutive x
+  const int y = tid >> 2, x0 = (tid & 3) * 16;
+  S base = T1[y];
+  if (x0 & 16) base += A[4 * H + y];
+  if (x0 & 32) base += A[5 * H + y];
+  const uint32_t z = z0 + (uint32_t)(y << kHalf) + (uint32_t)x0;
+  if (z >= (1u << n)) return;
+  S s[16];
+  s[0] = base;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const S au = A[u * H + y];
+#pragma unroll
+    for (int i = 0; i < (1 << u); ++i) s[i + (1 << u)] = s[i] + au;
+  }
+#pragma unroll
+  for (int i = 0; i < 16; ++i) s[i] += Q0[x0 + i];
+  put(z, s);
+}
+
 // One launch prepares every graph: blocks [0, cost_blocks) build the cost vectors (2^12
 // entries per block, C(z) = sum over edges of w [z_u != z_v], Sec. III-B's MaxCut cost, int32
 // for integer weights; float weights are quantised once to a common fixed point,
@@ -35,8 +118,9 @@ static_assert(QAOA_BATCH_MAX_N < 32, "cost-vector indices in 32 bits");
 __global__ void __launch_bounds__(kPrepThreads) batch_prep_kernel(const __grid_constant__ BatchArgs b,
                                                                    int64_t cost_blocks) {
   __shared__ int2 e_s[kMaxBatchEdges];
-  __shared__ int wi_s[kMaxBatchEdges];        // integer weights
-  __shared__ long long wq_s[kMaxBatchEdges];  // float weights in fixed point
+  __shared__ long long w_s[kMaxBatchEdges];  // integer weights (int) or float weights in fixed point
+  __shared__ long long W_s[QAOA_BATCH_MAX_N * QAOA_BATCH_MAX_N];
+  __shared__ long long tab_s[8 * (1 << kHalf) + 2 * kHalf + 1];
   __shared__ int shift_s;
   const int64_t blk = blockIdx.x;
   const int tid = threadIdx.x;
@@ -65,26 +149,31 @@ __global__ void __launch_bounds__(kPrepThreads) batch_prep_kernel(const __grid_c
     for (int k = tid; k < G.m; k += kPrepThreads) {
       e_s[k] = make_int2(b.edges[2 * (G.edge + k)], b.edges[2 * (G.edge + k) + 1]);
       const double w = b.ew[G.edge + k];
-      if (b.cost_f64) wq_s[k] = llrint(ldexp(w, shift_s));
-      else wi_s[k] = (int)w;
+      if (b.cost_f64) w_s[k] = llrint(ldexp(w, shift_s));
+      else ((int*)w_s)[k] = (int)w;
     }
-    __syncthreads();
     // n <= QAOA_BATCH_MAX_N < 32: 32-bit indices
     const uint32_t z0 = (uint32_t)(blk - b.blk_off[lo]) << kBatchCostBits;
-    const uint32_t zend = min(z0 + (1u << kBatchCostBits), 1u << G.n);
+    const int live = min(16, 1 << G.n);  // entries of a thread's 16 inside the vector
     if (b.cost_f64) {
-      for (uint32_t z = z0 + tid; z < zend; z += kPrepThreads) {
-        long long c = 0;
-        for (int k = 0; k < G.m; ++k)
-          if (((z >> e_s[k].x) ^ (z >> e_s[k].y)) & 1u) c += wq_s[k];
-        ((double*)b.C)[G.cost + (int64_t)z] = ldexp((double)c, -shift_s);
-      }
+      double* out = (double*)b.C + G.cost;
+      batch_costs<long long>(G.n, e_s, w_s, G.m, z0, W_s, tab_s, [&](uint32_t z, const long long(&s)[16]) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+          if (i < live) out[z + i] = fx::to_double(s[i], shift_s);
+      });
     } else {
-      for (uint32_t z = z0 + tid; z < zend; z += kPrepThreads) {
-        int c = 0;
-        for (int k = 0; k < G.m; ++k) c += (int)(((z >> e_s[k].x) ^ (z >> e_s[k].y)) & 1u) * wi_s[k];
-        ((int*)b.C)[G.cost + (int64_t)z] = c;
-      }
+      int* out = (int*)b.C + G.cost;
+      batch_costs<unsigned>(G.n, e_s, (const unsigned*)w_s, G.m, z0, (unsigned*)W_s, (unsigned*)tab_s,
+                            [&](uint32_t z, const unsigned(&s)[16]) {
+        if (live == 16) {  // graphs start 64-element aligned
+#pragma unroll
+          for (int i = 0; i < 16; i += 4) *(int4*)(out + z + i) =
+            make_int4((int)s[i], (int)s[i + 1], (int)s[i + 2], (int)s[i + 3]);
+        } else {
+          for (int i = 0; i < live; ++i) out[z + i] = (int)s[i];
+        }
+      });
     }
     return;
   }
