@@ -21,19 +21,19 @@ __device__ __forceinline__ void lean_tiles(Lean<CF, FX, TWO>& s, const SweepArgs
   const int64_t tiles = a.g.tiles;
   switch (last) {
     case 0:
-      for (int64_t t = 0; t < tiles; ++t) lean_tile<CF, FX, TWO, true, 0, true>(s, a, t, Cs);
+      for (int64_t t = 0; t < tiles; ++t) lean_tile<CF, FX, TWO, true, 0, true>(s, a, a.g, t, Cs);
       break;
     case 1:
       if constexpr (CF::NR > 1)
-        for (int64_t t = 0; t < tiles; ++t) lean_tile<CF, FX, TWO, true, (CF::NR > 1 ? 1 : 0), true>(s, a, t, Cs);
+        for (int64_t t = 0; t < tiles; ++t) lean_tile<CF, FX, TWO, true, (CF::NR > 1 ? 1 : 0), true>(s, a, a.g, t, Cs);
       break;
     case 2:
       if constexpr (CF::NR > 2)
-        for (int64_t t = 0; t < tiles; ++t) lean_tile<CF, FX, TWO, true, (CF::NR > 2 ? 2 : 0), true>(s, a, t, Cs);
+        for (int64_t t = 0; t < tiles; ++t) lean_tile<CF, FX, TWO, true, (CF::NR > 2 ? 2 : 0), true>(s, a, a.g, t, Cs);
       break;
     default:
       if constexpr (CF::NR > 3)
-        for (int64_t t = 0; t < tiles; ++t) lean_tile<CF, FX, TWO, true, (CF::NR > 3 ? 3 : 0), true>(s, a, t, Cs);
+        for (int64_t t = 0; t < tiles; ++t) lean_tile<CF, FX, TWO, true, (CF::NR > 3 ? 3 : 0), true>(s, a, a.g, t, Cs);
       break;
   }
 }
@@ -92,7 +92,8 @@ __global__ void __launch_bounds__(CF::NT, CF::MINB) batch_kernel(const __grid_co
         sa.init_f32 = P.init_f32;
         sa.fx_shift = P.fx_shift;
         sa.norm2_dev = nullptr;
-        sa.cmax_dev = nullptr;
+        sa.scan = nullptr;
+        sa.mirror = 0;
         sa.nops = bs.nops;
         sa.dev_trig = b.trig + gidx * 3 * p;
         sa.np = p;

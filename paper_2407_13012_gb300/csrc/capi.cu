@@ -113,7 +113,7 @@ struct Sweep {
 
 static int64_t tiles_of(const Group& g, int n) { return 1ll << (n - g.t - g.c); }
 
-constexpr size_t kScalarBytes = 256;                     // norm^2 (double), max|C| bits (u64)
+constexpr size_t kScalarBytes = 256;                     // norm^2 (double)
 constexpr size_t kNormPartialBytes = 1024 * sizeof(double);
 constexpr size_t kTrigBytes = 3 * QAOA_MAX_P * sizeof(double);  // per-layer terms of device angles
 
@@ -147,7 +147,8 @@ struct Ctx {
   cudaStream_t s;
   char* ws;
   size_t ws_bytes;
-  bool bound_ready = false;  // the workspace already holds max |C| (a later step of an optimiser loop)
+  // the workspace already holds the scan of C (a later step of an optimiser loop)
+  bool bound_ready = false;
 };
 
 static int cuda_status(cudaError_t e) { return e == cudaSuccess ? QAOA_OK : QAOA_ERR_CUDA; }
@@ -185,6 +186,14 @@ static int lean_kind(const Sweep& s, const Group& g, int tile_bits, int dtype) {
   return SWEEP_LEAN_OPS;
 }
 
+// The one-graph calls that check C for symmetry and sweep half the state (SweepArgs::half) if they may.
+// From these sizes on halving the tiles shortens a call by more than the read of C costs: whole -> half,
+// p = 6, complex128: n = 18 gradient 260 -> 230 us, n = 20 layers 182 -> 151, gradient 628 -> 389, n = 22
+// gradient 2143 -> 1271; complex64 n = 20 layers 96 -> 111 us, n = 21 134 -> 115, gradient 468 -> 324;
+// n = 30, p = 6 layers 194 -> 101 ms.  A C that is not symmetric pays for the read: n = 20, p = 6
+// complex128 layers 182 -> 188 us, n = 22 573 -> 587.
+static int half_min_n(int dtype, bool gradient) { return dtype == QAOA_C64 ? 21 : gradient ? 18 : 20; }
+
 // Run a list of sweeps with one shared grid, then reduce the partials into out[0..nout).
 // Fixed-point (complex128) calls also get: the input scale from the norm of a loaded
 // user state, the lambda scale from max |C| (gradient), and the mixer/turn tables.
@@ -213,7 +222,6 @@ static int run_sweeps(const Ctx& c, std::vector<Sweep>& sw, const std::vector<Gr
   // workspace carving
   char* p_ws = c.ws;
   double* norm2 = (double*)p_ws;
-  unsigned long long* cmax_bits = (unsigned long long*)(p_ws + 8);
   p_ws += kScalarBytes;
   double* norm_part = (double*)p_ws;
   p_ws += kNormPartialBytes;
@@ -237,9 +245,9 @@ static int run_sweeps(const Ctx& c, std::vector<Sweep>& sw, const std::vector<Gr
   p_ws += fx_table_bytes(c.dtype, p);
   if ((size_t)(p_ws - c.ws) > c.ws_bytes) return QAOA_ERR_WORKSPACE;
 
+  TableArgs t;
+  std::memset(&t, 0, sizeof(t));
   if (p > 0 && (span > 0 || fx || ang_dev != nullptr)) {
-    TableArgs t;
-    std::memset(&t, 0, sizeof(t));
     t.fx = fx;
     t.p = p;
     t.cmin = cmin;
@@ -256,7 +264,28 @@ static int run_sweeps(const Ctx& c, std::vector<Sweep>& sw, const std::vector<Gr
     t.phase = phase_table;
     t.dtab = d_table;
     t.turn = turn_table;
+  }
+  // whether C is symmetric (half states) and max |C| (the lambda scale): one read of C
+  bool half = c.n >= half_min_n(c.dtype, any_two) && c.n > tile_bits && p > 0 && !any_user_load;
+  for (const Sweep& s : sw) half &= lean_kind(s, gs[s.group], tile_bits, c.dtype) != SWEEP_GENERIC;
+  unsigned long long* scan = nullptr;
+  const int nscan = half || (fx && any_two) ? cost_scan_blocks(c.n) : 0;
+  const bool scan_now = nscan > 0 && !c.bound_ready;
+  // the tables ride on a scan of enough blocks: they are float64 work, which few SMs would serialise
+  const bool ride = scan_now && nscan >= 64;
+  if (nscan > 0) {
+    static_assert(kMaxScan * sizeof(unsigned long long) <= kNormPartialBytes, "the scan takes the norm partials' place");
+    if (any_user_load) return QAOA_ERR_UNSUPPORTED;  // (no plan has both)
+    scan = (unsigned long long*)norm_part;
+  }
+  if (t.p > 0 && !ride) {
     int rc = cuda_status(launch_tables(t, c.s));
+    if (rc) return rc;
+  }
+  if (scan_now) {
+    TableArgs none;
+    std::memset(&none, 0, sizeof(none));
+    int rc = cuda_status(launch_cost_scan(c.cost->C_dev, c.cost->dtype == QAOA_COST_F64, c.n, scan, ride ? t : none, c.s));
     if (rc) return rc;
   }
   if (fx && any_user_load) {  // input scale from |psi|^2 of the caller's state
@@ -272,10 +301,6 @@ static int run_sweeps(const Ctx& c, std::vector<Sweep>& sw, const std::vector<Gr
     rc = cuda_status(launch_reduce(r, norm_part, norm2, c.s));
     if (rc) return rc;
   }
-  if (fx && any_two && !c.bound_ready) {  // lambda scale from max |C|
-    int rc = cuda_status(launch_cost_bound(c.cost->C_dev, c.cost->dtype == QAOA_COST_F64, c.n, cmax_bits, c.s));
-    if (rc) return rc;
-  }
   const double amp0 = std::pow(2.0, -0.5 * c.n);
   const int S = fx_shift_for(tmax);
   for (const Sweep& s : sw) {
@@ -287,6 +312,10 @@ static int run_sweeps(const Ctx& c, std::vector<Sweep>& sw, const std::vector<Gr
     a.cost_dtype = c.cost->dtype;
     const Group& g = gs[s.group];
     a.g = {c.n, g.j0, g.t, g.c, tiles_of(g, c.n)};
+    a.half = half ? 2 : 0;
+    a.mirror = half && s.store_user;
+    a.scan = scan;
+    a.nscan = nscan;
     a.tile_bits = tile_bits;
     a.load_fmt = s.init ? 2 : (s.load_user ? 1 : 0);
     a.store_fmt = !s.store_psi ? -1 : (s.store_user ? 1 : 0);
@@ -296,7 +325,6 @@ static int run_sweeps(const Ctx& c, std::vector<Sweep>& sw, const std::vector<Gr
     a.init_fx = (long long)std::llrint(std::ldexp(amp0, S));
     a.init_f32 = (float)amp0;
     a.norm2_dev = (fx && any_user_load) ? norm2 : nullptr;
-    a.cmax_dev = (fx && any_two) ? cmax_bits : nullptr;
     if ((int)s.ops.size() > kMaxOps) return QAOA_ERR_UNSUPPORTED;
     a.nops = (int)s.ops.size();
     bool reads_c = false;
@@ -339,9 +367,10 @@ static int run_sweeps(const Ctx& c, std::vector<Sweep>& sw, const std::vector<Gr
       const double per = S_b * ((s.init ? 0 : 1) + (s.store_psi ? 1 : 0) + (s.two && s.load_lam ? 1 : 0) +
                                 (s.two && s.store_lam ? 1 : 0)) +
                          (reads_c ? cb : 0.0);
-      a.algo_bytes = per * (double)(1ull << c.n);
+      a.algo_bytes = per * (double)(1ull << (c.n - half));  // (only the device knows whether C is symmetric)
     }
     a.kind = lean_kind(s, g, tile_bits, c.dtype);
+    if (a.mirror) a.kind = SWEEP_LEAN_OPS;  // (the plain mixer kernels store no complements)
     int rc = cuda_status(launch_sweep(c.dtype, s.two, a, c.s));
     if (rc) return rc;
   }
@@ -354,7 +383,7 @@ static int run_sweeps(const Ctx& c, std::vector<Sweep>& sw, const std::vector<Gr
       r.ncontrib[o] = ncontrib[o];
       r.scale[o] = 1.0;
     }
-    int rc = cuda_status(launch_reduce(r, partials, out, c.s));
+    int rc = cuda_status(launch_reduce(r, partials, out, c.s, half ? scan : nullptr, nscan));
     if (rc) return rc;
   }
   return QAOA_OK;
@@ -1203,6 +1232,7 @@ static int run_group(int dtype, int p, const BatchLayout& L, const BatchArgs& b,
     a.cost_dtype = L.cost_f64 ? QAOA_COST_F64 : QAOA_COST_I32;
     const Group& g = G.gs[s.group];
     a.g = {n, g.j0, g.t, g.c, tiles_of(g, n)};
+    a.half = 1;  // every graph's cost is a cut: symmetric
     a.tile_bits = G.B;
     a.load_fmt = s.init ? 2 : 0;
     a.store_fmt = s.store_psi ? 0 : -1;
@@ -1243,7 +1273,7 @@ static int run_group(int dtype, int p, const BatchLayout& L, const BatchArgs& b,
     const double per = (double)vs * ((s.init ? 0 : 1) + (s.store_psi ? 1 : 0) + (s.two && s.load_lam ? 1 : 0) +
                                      (s.two && s.store_lam ? 1 : 0)) +
                        (reads_c ? cb : 0.0);
-    a.algo_bytes = per * (double)(1ull << n) * ng;
+    a.algo_bytes = per * (double)(1ull << (n - 1)) * ng;
     a.kind = lean_kind(s, g, G.B, dtype);
     if (a.kind == SWEEP_GENERIC) return QAOA_ERR_UNSUPPORTED;
     const int rc = cuda_status(launch_sweep(dtype, s.two, a, st));
@@ -1255,7 +1285,7 @@ static int run_group(int dtype, int p, const BatchLayout& L, const BatchArgs& b,
   r.grid = grid;
   for (int o = 0; o < G.nout; ++o) {
     r.ncontrib[o] = G.ncontrib[o];
-    r.scale[o] = 1.0;
+    r.scale[o] = 2.0;
   }
   return cuda_status(launch_group_reduce(r, ng, G.bpg, row, partials, b.out, st));
 }

@@ -53,6 +53,7 @@ struct SweepGeom {
   int t;      // group qubits in the tile (j0 + t <= n)
   int c;      // low index bits carried in the tile (c <= j0), 0 for the first group
   int64_t tiles;  // number of tiles = 2^(n - t - c)
+  int pair;       // half states: the tile's top group bit is the flip of all qubits (SweepArgs::half)
 };
 
 enum SweepKind : int { SWEEP_GENERIC = 0, SWEEP_LEAN_MIX = 1, SWEEP_LEAN_OPS = 2 };
@@ -82,12 +83,26 @@ struct SweepArgs {
   // store 0 = internal, 1 = user, -1 = none.  complex64 internal == user.
   int load_fmt, store_fmt;
   int load_lam, store_lam;
+  // Half states (lean sweeps).  If C(z) = C(~z) (every cut), psi(z) = psi(~z) from |+> on, and the
+  // z with a clear top bit carry the whole state.  On those n - 1 qubits the mixer is
+  // exp(-i beta (X_0 + ... + X_(n-2) + X_0 X_1 ... X_(n-2))): the last term, X_(n-1), flips
+  // everything.  The first group's tile takes it: one of its 2^B local bits is then not a qubit but
+  // chooses between z and its complement, which turns the flip into an ordinary X on that bit;
+  // the other groups move down by one qubit and keep their sizes.  So a sweep runs the same code on
+  // half the tiles (half_geom), the layout of the state in memory is the plain one, only the first
+  // group's addresses differ (lean_tile), and sums double.  half = 1: run so; half = 2: run so if
+  // C is symmetric (scan; C is read once in each call).  The last sweep also stores the complements
+  // (mirror).
+  int half, mirror;
   int stage;          // lean two-buffer sweeps: psi of the block's next tile staged in shared memory
   long long init_fx;  // |+> amplitude in fixed point
   float init_f32;     // |+> amplitude in float32
   int fx_shift;       // fixed-point scale S (value = integer * 2^-S)
   const double* norm2_dev;             // optional: |psi|^2 of a user state (input scale)
-  const unsigned long long* cmax_dev;  // optional: bits of max |C| (lambda scale)
+  // optional: a scan of C, one entry per block of launch_cost_scan: the bits of its max |C| (the
+  // lambda scale), sign bit set if it met C(z) != C(~z)
+  const unsigned long long* scan;
+  int nscan;
   int nops;
   uint32_t ops[kMaxOps];
   // per layer angles, indexed by the op's layer field (dev_trig overrides them when the
@@ -151,13 +166,19 @@ void lean_f2(const SweepArgs& a, size_t sm, cudaStream_t s);         // complex6
 
 // launchers (return a CUDA error code)
 cudaError_t launch_sweep(int dtype, bool two, const SweepArgs& a, cudaStream_t s);
-cudaError_t launch_reduce(const ReducePlan& r, const double* partials, double* out, cudaStream_t s);
+// scan: optional, the sums double if C is symmetric
+cudaError_t launch_reduce(const ReducePlan& r, const double* partials, double* out, cudaStream_t s,
+                          const unsigned long long* scan = nullptr, int nscan = 0);
 // out[out_row[g] * nout + o] = sum over contributions k < ncontrib[o] and the blocks j < bpg of
 // graph g of partials[(o * kMaxContrib + k) * grid + g * bpg + j], for graphs g < ngraphs
 cudaError_t launch_group_reduce(const ReducePlan& r, int ngraphs, int bpg, const int* out_row,
                                 const double* partials, double* out, cudaStream_t s);
 cudaError_t launch_tables(const TableArgs& t, cudaStream_t s);
-cudaError_t launch_cost_bound(const void* C, int f64, int n, unsigned long long* out, cudaStream_t s);
+// scan of a cost vector of 2^n entries (SweepArgs::scan): cost_scan_blocks(n) entries, at most kMaxScan;
+// t: tables to build in the same launch (t.p = 0: none)
+constexpr int kMaxScan = 256;
+int cost_scan_blocks(int n);
+cudaError_t launch_cost_scan(const void* C, int f64, int n, unsigned long long* scan, const TableArgs& t, cudaStream_t s);
 cudaError_t launch_norm(const void* psi, int dtype, int n, double* partials, int* nblocks, cudaStream_t s);
 cudaError_t launch_adam(double* ang, const double* g, double* state, long long* step, int p, double lr, double b1,
                         double b2, double eps, double* history, long long row0, long long max_rows, cudaStream_t s);

@@ -105,6 +105,8 @@ __global__ void __launch_bounds__(CF::NT, CF::MINB) lean_kernel(const __grid_con
     else facc[r] = make_float2(0.f, 0.f);
     if (r < kLeanAcc) ishift[r] = 0;
   }
+  const CostScan scan = a.half == 2 ? read_scan(a.scan, a.nscan) : CostScan{a.half != 0, 0};
+  const SweepGeom g = scan.symmetric ? half_geom(a.g) : a.g;
   S s(a, X, Cs, nullptr, nullptr);
   s.wacc = wacc;
   if constexpr (FX) {
@@ -168,18 +170,15 @@ __global__ void __launch_bounds__(CF::NT, CF::MINB) lean_kernel(const __grid_con
   if constexpr (FX && TWO) {
     if (a.gslot != nullptr) {
       s.lam_shift = a.gslot[blockIdx.x / a.gbpg].lam_shift;
-    } else if (a.cmax_dev != nullptr) {
-      const unsigned long long b = *a.cmax_dev;
-      const int ex = (int)((b >> 52) & 0x7FF);
-      const int k = ex == 0 ? 0 : ex - 1023 + ((b & ((1ull << 52) - 1)) != 0 ? 1 : 0);
-      s.lam_shift = k < 0 ? 0 : k;
+    } else if (a.scan != nullptr) {
+      s.lam_shift = a.half == 2 ? scan.shift : read_scan(a.scan, a.nscan).shift;
     }
   }
   __syncthreads();
   bool have = false;  // this tile's psi is in the staging area
-  for (int64_t tile = t0; tile < a.g.tiles; tile += tstep) {
-    const int64_t next = tile + tstep < a.g.tiles ? tile + tstep : -1;
-    lean_tile<CF, FX, TWO, OPS, LAST, false, C>(s, a, tile, Cs, next, have);
+  for (int64_t tile = t0; tile < g.tiles; tile += tstep) {
+    const int64_t next = tile + tstep < g.tiles ? tile + tstep : -1;
+    lean_tile<CF, FX, TWO, OPS, LAST, false, C>(s, a, g, tile, Cs, next, have);
     have = s.Ps != nullptr && next >= 0;
   }
   __syncthreads();

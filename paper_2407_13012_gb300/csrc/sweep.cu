@@ -29,12 +29,7 @@ __global__ void __launch_bounds__(CF::NT, CF::MINB) sweep_kernel(const __grid_co
   const SweepGeom& g = a.g;
   s.evalid = 1u << (g.t + g.c);
   if constexpr (FX) {
-    if (a.cmax_dev != nullptr) {  // smallest k >= 0 with 2^k >= max |C|
-      const unsigned long long b = *a.cmax_dev;
-      const int ex = (int)((b >> 52) & 0x7FF);
-      int k = ex == 0 ? 0 : ex - 1023 + ((b & ((1ull << 52) - 1)) != 0 ? 1 : 0);
-      s.lam_shift = k < 0 ? 0 : k;
-    }
+    if (a.scan != nullptr) s.lam_shift = read_scan(a.scan, a.nscan).shift;
     if (a.norm2_dev != nullptr) {  // 2^k with |psi| / 2^k in [1, 2)
       const unsigned long long b = (unsigned long long)__double_as_longlong(*a.norm2_dev);
       const int ex = (int)((b >> 52) & 0x7FF);
@@ -51,7 +46,8 @@ __global__ void __launch_bounds__(CF::NT, CF::MINB) sweep_kernel(const __grid_co
 // ------------------------------------------------------------------ small kernels
 
 __global__ void reduce_kernel(const __grid_constant__ ReducePlan r, const double* __restrict__ partials,
-                              double* __restrict__ out) {
+                              double* __restrict__ out, const unsigned long long* scan, int nscan) {
+  const bool twice = scan != nullptr && read_scan(scan, nscan).symmetric;
   const int o = blockIdx.x;
   __shared__ double sh[256];
   double v = 0.0;
@@ -64,7 +60,7 @@ __global__ void reduce_kernel(const __grid_constant__ ReducePlan r, const double
     if ((int)threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
     __syncthreads();
   }
-  if (threadIdx.x == 0) out[o] = sh[0] * r.scale[o];
+  if (threadIdx.x == 0) out[o] = sh[0] * r.scale[o] * (twice ? 2.0 : 1.0);
 }
 
 // grouped sweeps: one warp per (graph, output), summing the graph's contributions and blocks
@@ -87,12 +83,16 @@ __global__ void group_reduce_kernel(const __grid_constant__ ReducePlan r, int ng
 
 // integer-cost phase tables exp(-i gamma_l c), c = cmin + k; then (fixed point) the
 // mixer diagonals exp(-i beta_l (t - 2k)) for t = 1..13, k = 0..t, and the turn tables
-__global__ void tables_kernel(const __grid_constant__ TableArgs ta) {
+__host__ __device__ inline int64_t table_entries(const TableArgs& t) {
+  return (int64_t)t.p * t.span + (t.fx ? (int64_t)t.p * 196 + kTurnEntries : 0) + (t.trig != nullptr ? t.p : 0);
+}
+// entries first, first + step, ... of the call's tables
+__device__ void make_tables(const TableArgs& ta, int64_t first, int64_t step) {
   const int64_t nphase = (int64_t)ta.p * ta.span;
   const int64_t nd = ta.fx ? (int64_t)ta.p * 14 * 14 : 0;
   const int64_t nt = ta.fx ? kTurnEntries : 0;
-  const int64_t total = nphase + nd + nt + (ta.trig != nullptr ? ta.p : 0);
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+  const int64_t total = table_entries(ta);
+  for (int64_t i = first; i < total; i += step) {
     if (i >= nphase + nd + nt) {  // [g2pi p | cos(beta) p | sin(beta) p] from device angles [gamma p | beta p]
       const int l = (int)(i - nphase - nd - nt);
       ta.trig[l] = ta.dev_angles[l] / (2.0 * 3.141592653589793238);
@@ -114,6 +114,9 @@ __global__ void tables_kernel(const __grid_constant__ TableArgs ta) {
       ((longlong2*)ta.turn)[i - nphase - nd] = turn_entry((int)(i - nphase - nd));
     }
   }
+}
+__global__ void tables_kernel(const __grid_constant__ TableArgs ta) {
+  make_tables(ta, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x);
 }
 
 // One Adam ascent step on the angles from the gradient output g = [E, norm, dE/dgamma,
@@ -146,20 +149,55 @@ __global__ void adam_kernel(double* __restrict__ ang, const double* __restrict__
   if (i == 0) *step = t + 1;
 }
 
-// max |C(z)| over the cost vector -> lam_shift = smallest k with 2^k >= max|C| (device scalar)
-__global__ void cost_bound_kernel(const void* __restrict__ C, int f64, int64_t count, unsigned long long* out) {
-  unsigned long long mx = 0;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
-    double c = f64 ? __ldg((const double*)C + i) : (double)__ldg((const int*)C + i);
-    c = fabs(c);
-    const unsigned long long b = (unsigned long long)__double_as_longlong(c);  // monotone for c >= 0
-    mx = b > mx ? b : mx;
+// |C| as an unsigned integer that orders like it
+__device__ __forceinline__ unsigned cost_abs(unsigned c) { return (int)c < 0 ? 0u - c : c; }
+__device__ __forceinline__ unsigned long long cost_abs(unsigned long long c) { return c & ~(1ull << 63); }
+
+// One read of C (float64 bits or int32): per block, the bits of max |C| as a double, with the sign
+// bit set if C[i] != C[count - 1 - i] for some i.  16 bytes at a time (both ends of C 16-byte
+// aligned) or one by one.  The call's tables (ta.p = 0: none) ride along, a warp's worth of entries to
+// each block before a second to any.
+template <class T>
+__global__ void __launch_bounds__(1024) cost_scan_kernel(const T* __restrict__ C, int64_t count, int vec,
+                                                         unsigned long long* __restrict__ scan,
+                                                         const __grid_constant__ TableArgs ta) {
+  if (ta.p > 0)
+    make_tables(ta, ((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31),
+                (int64_t)gridDim.x * blockDim.x);
+  const int64_t half = count >> 1, stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  constexpr int E = 16 / sizeof(T);
+  T mx = 0;
+  bool asym = false;
+  auto pair = [&](T x, T y) {
+    mx = max(mx, max(cost_abs(x), cost_abs(y)));
+    asym |= x != y;
+  };
+  union Q {
+    uint4 v;
+    T e[E];
+  };
+  if (vec) {
+#pragma unroll 4
+    for (int64_t i = first; i < (half + E - 1) / E; i += stride) {
+      Q x, y;
+      x.v = __ldg((const uint4*)C + i);
+      y.v = __ldg((const uint4*)(C + count) - 1 - i);
+#pragma unroll
+      for (int e = 0; e < E; ++e) pair(x.e[e], y.e[E - 1 - e]);
+    }
+  } else {
+    for (int64_t i = first; i < half; i += stride) pair(__ldg(C + i), __ldg(C + count - 1 - i));
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long y = __shfl_down_sync(0xffffffffu, mx, o);
-    mx = y > mx ? y : mx;
+  __shared__ T wmax[32];
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_down_sync(0xffffffffu, mx, o));
+  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = mx;
+  const bool any = __syncthreads_or(asym);
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) mx = max(mx, wmax[w]);
+    const unsigned long long b = sizeof(T) == 4 ? (unsigned long long)__double_as_longlong((double)mx) : (unsigned long long)mx;
+    scan[blockIdx.x] = b | (any ? 1ull << 63 : 0);
   }
-  if ((threadIdx.x & 31) == 0) atomicMax(out, mx);
 }
 
 // state norm^2 of a user (float64 / float32) state, for the fixed-point input scale
@@ -364,9 +402,10 @@ cudaError_t launch_expect(int dtype, const void* psi, const void* C, int cost_dt
   return cudaGetLastError();
 }
 
-cudaError_t launch_reduce(const ReducePlan& r, const double* partials, double* out, cudaStream_t s) {
+cudaError_t launch_reduce(const ReducePlan& r, const double* partials, double* out, cudaStream_t s,
+                          const unsigned long long* scan, int nscan) {
   note_launch(3, s, true);
-  reduce_kernel<<<r.nout, 256, 0, s>>>(r, partials, out);
+  reduce_kernel<<<r.nout, 256, 0, s>>>(r, partials, out, scan, nscan);
   note_launch(3, s, false);
   return cudaGetLastError();
 }
@@ -382,8 +421,7 @@ cudaError_t launch_group_reduce(const ReducePlan& r, int ngraphs, int bpg, const
 }
 
 cudaError_t launch_tables(const TableArgs& t, cudaStream_t s) {
-  const int64_t total =
-      (int64_t)t.p * t.span + (t.fx ? (int64_t)t.p * 196 + kTurnEntries : 0) + (t.trig != nullptr ? t.p : 0);
+  const int64_t total = table_entries(t);
   if (total <= 0) return cudaSuccess;
   // an entry is a float64 sincos, ~100 operations of which an SM quarter retires one per 64 cycles
   // and warp: one warp per block spreads them over the chip (with the angle terms in the same launch
@@ -395,14 +433,18 @@ cudaError_t launch_tables(const TableArgs& t, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_cost_bound(const void* C, int f64, int n, unsigned long long* out, cudaStream_t s) {
-  note_launch(3, s, true, (double)(1ull << n) * (f64 ? 8.0 : 4.0));
-  cudaMemsetAsync(out, 0, sizeof(unsigned long long), s);
+int cost_scan_blocks(int n) {
+  const int64_t blocks = ((1ll << n) + 8191) / 8192;
+  return (int)std::min<int64_t>({blocks, (int64_t)num_sms(), (int64_t)kMaxScan});
+}
+
+cudaError_t launch_cost_scan(const void* C, int f64, int n, unsigned long long* scan, const TableArgs& t, cudaStream_t s) {
   const int64_t count = 1ll << n;
-  int64_t blocks = (count + 255) / 256;
-  if (blocks > (int64_t)num_sms() * 8) blocks = (int64_t)num_sms() * 8;
-  cost_bound_kernel<<<(int)blocks, 256, 0, s>>>(C, f64, count, out);
-  note_launch(3, s, false, (double)(1ull << n) * (f64 ? 8.0 : 4.0));
+  const int vec = ((uintptr_t)C & 15) == 0 && n >= 2;
+  note_launch(3, s, true);
+  if (f64) cost_scan_kernel<<<cost_scan_blocks(n), 1024, 0, s>>>((const unsigned long long*)C, count, vec, scan, t);
+  else cost_scan_kernel<<<cost_scan_blocks(n), 1024, 0, s>>>((const unsigned*)C, count, vec, scan, t);
+  note_launch(3, s, false, (double)count * (f64 ? 8.0 : 4.0));
   return cudaGetLastError();
 }
 

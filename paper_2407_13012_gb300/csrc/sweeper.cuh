@@ -105,7 +105,33 @@ __device__ __forceinline__ uint64_t tile_base(const SweepGeom& g, int64_t tile) 
   const int lowrest_bits = g.j0 - g.c;
   const uint64_t lowrest = (uint64_t)tile & ((1ull << lowrest_bits) - 1);
   const uint64_t highrest = (uint64_t)tile >> lowrest_bits;
-  return (lowrest << g.c) | (highrest << (g.j0 + g.t));
+  return (lowrest << g.c) | (highrest << (g.j0 + g.t - g.pair));
+}
+// What a scan of C says, read by each warp for itself: whether C(z) = C(~z), and the smallest k >= 0
+// with 2^k >= max |C|.
+struct CostScan {
+  bool symmetric;
+  int shift;
+};
+__device__ __forceinline__ CostScan read_scan(const unsigned long long* scan, int nscan) {
+  bool asym = false;
+  int k = 0;
+  for (int i = threadIdx.x & 31; i < nscan; i += 32) {
+    const unsigned long long b = scan[i];
+    const int ex = (int)(b >> 52) & 0x7FF;
+    asym |= (b >> 63) != 0;
+    if (ex != 0) k = max(k, ex - 1023 + ((b & ((1ull << 52) - 1)) != 0 ? 1 : 0));
+  }
+  return {!__any_sync(0xffffffffu, asym), __reduce_max_sync(0xffffffffu, k)};
+}
+
+// the sweep's geometry on a half state
+__device__ __forceinline__ SweepGeom half_geom(SweepGeom g) {
+  g.n -= 1;
+  g.tiles >>= 1;
+  g.pair = g.j0 == 0;
+  g.j0 -= g.j0 != 0;
+  return g;
 }
 
 __device__ __forceinline__ uint64_t local_to_z(const SweepGeom& g, uint64_t base, uint32_t i) {
@@ -219,7 +245,7 @@ struct Sweeper {
   // float64 costs read from memory by the ops (layout 0) instead of from a staged tile: this
   // thread's first entry, and the stride of the register index; nullptr: the tile
   const double* Cg = nullptr;
-  uint64_t czs = 0;
+  uint64_t czs = 0, chi = 0;  // strides; offset of the upper half of the registers
   // the graph's data: a's, or one graph's of a grouped sweep (lean kernels)
   int64_t zoff;          // element offset of psi, lambda and C
   const void* ptab;      // phase tables
@@ -418,11 +444,11 @@ struct Sweeper {
   // psi (or lambda) *= exp(-i s gamma_l C): table lookups first, the rest out of line
   // the float64 cost of register r
   __device__ __forceinline__ double cost_at(bool f64, int r) const {
-    if (!FX && Cg != nullptr) return __ldg(Cg + (uint64_t)r * czs);
+    if (!FX && Cg != nullptr) return __ldg(Cg + (uint64_t)r * czs + (r >= R / 2 ? chi : 0));
     return cost_f(Cs, f64, idx(r));
   }
   __device__ __forceinline__ float cost32_at(bool f64, int r) const {
-    if (!FX && Cg != nullptr) return (float)__ldg(Cg + (uint64_t)r * czs);
+    if (!FX && Cg != nullptr) return (float)__ldg(Cg + (uint64_t)r * czs + (r >= R / 2 ? chi : 0));
     return cost_f32(Cs, f64, idx(r));
   }
   // u (and u2, if TWO_U) *= the directly computed phase factors of the registers in miss; the
@@ -1338,21 +1364,27 @@ struct Lean : Sweeper<CF, FX, TWO> {
 // `have` says that this tile's psi is there.  Each thread copies and reads back only its own
 // layout-0 slots, so the staging needs no barrier, only waits for the thread's own copy
 // groups; the cost tile's group is committed after the prefetch of this tile's psi and before
-// the prefetch of the next one.
+// the prefetch of the next one.  On a half state's first group (g.pair) the top local bit s, the top
+// register bit in layout 0, selects amplitude z (s = 0, bit n - 1 of z clear) or its complement
+// 2^n - 1 - z; the cost of the latter is C[z + 2^n], that of the same basis state with the full
+// state's top qubit set, so that cost tiles still travel in contiguous runs.
 template <class CF, bool FX, bool TWO, bool OPS, int LAST, bool COHERENT, int C = -1>
-__device__ __forceinline__ void lean_tile(Lean<CF, FX, TWO, C>& s, const SweepArgs& a, int64_t tile, void* Cs,
-                                          int64_t next = -1, bool have = false) {
+__device__ __forceinline__ void lean_tile(Lean<CF, FX, TWO, C>& s, const SweepArgs& a, const SweepGeom& g,
+                                          int64_t tile, void* Cs, int64_t next = -1, bool have = false) {
   using V = typename Lean<CF, FX, TWO, C>::V;
   constexpr int R = CF::R;
   V (&v)[R] = s.v;
   V (&w)[R] = s.w;
-  const SweepGeom& g = a.g;
   const uint32_t tid = threadIdx.x;
   const bool cf64 = a.cost_dtype == QAOA_COST_F64;
   const bool direct = !FX && OPS && a.needs_cost && cf64;  // float64 costs, read by the ops
   const bool cost = OPS && a.needs_cost && !direct;
   const uint32_t tb0 = CF::idx(0, tid, 0);
   const uint64_t zs = 1ull << (CF::lo(0) - s.gc() + g.j0);
+  static_assert(CF::lo(0) == CF::B - CF::RB, "the top local bit is the top register bit of layout 0");
+  // register r at z0 + r zs, for r >= R / 2 at upper(z0) + r zu
+  const uint64_t zu = g.pair ? 0 - zs : zs;
+  auto upper = [&](uint64_t z0) { return g.pair ? (1ull << g.n) - 1 - z0 + (R / 2) * zs : z0; };
   const bool init = OPS && a.load_fmt == 2;
   const bool ld_lam = TWO && (!OPS || a.load_lam), st_lam = TWO && (!OPS || a.store_lam);
   const int st_fmt = OPS ? a.store_fmt : 0;
@@ -1368,7 +1400,8 @@ __device__ __forceinline__ void lean_tile(Lean<CF, FX, TWO, C>& s, const SweepAr
     const uint32_t nch = 1u << (CF::B - pb);
     for (uint32_t ch = tid; ch < nch; ch += CF::NT) {
       const uint32_t i = ch << pb;
-      const uint64_t z = local_to_z(g, base, i);
+      const uint64_t z = g.pair ? (base | (i & ((1u << (CF::B - 1)) - 1))) + ((uint64_t)(i >> (CF::B - 1)) << g.n)
+                                : local_to_z(g, base, i);
       char* dst = (char*)Cs + ((size_t)phys_cost(i, cf64) << eb);
       const char* src = (const char*)a.C + ((s.zoff + z) << eb);
       if (pb + eb == 4) cp_async16(dst, src);
@@ -1385,21 +1418,23 @@ __device__ __forceinline__ void lean_tile(Lean<CF, FX, TWO, C>& s, const SweepAr
   if (direct) {
     s.Cg = (const double*)a.C + s.zoff + z0;
     s.czs = zs;
+    s.chi = g.pair ? (1ull << g.n) - (R / 2) * zs : 0;
   }
+  const uint64_t z0u = upper(z0);
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    const uint64_t z = z0 + (uint64_t)r * zs;
+    const uint64_t z = r < R / 2 ? z0 + (uint64_t)r * zs : z0u + (uint64_t)r * zu;
     const uint32_t ps = tb0 + ((uint32_t)r << CF::lo(0));
     if constexpr (FX) v[r] = init ? make_longlong2(a.init_fx, 0) : staged ? s.Ps[ps] : ld_state<COHERENT>((const V*)a.psi + s.zoff + z);
     else v[r] = init ? make_float2(a.init_f32, 0.f) : staged ? s.Ps[ps] : ld_state<COHERENT>((const V*)a.psi + s.zoff + z);
     if constexpr (TWO) w[r] = ld_lam ? ld_state<COHERENT>((const V*)a.lam + s.zoff + z) : V{};
   }
   if (stage && next >= 0) {
-    const uint64_t zn = local_to_z(g, tile_base(g, next), tb0);
+    const uint64_t zn = local_to_z(g, tile_base(g, next), tb0), znu = upper(zn);
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       V* dst = s.Ps + tb0 + ((uint32_t)r << CF::lo(0));
-      const V* src = (const V*)a.psi + s.zoff + zn + (uint64_t)r * zs;
+      const V* src = (const V*)a.psi + s.zoff + (r < R / 2 ? zn + (uint64_t)r * zs : znu + (uint64_t)r * zu);
       if constexpr (sizeof(V) == 16) cp_async16(dst, src);
       else cp_async8(dst, src);
     }
@@ -1415,16 +1450,25 @@ __device__ __forceinline__ void lean_tile(Lean<CF, FX, TWO, C>& s, const SweepAr
     __syncthreads();
   }
   s.template run<LAST, OPS>();
-  const uint64_t z1 = local_to_z(g, base, tb0);
+  const uint64_t z1 = local_to_z(g, base, tb0), z1u = upper(z1);
+  const bool mirror = OPS && a.mirror && g.n != a.g.n;  // (one-graph calls: zoff = 0)
+  const uint64_t zc = (1ull << a.g.n) - 1;
 #pragma unroll
   for (int r = 0; r < R; ++r) {
-    const uint64_t z = s.zoff + z1 + (uint64_t)r * zs;
+    const uint64_t z = s.zoff + (r < R / 2 ? z1 + (uint64_t)r * zs : z1u + (uint64_t)r * zu);
     if constexpr (FX) {
-      if (st_fmt == 0) ((V*)a.psi)[z] = v[r];
-      else if (st_fmt == 1)
-        ((double2*)a.psi)[z] = make_double2(fx_to_double(v[r].x, a.fx_shift), fx_to_double(v[r].y, a.fx_shift));
+      if (st_fmt == 0) {
+        ((V*)a.psi)[z] = v[r];
+      } else if (st_fmt == 1) {
+        const double2 d = make_double2(fx_to_double(v[r].x, a.fx_shift), fx_to_double(v[r].y, a.fx_shift));
+        ((double2*)a.psi)[z] = d;
+        if (mirror) ((double2*)a.psi)[zc - z] = d;
+      }
     } else {
-      if (st_fmt >= 0) ((V*)a.psi)[z] = v[r];
+      if (st_fmt >= 0) {
+        ((V*)a.psi)[z] = v[r];
+        if (mirror) ((V*)a.psi)[zc - z] = v[r];
+      }
     }
     if (st_lam) ((V*)a.lam)[z] = w[r];
   }
