@@ -1165,18 +1165,52 @@ struct Lean : Sweeper<CF, FX, TWO> {
     wht_mask(this->v, m);
     if constexpr (TWO) if (lam) wht_mask(this->w, m);
   }
+  // round K on both buffers and the move to layout T, psi's stores ahead of lambda's round, so that they
+  // overlap it (n = 28, p = 6 gradient 83.0 -> 81.6 ms)
+  template <int K, int T>
+  __device__ __forceinline__ void wht_move(bool lam) {
+    const unsigned m = gmask<K>();
+    const uint32_t pf = CF::phys(CF::idx(K, this->tid, 0)), pt = CF::phys(CF::idx(T, this->tid, 0));
+    V* X = this->X;
+    V* X2 = X + (1u << CF::B);
+    wht_mask(this->v, m);
+#pragma unroll
+    for (int r = 0; r < R; ++r) X[pf ^ CF::phys((uint32_t)r << CF::lo(K))] = this->v[r];
+    asm volatile("" ::: "memory");
+    if (lam) wht_mask(this->w, m);
+#pragma unroll
+    for (int r = 0; r < R; ++r) X2[pf ^ CF::phys((uint32_t)r << CF::lo(K))] = this->w[r];
+    this->template xsync<K, T>();
+#pragma unroll
+    for (int r = 0; r < R; ++r) this->v[r] = X[pt ^ CF::phys((uint32_t)r << CF::lo(T))];
+#pragma unroll
+    for (int r = 0; r < R; ++r) this->w[r] = X2[pt ^ CF::phys((uint32_t)r << CF::lo(T))];
+    this->cur = T;
+  }
   template <int K, int L>
   __device__ __forceinline__ void fx_fwd(bool lam) {
-    if constexpr (K > 0) exb<K - 1, K>();
-    wht_k<K>(lam);
-    if constexpr (K < L) fx_fwd<K + 1, L>(lam);
+    if constexpr (TWO && K < L) {
+      wht_move<K, K + 1>(lam);
+      fx_fwd<K + 1, L>(lam);
+    } else {
+      wht_k<K>(lam);
+      if constexpr (K < L) {
+        exb<K, K + 1>();
+        fx_fwd<K + 1, L>(lam);
+      }
+    }
   }
   template <int K>
   __device__ __forceinline__ void fx_back(bool lam) {
-    wht_k<K>(lam);
-    if constexpr (K > 0) {
-      exb<K, K - 1>();
+    if constexpr (TWO && K > 0) {
+      wht_move<K, K - 1>(lam);
       fx_back<K - 1>(lam);
+    } else {
+      wht_k<K>(lam);
+      if constexpr (K > 0) {
+        exb<K, K - 1>();
+        fx_back<K - 1>(lam);
+      }
     }
   }
   template <int L>
