@@ -162,6 +162,7 @@ void lean_x2_ops(const SweepArgs& a, size_t sm, cudaStream_t s);     // complex1
 void lean_xt1(const SweepArgs& a, size_t sm, cudaStream_t s);        // complex128, small tiles, one buffer
 void lean_xt2(const SweepArgs& a, size_t sm, cudaStream_t s);        // complex128, small tiles, two buffers
 void lean_f1(const SweepArgs& a, size_t sm, cudaStream_t s);         // complex64, one buffer
+void lean_f1d(const SweepArgs& a, size_t sm, cudaStream_t s);        // complex64, one buffer, float64 costs
 void lean_f2(const SweepArgs& a, size_t sm, cudaStream_t s);         // complex64, two buffers
 
 // launchers (return a CUDA error code)

@@ -58,6 +58,11 @@ inline void once_per_device(std::mutex& mu, uint64_t& done, F&& setup) {
 
 // complex64 single buffer: 8192-amplitude tiles, 32 per thread, 256 threads
 using CfgF1 = Cfg<13, 5, 5, 4, 2>;
+// the same tiles at 16 per thread, 512 threads, for op programs that read float64 costs: a computed
+// phase is a chain (turn fraction, then sine and cosine) that twice the warps hide better (n = 29,
+// p = 5 layers 19.3 -> 17.0 ms, n = 24, p = 4 575 -> 474 us; with integer costs the extra exchange costs
+// more: n = 26, p = 4 layers 2.94 -> 3.18 ms)
+using CfgF1D = Cfg<13, 4, 4, 4, 2>;
 // complex64 two buffers (gradient) with 8192-amplitude tiles: 16 amplitudes per thread per
 // buffer, 512 threads, one block per SM; at n = 32 this keeps >= 3 carried low bits (64-byte
 // rows)
