@@ -192,7 +192,7 @@ static int lean_kind(const Sweep& s, const Group& g, int tile_bits, int dtype) {
 // gradient 2143 -> 1271; complex64 n = 20 layers 96 -> 111 us, n = 21 134 -> 115, gradient 468 -> 324;
 // n = 30, p = 6 layers 194 -> 101 ms.  A C that is not symmetric pays for the read: n = 20, p = 6
 // complex128 layers 182 -> 188 us, n = 22 573 -> 587.
-static int half_min_n(int dtype, bool gradient) { return dtype == QAOA_C64 ? 21 : gradient ? 18 : 20; }
+static int half_min_n(int dtype, bool gradient) { return dtype == QAOA_C64 ? 21 : gradient ? 18 : 19; }
 
 // Run a list of sweeps with one shared grid, then reduce the partials into out[0..nout).
 // Fixed-point (complex128) calls also get: the input scale from the norm of a loaded

@@ -160,6 +160,8 @@ void lean_x1(const SweepArgs& a, size_t sm, cudaStream_t s);         // complex1
 void lean_x2_mix(const SweepArgs& a, size_t sm, cudaStream_t s);     // complex128, two buffers: one mixer
 void lean_x2_ops(const SweepArgs& a, size_t sm, cudaStream_t s);     // complex128, two buffers: op programs
 void lean_xt1(const SweepArgs& a, size_t sm, cudaStream_t s);        // complex128, small tiles, one buffer
+void lean_xm1(const SweepArgs& a, size_t sm, cudaStream_t s);        // complex128, 1024-amplitude tiles
+void lean_xm2(const SweepArgs& a, size_t sm, cudaStream_t s);        // the same, two buffers
 void lean_xt2(const SweepArgs& a, size_t sm, cudaStream_t s);        // complex128, small tiles, two buffers
 void lean_f1(const SweepArgs& a, size_t sm, cudaStream_t s);         // complex64, one buffer
 void lean_f1d(const SweepArgs& a, size_t sm, cudaStream_t s);        // complex64, one buffer, float64 costs

@@ -259,6 +259,7 @@ int blocks_per_sm(int cost_bytes) {
 template <class CF, bool FX, bool TWO>
 void lean_launch_cfg(const SweepArgs& a, size_t sm, cudaStream_t s) {
   if constexpr (CF::B == CfgXT::B) TWO ? lean_xt2(a, sm, s) : lean_xt1(a, sm, s);
+  else if constexpr (CF::B == CfgXM::B) TWO ? lean_xm2(a, sm, s) : lean_xm1(a, sm, s);
   else if constexpr (FX && !TWO) lean_x1(a, sm, s);
   else if constexpr (FX) a.kind == SWEEP_LEAN_OPS ? lean_x2_ops(a, sm, s) : lean_x2_mix(a, sm, s);
   else if constexpr (!TWO) lean_f1(a, sm, s);
@@ -347,11 +348,13 @@ __global__ void expect_kernel(const void* __restrict__ psi, const void* __restri
 // same number of sweeps as on 4096-amplitude tiles): they fill the chip better while the large
 // tiles of such a state are fewer than its SMs.  Measured, 4096- -> 512-amplitude tiles: n = 14, p = 4,
 // 50 Adam steps 12.4 -> 5.5 ms; n = 16 and 18, p = 6 gradients 353 -> 175 and 366 -> 266 us; n = 17,
-// p = 6 layers 151 -> 88 us.
-constexpr int kSmallTileN = 18;
+// p = 6 layers 151 -> 88 us.  n = 19 (4096- -> 1024-amplitude tiles, half states): p = 6 layers 151 -> 118 us,
+// gradient 383 -> 314 us, 50 Adam steps 12.3 -> 10.2 ms.  At n = 20 those lose: layers 151 -> 153, gradient
+// 389 -> 430 us, and a cost that is not symmetric 189 -> 230 us.
+constexpr int kSmallTileN = 18, kMidTileN = 19;
 
 int sweep_tile_bits(int dtype, int n) {
-  return dtype == QAOA_C128 ? (n <= kSmallTileN ? CfgXT::B : CfgX1::B) : CfgF1::B;
+  return dtype == QAOA_C128 ? (n <= kSmallTileN ? CfgXT::B : n <= kMidTileN ? CfgXM::B : CfgX1::B) : CfgF1::B;
 }
 
 // values stay below 2^61 through a group's Walsh-Hadamard transform (growth 2^(t/2)) for
@@ -362,6 +365,8 @@ int sweep_grid(int dtype, bool two, int tile_bits, int cost_bytes, int64_t tiles
   int per_sm;
   if (dtype == QAOA_C128 && tile_bits == CfgXT::B) {
     per_sm = two ? blocks_per_sm<CfgXT, true, true>(cost_bytes) : blocks_per_sm<CfgXT, true, false>(cost_bytes);
+  } else if (dtype == QAOA_C128 && tile_bits == CfgXM::B) {
+    per_sm = two ? blocks_per_sm<CfgXM, true, true>(cost_bytes) : blocks_per_sm<CfgXM, true, false>(cost_bytes);
   } else if (dtype == QAOA_C128) {
     per_sm = two ? blocks_per_sm<CfgX2, true, true>(cost_bytes) : blocks_per_sm<CfgX1, true, false>(cost_bytes);
   } else if (two) {
@@ -378,6 +383,9 @@ cudaError_t launch_sweep(int dtype, bool two, const SweepArgs& a, cudaStream_t s
   if (dtype == QAOA_C128 && a.tile_bits == CfgXT::B) {
     if (two) launch_t<CfgXT, true, true>(a, s);
     else launch_t<CfgXT, true, false>(a, s);
+  } else if (dtype == QAOA_C128 && a.tile_bits == CfgXM::B) {
+    if (two) launch_t<CfgXM, true, true>(a, s);
+    else launch_t<CfgXM, true, false>(a, s);
   } else if (dtype == QAOA_C128) {
     if (two) launch_t<CfgX2, true, true>(a, s);
     else launch_t<CfgX1, true, false>(a, s);

@@ -77,6 +77,8 @@ using CfgX2 = Cfg<12, 3, 3, 3, 1>;
 // (~25 us, whatever the rest of the chip does); 512-amplitude tiles spread it over 32 SMs with an
 // eighth of the work per SM quarter.
 using CfgXT = Cfg<9, 2, 2, 3, 4>;
+// and one size more: 1024-amplitude tiles, still two groups
+using CfgXM = Cfg<10, 2, 2, 3, 3>;
 
 // cost-tile slot of local index i; the XOR leaves the bits inside a 16-byte chunk alone so
 // the tile can be fetched with 16-byte asynchronous copies
