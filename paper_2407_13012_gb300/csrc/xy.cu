@@ -140,7 +140,8 @@ __global__ void __launch_bounds__(kXYThreads) xy_cost_kernel(const __grid_consta
 }
 
 template <typename T>
-__global__ void xy_init_kernel(T* __restrict__ psi, unsigned long long D, double amp) {
+__global__ void xy_init_kernel(T* __restrict__ psi, unsigned long long D, double amp, const unsigned* half_flag) {
+  if (half_flag != nullptr && *half_flag == 0) D >>= 1;
   for (unsigned long long r = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; r < D;
        r += (unsigned long long)gridDim.x * blockDim.x) {
     T v;
@@ -162,6 +163,27 @@ __device__ __forceinline__ float2 phase_of(double theta, float2*) {
   float sn, cs;
   sincosf((float)red, &sn, &cs);
   return make_float2(cs, -sn);
+}
+
+// *asym = 1 if C[i] != C[D - 1 - i] (bitwise) for some i (cleared by the caller)
+template <class C>
+__global__ void xy_symmetry_kernel(const C* __restrict__ c, unsigned long long D, unsigned* asym) {
+  bool bad = false;
+#pragma unroll 4
+  for (unsigned long long r = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; r < D / 2;
+       r += (unsigned long long)gridDim.x * blockDim.x)
+    bad |= __ldg(c + r) != __ldg(c + (D - 1 - r));
+  if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(asym, 1u);
+}
+
+// the whole state from its first half, if C is symmetric
+template <typename T>
+__global__ void xy_mirror_kernel(T* __restrict__ psi, unsigned long long D, const unsigned* asym) {
+  if (*asym != 0) return;
+#pragma unroll 4
+  for (unsigned long long r = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; r < D / 2;
+       r += (unsigned long long)gridDim.x * blockDim.x)
+    psi[D - 1 - r] = psi[r];
 }
 
 template <typename T>
@@ -243,7 +265,9 @@ struct Acc<float2> {
 template <typename T>
 __global__ void __launch_bounds__(kXYThreads)
     xy_lambda_kernel(const T* __restrict__ psi, T* __restrict__ lam, const void* __restrict__ C, int cost_dtype,
-                     unsigned long long D, double* __restrict__ pe, double* __restrict__ pn) {
+                     unsigned long long D, double* __restrict__ pe, double* __restrict__ pn,
+                     const unsigned* half_flag) {
+  if (half_flag != nullptr && *half_flag == 0) D >>= 1;
   __shared__ double red[kXYThreads / 32];
   using R = typename Real<T>::type;
   Acc<T> e, nn;
@@ -287,29 +311,19 @@ __device__ __forceinline__ void xy_rotate(T& x, T& y, typename Real<T>::type cb,
 // of bases per column.  So a pair costs two table reads and two additions, with consecutive
 // threads on consecutive patterns; walking all ranks took 250 instructions per amplitude with a
 // quarter of the lanes on a pair (463 us at n = 28, k = 14 complex128, a tenth of a layer).
-constexpr int kCloseBits = 10;   // most low bits: both parts are below binom(11, 5) + ... < 2^16
-constexpr int kCloseCols = 256;  // columns per tile
-constexpr int kClosePairs = 2048;
-struct XYClosing {
-  int n, k, lb, nh, ncls;
-  unsigned long long tiles;
-  struct Cls {
-    unsigned long long first_tile, ncols;
-    int kl, rows, start, m;
-  } cls[kCloseBits + 1];
-};
-
 // TWO: backwards on psi and lambda, taking the gate's term 2 Im <lambda|K|psi> first (one partial
 // per block)
-template <typename T, bool TWO>
+// FOLD: on half the state; launches with a flag come in both forms, the one not asked for returning.
+template <typename T, bool TWO, bool FOLD>
 __global__ void __launch_bounds__(kXYThreads)
-    xy_closing_kernel(const __grid_constant__ XYClosing W, T* __restrict__ psi, T* __restrict__ lam,
+    xy_closing_kernel(const __grid_constant__ xyw::Closing W, T* __restrict__ psi, T* __restrict__ lam,
                       typename Real<T>::type cb, typename Real<T>::type sb, double* __restrict__ part) {
   __shared__ unsigned long long B[kBN][kBN];
-  __shared__ unsigned short r1[1 << kCloseBits], r0[1 << kCloseBits];
-  __shared__ unsigned long long b1[kCloseCols], b0[kCloseCols];
+  __shared__ unsigned short r1[1 << xyw::kCloseBits], r0[1 << xyw::kCloseBits];
+  __shared__ unsigned long long b1[xyw::kCloseCols], b0[xyw::kCloseCols];
   __shared__ double red[kXYThreads / 32];
   const int tid = threadIdx.x;
+  if (W.f.flag != nullptr && (*W.f.flag == 0) != FOLD) return;
   for (int i = tid; i < (W.n + 1) * kBN; i += kXYThreads) (&B[0][0])[i] = (&g_pascal.v[0][0])[i];
   __syncthreads();
   for (unsigned x = tid; x < (1u << W.lb); x += kXYThreads) {
@@ -329,13 +343,17 @@ __global__ void __launch_bounds__(kXYThreads)
     r0[at] = (unsigned short)u0;
   }
   Acc<T> acc;
-  const unsigned long long t0 = W.tiles * blockIdx.x / gridDim.x, t1 = W.tiles * (blockIdx.x + 1ull) / gridDim.x;
+  constexpr bool half = FOLD;
+  [[maybe_unused]] const unsigned long long fold = W.f.last;
+  const unsigned long long tiles = half ? W.half_tiles : W.tiles;
+  const unsigned long long t0 = tiles * blockIdx.x / gridDim.x, t1 = tiles * (blockIdx.x + 1ull) / gridDim.x;
   int ci = 0;
   for (unsigned long long tile = t0; tile < t1; ++tile) {
-    while (ci + 1 < W.ncls && W.cls[ci + 1].first_tile <= tile) ++ci;
-    const XYClosing::Cls& C = W.cls[ci];
-    const unsigned long long col0 = (tile - C.first_tile) * (unsigned long long)C.m;
-    const int ncol = (int)(C.ncols - col0 < (unsigned long long)C.m ? C.ncols - col0 : (unsigned long long)C.m);
+    while (ci + 1 < W.ncls && (half ? W.cls[ci + 1].half_first : W.cls[ci + 1].first_tile) <= tile) ++ci;
+    const xyw::Closing::Cls& C = W.cls[ci];
+    const unsigned long long col0 = (tile - (half ? C.half_first : C.first_tile)) * (unsigned long long)C.m;
+    const unsigned long long cols = (half ? C.half_cols : C.ncols) - col0;
+    const int ncol = (int)(cols < (unsigned long long)C.m ? cols : (unsigned long long)C.m);
     __syncthreads();  // the tables are in; the previous tile is done with the bases
     for (int c = tid; c < ncol; c += kXYThreads) {
       unsigned long long h = xyw::unrank_bits(col0 + c, W.nh, W.k - 1 - C.kl, B);
@@ -355,7 +373,7 @@ __global__ void __launch_bounds__(kXYThreads)
 #pragma unroll 4
     for (int e = tid; e < items; e += kXYThreads) {
       const int c = (int)xyw::div_small((unsigned)e, mg), r = e - c * C.rows + C.start;
-      const unsigned long long rz = b1[c] + r1[r], rp = b0[c] + r0[r];
+      const unsigned long long rz = b1[c] + r1[r], rp = FOLD ? xyw::fold_rank(fold, b0[c] + r0[r]) : b0[c] + r0[r];
       T x = psi[rz], y = psi[rp];
       if constexpr (TWO) {
         T lx = lam[rz], ly = lam[rp];
@@ -557,7 +575,9 @@ __host__ __device__ inline size_t xy_binom_bytes(int n) {
 // With the closing pair's pass above: n = 30, k = 15, p = 3 layers 57.4 -> 47.4 ms complex128,
 // n = 27, k = 12, p = 2 gradient 10.4 -> 4.0 ms complex64.  Bound: the per-tile work (rotations and
 // conversions) and its latency at four blocks per SM, not memory.
-template <typename T, bool TWO, bool PH>
+// FOLD: the last window on half the state (without the cost unitary); with a flag its launches come in
+// both forms, the one not asked for returning at once.
+template <typename T, bool TWO, bool PH, bool FOLD>
 __global__ void __launch_bounds__(xy_window_threads(TWO), TWO ? 2 : 4)
     xy_window_kernel(const __grid_constant__ xyw::Window W, T* __restrict__ psi, T* __restrict__ lam,
                      typename Real<T>::type cb, typename Real<T>::type sb, double* __restrict__ part, int part_cols,
@@ -587,14 +607,19 @@ __global__ void __launch_bounds__(xy_window_threads(TWO), TWO ? 2 : 4)
   Acc<T> acc, cacc;
   double cacc_d = 0.0;
   int cur = -1;  // class whose row tables are in shared memory (the same in every thread)
-  const unsigned long long t0 = W.tiles * blockIdx.x / gridDim.x, t1 = W.tiles * (blockIdx.x + 1ull) / gridDim.x;
-  int ci = t0 < t1 ? xyw::find_class(W, t0) : 0;
+  const bool half = W.f.flag != nullptr && *W.f.flag == 0;
+  if (FOLD != (half && W.nh == 0)) return;
+  [[maybe_unused]] const unsigned long long fold = W.f.last;
+  const unsigned long long tiles = half ? W.half_tiles : W.tiles;
+  const unsigned long long t0 = tiles * blockIdx.x / gridDim.x, t1 = tiles * (blockIdx.x + 1ull) / gridDim.x;
+  int ci = t0 < t1 ? xyw::find_class(W, t0, half) : 0;
   for (unsigned long long tile = t0; tile < t1; ++tile) {
-    while (ci + 1 < W.ncls && W.cls[ci + 1].first_tile <= tile) ++ci;
+    while (ci + 1 < W.ncls && (half ? W.cls[ci + 1].half_first : W.cls[ci + 1].first_tile) <= tile) ++ci;
     const xyw::Class& C = W.cls[ci];
     const int rows = C.rows, mb = C.mb, m = 1 << mb;
-    const unsigned long long col0 = (tile - C.first_tile) << mb;
-    const int ncol = (int)(C.ncols - col0 < (unsigned long long)m ? C.ncols - col0 : (unsigned long long)m);
+    const unsigned long long col0 = (tile - (half ? C.half_first : C.first_tile)) << mb;
+    const unsigned long long cols = (half ? C.half_cols : C.ncols) - col0;
+    const int ncol = (int)(cols < (unsigned long long)m ? cols : (unsigned long long)m);
     const bool cm = C.len == 1;  // a column's rows are consecutive ranks
     const int stride = cm ? m + 1 : m;
     __syncthreads();  // the binomials are in; the previous tile is stored
@@ -645,7 +670,7 @@ __global__ void __launch_bounds__(xy_window_threads(TWO), TWO ? 2 : 4)
       for (int e = tid; e < ns; e += NT) {
         int r, c;
         if (!place(e, r, c)) continue;
-        const unsigned long long rk = rowoff[r] + colbase[c];
+        const unsigned long long rk = FOLD ? xyw::fold_rank(fold, rowoff[r] + colbase[c]) : rowoff[r] + colbase[c];
         const T x = psi[rk];  // raw bits for now; the exponents give the tile's scales
         exp_psi = max(exp_psi, xy_exp_bits(x));
         tp[r * stride + c] = make_longlong2((long long)fx::double_to_bits(x.x), (long long)fx::double_to_bits(x.y));
@@ -685,7 +710,7 @@ __global__ void __launch_bounds__(xy_window_threads(TWO), TWO ? 2 : 4)
       for (int e = tid; e < ns; e += NT) {
         int r, c;
         if (!place(e, r, c)) continue;
-        const unsigned long long rk = rowoff[r] + colbase[c];
+        const unsigned long long rk = FOLD ? xyw::fold_rank(fold, rowoff[r] + colbase[c]) : rowoff[r] + colbase[c];
         T v = psi[rk];
         if constexpr (PH && !TWO) {
           double cf = 0.0;
@@ -737,7 +762,7 @@ __global__ void __launch_bounds__(xy_window_threads(TWO), TWO ? 2 : 4)
     for (int e = tid; e < ns; e += NT) {
       int r, c;
       if (!place(e, r, c)) continue;
-      const unsigned long long rk = rowoff[r] + colbase[c];
+      const unsigned long long rk = FOLD ? xyw::fold_rank(fold, rowoff[r] + colbase[c]) : rowoff[r] + colbase[c];
       S X = tp[r * stride + c], L;
       if constexpr (TWO) L = tl[r * stride + c];
       if constexpr (TWO && PH) {  // the gamma term at the state right after the cost unitary, then undo it
@@ -799,7 +824,8 @@ constexpr int kXYPartStride = 2048;  // partial slots per launch (>= any grid us
 
 __global__ void __launch_bounds__(kXYThreads) xy_grad_reduce_kernel(const __grid_constant__ XYReducePlan rp,
                                                                     const double* __restrict__ part,
-                                                                    double* __restrict__ out) {
+                                                                    double* __restrict__ out,
+                                                                    const unsigned* half_flag) {
   __shared__ double red[kXYThreads / 32];
   const int o = blockIdx.x;
   double acc = 0.0;
@@ -808,7 +834,7 @@ __global__ void __launch_bounds__(kXYThreads) xy_grad_reduce_kernel(const __grid
     for (int b = threadIdx.x; b < rp.cols[o]; b += kXYThreads) acc += src[b];
   }
   const double t = block_sum(acc, red);
-  if (threadIdx.x == 0) out[o] = t;
+  if (threadIdx.x == 0) out[o] = half_flag != nullptr && *half_flag == 0 ? 2.0 * t : t;
 }
 
 // block partials of [sum C |psi|^2, sum |psi|^2] in float64, fixed order for a fixed grid
@@ -1020,22 +1046,39 @@ struct XYMixPlan {
   int nwin;
   bool closing;
   xyw::Window win[xyw::kMaxWindows];
+  xyw::Closing close;
 };
 
+// Smallest n of the balanced calls that check C for symmetry and run on half the state if they may
+// (xy_window.cuh).  Whole -> half: n = 26, p = 1 layers 1057 -> 597 us complex128, 400 -> 280 complex64,
+// p = 4 gradient 13.9 -> 7.2 and 4.54 -> 2.53 ms; n = 30, p = 3 complex128 layers 48.0 -> 25.5 ms.  A cost that
+// is not symmetric pays for the read of C and the launches that return at once: n = 26, p = 1 layers 1057 ->
+// 1077 us complex128, 400 -> 431 complex64, n = 28 4033 -> 4070 and 1647 -> 1695; below n = 26 that share grows.
+constexpr int kXYHalfMinN = 26;
+bool half_plan(const XYShape& s, int p, int init) {
+  return init && p > 0 && s.n >= kXYHalfMinN && s.n % 2 == 0 && s.k == s.n / 2;
+}
+
 template <typename T>
-XYMixPlan* make_mix_plan(const XYShape& s) {
+XYMixPlan* make_mix_plan(const XYShape& s, const unsigned* half_flag) {
   XYMixPlan* mp = new XYMixPlan;
   int lo[xyw::kMaxWindows + 1], w[xyw::kMaxWindows + 1];
   mp->nwin = xyw::plan_ring_windows(s.n, lo, w);
-  for (int i = 0; i < mp->nwin; ++i)
-    xyw::plan_window(mp->win[i], s.n, s.k, lo[i], w[i], xy_tile_elems<T>(), s.binom, i == 0);
+  for (int i = 0; i < mp->nwin; ++i) {
+    xyw::plan_window(mp->win[i], s.n, s.k, lo[i], w[i], xy_tile_elems<T>(), s.binom, i == 0, half_flag != nullptr);
+    mp->win[i].f.flag = half_flag;
+  }
   mp->closing = s.n >= 3;
+  if (mp->closing) {
+    mp->close = xyw::plan_closing(s.n, s.k, s.binom, half_flag != nullptr);
+    mp->close.f.flag = half_flag;
+  }
   return mp;
 }
 
 // one windowed pass on every SM's resident blocks; part_cols: the partial slots of a row (backward)
-template <typename T, bool TWO, bool PH>
-cudaError_t launch_window(const xyw::Window& W, T* psi, T* lam, typename Real<T>::type cb,
+template <typename T, bool TWO, bool PH, bool FOLD>
+cudaError_t launch_window_as(const xyw::Window& W, T* psi, T* lam, typename Real<T>::type cb,
                           typename Real<T>::type sb, double* part, int part_cols, const XYPhaseArgs<T>& ph,
                           cudaStream_t st) {
   static std::mutex mu;
@@ -1050,8 +1093,8 @@ cudaError_t launch_window(const xyw::Window& W, T* psi, T* lam, typename Real<T>
     std::lock_guard<std::mutex> lk(mu);
     if (!(done & (1ull << (dev & 63)))) {
       const size_t most = xy_binom_bytes(xyw::kMaxN) + xy_buffer_bytes<T>() * (TWO ? 2 : 1);
-      cudaFuncSetAttribute(xy_window_kernel<T, TWO, PH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[dev & 63], xy_window_kernel<T, TWO, PH>, NT,
+      cudaFuncSetAttribute(xy_window_kernel<T, TWO, PH, FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[dev & 63], xy_window_kernel<T, TWO, PH, FOLD>, NT,
                                                     xy_binom_bytes(32) + xy_buffer_bytes<T>() * (TWO ? 2 : 1));
       if (per_sm[dev & 63] < 1) per_sm[dev & 63] = 1;
       done |= 1ull << (dev & 63);
@@ -1063,52 +1106,61 @@ cudaError_t launch_window(const xyw::Window& W, T* psi, T* lam, typename Real<T>
   unsigned long long g = (unsigned long long)sm_count() * resident;
   if (TWO && g > (unsigned long long)part_cols) g = part_cols;
   const unsigned grid = (unsigned)(W.tiles < g ? W.tiles : g);
-  const double cb_bytes = PH ? (double)W.elems * cost_bytes(ph.cost_dtype) : 0.0;
-  const double bytes = (double)W.elems * sizeof(T) * 2 * (TWO ? 2 : 1) + cb_bytes;
+  // (only the device knows whether C is symmetric)
+  const double elems = W.f.flag == nullptr ? (double)W.elems : W.nh == 0 && !FOLD ? 0.0 : (double)W.half_elems;
+  const double cb_bytes = PH ? elems * cost_bytes(ph.cost_dtype) : 0.0;
+  const double bytes = elems * sizeof(T) * 2 * (TWO ? 2 : 1) + cb_bytes;
   note_launch(0, st, true);
-  xy_window_kernel<T, TWO, PH><<<grid, NT, smem, st>>>(W, psi, lam, cb, sb, part, part_cols, ph);
+  xy_window_kernel<T, TWO, PH, FOLD><<<grid, NT, smem, st>>>(W, psi, lam, cb, sb, part, part_cols, ph);
   note_launch(0, st, false, bytes);
   return cudaGetLastError();
 }
 
-// the closing pair's classes and tiles (n >= 3, 0 < k < n)
-XYClosing make_closing(const XYShape& s) {
-  XYClosing W;
-  std::memset(&W, 0, sizeof(W));
-  W.n = s.n;
-  W.k = s.k;
-  W.lb = std::max(0, std::min(kCloseBits, s.n - 2));
-  W.nh = std::max(0, s.n - 2 - W.lb);
-  int start = 0;
-  for (int kl = 0; kl <= W.lb; ++kl) {
-    const int rows = (int)s.binom[W.lb][kl], kh = s.k - 1 - kl;
-    if (kh >= 0 && kh <= W.nh) {
-      XYClosing::Cls& C = W.cls[W.ncls++];
-      C.kl = kl;
-      C.rows = rows;
-      C.start = start;
-      C.ncols = s.binom[W.nh][kh];
-      C.m = std::max(1, std::min(kCloseCols, kClosePairs / rows));
-      C.first_tile = W.tiles;
-      W.tiles += (C.ncols + C.m - 1) / C.m;
+template <typename T, bool TWO, bool PH>
+cudaError_t launch_window(const xyw::Window& W, T* psi, T* lam, typename Real<T>::type cb,
+                          typename Real<T>::type sb, double* part, int part_cols, const XYPhaseArgs<T>& ph,
+                          cudaStream_t st) {
+  if constexpr (!PH)
+    if (W.f.flag != nullptr && W.nh == 0) {
+      const cudaError_t e = launch_window_as<T, TWO, false, true>(W, psi, lam, cb, sb, part, part_cols, ph, st);
+      if (e != cudaSuccess) return e;
     }
-    start += rows;
-  }
-  return W;
+  return launch_window_as<T, TWO, PH, false>(W, psi, lam, cb, sb, part, part_cols, ph, st);
+}
+
+template <typename T, bool TWO>
+void launch_closing(const xyw::Closing& W, T* psi, T* lam, typename Real<T>::type cb, typename Real<T>::type sb,
+                    double* part, unsigned grid, cudaStream_t st) {
+  const double pairs = (double)(W.f.flag != nullptr ? W.half_pairs : W.pairs);
+  note_launch(0, st, true);
+  if (W.f.flag != nullptr) xy_closing_kernel<T, TWO, true><<<grid, kXYThreads, 0, st>>>(W, psi, lam, cb, sb, part);
+  xy_closing_kernel<T, TWO, false><<<grid, kXYThreads, 0, st>>>(W, psi, lam, cb, sb, part);
+  note_launch(0, st, false, pairs * 2 * sizeof(T) * (TWO ? 4 : 2));
 }
 
 template <typename T>
 int layers_t(const XYShape& s, T* psi, const qaoa_cost_t* cost, const double* gamma, const double* beta, int p,
-             int init, double* expect_dev, char* ws, cudaStream_t st) {
+             int init, double* expect_dev, char* ws, cudaStream_t st, bool whole = true) {
   using R = typename Real<T>::type;
   const int sms = sm_count();
   const size_t sb = sizeof(T);
   double* part = (double*)ws;
   const long long span = p > 0 ? table_span(cost) : 0;
   T* tab = span > 0 ? (T*)(ws + round256(2 * (size_t)kXYRedBlocks * sizeof(double))) : nullptr;
+  const bool half = half_plan(s, p, init);
+  unsigned* flag = half ? (unsigned*)part : nullptr;  // (in the partials' place: they are written after its last use)
+  if (half) {
+    note_launch(3, st, true);
+    cudaMemsetAsync(flag, 0, sizeof(unsigned), st);
+    if (cost->dtype == QAOA_COST_F64)
+      xy_symmetry_kernel<<<(unsigned)sms * 8, kXYThreads, 0, st>>>((const unsigned long long*)cost->C_dev, s.D, flag);
+    else
+      xy_symmetry_kernel<<<(unsigned)sms * 8, kXYThreads, 0, st>>>((const unsigned*)cost->C_dev, s.D, flag);
+    note_launch(3, st, false, (double)s.D * cost_bytes(cost->dtype));
+  }
   if (init) {
     note_launch(3, st, true);
-    xy_init_kernel<T><<<grid_for(s.D, sms), kXYThreads, 0, st>>>(psi, s.D, 1.0 / std::sqrt((double)s.D));
+    xy_init_kernel<T><<<grid_for(s.D, sms), kXYThreads, 0, st>>>(psi, s.D, 1.0 / std::sqrt((double)s.D), flag);
     note_launch(3, st, false, (double)s.D * sb);
   }
   if (tab != nullptr) {
@@ -1125,10 +1177,7 @@ int layers_t(const XYShape& s, T* psi, const qaoa_cost_t* cost, const double* ga
     note_launch(3, st, false);
   }
   const bool mixes = s.k > 0 && s.k < s.n && s.n >= 2;
-  XYMixPlan* mp = mixes && p > 0 ? make_mix_plan<T>(s) : nullptr;
-  const unsigned long long moved = s.n >= 2 && s.k >= 1 && s.k <= s.n - 1 ? 2 * s.binom[s.n - 2][s.k - 1] : 0;
-  const XYClosing cw = make_closing(s);
-  const unsigned cgrid = (unsigned)std::max<unsigned long long>(1, std::min<unsigned long long>(cw.tiles, (unsigned)sms * 6u));
+  XYMixPlan* mp = mixes && p > 0 ? make_mix_plan<T>(s, flag) : nullptr;
   for (int l = 0; l < p; ++l) {
     const XYPhaseArgs<T> ph = {cost->C_dev, cost->dtype, tab ? tab + (size_t)l * span : nullptr, cost->cmin, span,
                                gamma[l], nullptr};
@@ -1150,9 +1199,9 @@ int layers_t(const XYShape& s, T* psi, const qaoa_cost_t* cost, const double* ga
         }
       }
       if (mp->closing) {
-        note_launch(0, st, true);
-        xy_closing_kernel<T, false><<<cgrid, kXYThreads, 0, st>>>(cw, psi, nullptr, cb, snb, nullptr);
-        note_launch(0, st, false, (double)moved * 2 * sb);
+        const unsigned long long most = std::min<unsigned long long>(mp->close.tiles, (unsigned)sms * 6u);
+        launch_closing<T, false>(mp->close, psi, nullptr, cb, snb, nullptr,
+                                 (unsigned)std::max<unsigned long long>(1, most), st);
       }
     }
     const int rc = status_of(cudaGetLastError());
@@ -1162,6 +1211,11 @@ int layers_t(const XYShape& s, T* psi, const qaoa_cost_t* cost, const double* ga
     }
   }
   delete mp;
+  if (half && whole) {
+    note_launch(3, st, true);
+    xy_mirror_kernel<T><<<(unsigned)sms * 8, kXYThreads, 0, st>>>(psi, s.D, flag);
+    note_launch(3, st, false, (double)s.D * sb);
+  }
   if (expect_dev != nullptr) return expectation_t<T>(s, psi, cost, expect_dev, part, st);
   return status_of(cudaGetLastError());
 }
@@ -1181,7 +1235,7 @@ int gradient_t(const XYShape& s, T* psi, T* lam, const qaoa_cost_t* cost, const 
   const int sms = sm_count();
   const size_t sb = sizeof(T);
   // forward pass (Dicke start, p layers) with the layer workspace at the front
-  int rc = layers_t<T>(s, psi, cost, gamma, beta, p, 1, nullptr, ws, st);
+  int rc = layers_t<T>(s, psi, cost, gamma, beta, p, 1, nullptr, ws, st, false);
   if (rc) return rc;
   const long long span = p > 0 ? table_span(cost) : 0;
   const T* tab = span > 0 ? (const T*)(ws + round256(2 * (size_t)kXYRedBlocks * sizeof(double))) : nullptr;
@@ -1191,25 +1245,22 @@ int gradient_t(const XYShape& s, T* psi, T* lam, const qaoa_cost_t* cost, const 
   const unsigned gr = std::min<unsigned>(grid_for(s.D, sms), kXYPartStride);  // one partial slot per block
   const unsigned long long nch = (s.D + kXYChunk - 1) / kXYChunk;
   const unsigned gg = std::min<unsigned>(grid_for(nch, sms), kXYPartStride);
-  const unsigned long long moved = s.n >= 2 && s.k >= 1 && s.k <= s.n - 1 ? 2 * s.binom[s.n - 2][s.k - 1] : 0;
+  const bool half = half_plan(s, p, 1);
+  const unsigned* flag = half ? (const unsigned*)ws : nullptr;  // set by the forward pass
   note_launch(0, st, true);
-  xy_lambda_kernel<T><<<gr, kXYThreads, 0, st>>>(psi, lam, cost->C_dev, cost->dtype, s.D, part, part + kXYPartStride);
+  xy_lambda_kernel<T><<<gr, kXYThreads, 0, st>>>(psi, lam, cost->C_dev, cost->dtype, s.D, part, part + kXYPartStride,
+                                                 flag);
   note_launch(0, st, false, (double)s.D * (2 * sb + cost_bytes(cost->dtype)));
   // beta rows of layer l: one per window and one for the closing pair (at most np of them), every row's gg slots written
-  XYMixPlan* mp = np > 0 && p > 0 ? make_mix_plan<T>(s) : nullptr;
-  const XYClosing cw = make_closing(s);
+  XYMixPlan* mp = np > 0 && p > 0 ? make_mix_plan<T>(s, flag) : nullptr;
   const int brows = mp != nullptr ? mp->nwin + (mp->closing ? 1 : 0) : 0;
   const bool fused = mp != nullptr;  // gamma terms from the first window's pass (gg blocks)
   for (int l = p - 1; l >= 0; --l) {
     const R cb = (R)std::cos(beta[l]), snb = (R)(-std::sin(beta[l]));
     double* rows = part + (size_t)(2 + p + (size_t)l * np) * kXYPartStride;
     if (mp != nullptr) {
-      if (mp->closing) {  // applied last in the layer, undone first
-        note_launch(0, st, true);
-        xy_closing_kernel<T, true><<<gg, kXYThreads, 0, st>>>(cw, psi, lam, cb, snb,
-                                                               rows + (size_t)mp->nwin * kXYPartStride);
-        note_launch(0, st, false, (double)moved * 4 * sb);
-      }
+      if (mp->closing)  // applied last in the layer, undone first
+        launch_closing<T, true>(mp->close, psi, lam, cb, snb, rows + (size_t)mp->nwin * kXYPartStride, gg, st);
       // the first window's pass also takes the gamma term and undoes the cost unitary
       const XYPhaseArgs<T> ph = {cost->C_dev, cost->dtype, tab ? tab + (size_t)l * span : nullptr, cost->cmin,
                                  span, gamma[l], part + (size_t)(2 + l) * kXYPartStride};
@@ -1235,6 +1286,11 @@ int gradient_t(const XYShape& s, T* psi, T* lam, const qaoa_cost_t* cost, const 
       return rc;
     }
   }
+  if (half) {
+    note_launch(3, st, true);
+    xy_mirror_kernel<T><<<(unsigned)sms * 8, kXYThreads, 0, st>>>(psi, s.D, flag);
+    note_launch(3, st, false, (double)s.D * sb);
+  }
   delete mp;
   XYReducePlan rp;
   std::memset(&rp, 0, sizeof(rp));
@@ -1245,7 +1301,7 @@ int gradient_t(const XYShape& s, T* psi, T* lam, const qaoa_cost_t* cost, const 
     rp.first[2 + p + l] = 2 + p + l * np, rp.rows[2 + p + l] = brows, rp.cols[2 + p + l] = (int)gg;
   }
   note_launch(3, st, true);
-  xy_grad_reduce_kernel<<<rp.nout, kXYThreads, 0, st>>>(rp, part, out);
+  xy_grad_reduce_kernel<<<rp.nout, kXYThreads, 0, st>>>(rp, part, out, flag);
   note_launch(3, st, false);
   return status_of(cudaGetLastError());
 }

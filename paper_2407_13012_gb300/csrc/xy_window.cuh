@@ -26,9 +26,20 @@
 // pairs; pairs of different windows either commute or come in the order of the sets (an odd
 // pair that crosses e_i - 1 needs the even pair (e_i, e_i + 1), which its own window applies
 // first).  The closing pair is a pass of its own.
+//
+// Half states.  With k = n / 2 the complement ~z of a state is in F_k too, at rank D - 1 - rank(z)
+// (D = binom(n, k): complementing reverses the order), and it commutes with every pair gate.  So if
+// C(z) = C(~z) (every cut), psi(z) = psi(~z) from the Dicke state on, and the first D / 2 ranks, the
+// states with qubit n - 1 clear, carry the whole state.  A window below qubit n - 1 runs on the
+// columns whose H has a clear top bit: a prefix of each class's.  The last window and the closing
+// pair move qubit n - 1: they visit one of every two complementary columns (pairs), those whose top
+// bit below the window (of the middle bits) is clear, again a prefix of each class's, and an
+// element of rank r lives at min(r, D - 1 - r).
 #pragma once
 
 #include <stdint.h>
+
+#include <algorithm>
 
 #ifdef __CUDACC__
 #define XYW_HD __host__ __device__ __forceinline__
@@ -51,12 +62,21 @@ constexpr int kMaxWindows = (kMaxN + 6) / 8 + 1;         // [0, 8), then 8 new q
 
 typedef unsigned long long u64;
 
+// Half states: a launch with a flag (device) runs on half the state if *flag == 0; D - 1.
+struct Fold {
+  u64 last;
+  const unsigned* flag;
+};
+XYW_HD u64 fold_rank(u64 last, u64 r) { return r < last - r ? r : last - r; }
+
 struct Class {
   u64 first_tile;  // tiles of the classes before this one
   u64 ncols;       // binom(nh, h) * len
+  u64 half_first, half_cols;  // the same on a half state
   u64 len;         // binom(lo, kL): ranks per row run of one H
-  int h, kw, kL;   // popcounts above, inside and below the window
-  int rows, m, mb; // binom(w, kw); columns per tile, a power of two: m = 2^mb
+  unsigned char h, kw, kL;  // popcounts above, inside and below the window
+  unsigned char mb;         // columns per tile, a power of two: m = 2^mb
+  unsigned short rows, m;   // binom(w, kw)
 };
 
 struct Window {
@@ -67,6 +87,8 @@ struct Window {
   int tile_elems;     // largest rows * m over the classes
   u64 tiles;
   u64 elems;          // amplitudes visited by one pass
+  u64 half_tiles, half_elems;
+  Fold f;
   Class cls[kMaxClasses];
 };
 
@@ -134,11 +156,11 @@ XYW_HD unsigned div_small(unsigned x, unsigned m) {
 #endif
 }
 
-XYW_HD int find_class(const Window& W, u64 tile) {
+XYW_HD int find_class(const Window& W, u64 tile, bool half = false) {
   int a = 0, b = W.ncls - 1;
   while (a < b) {
     const int mid = (a + b + 1) / 2;
-    if (W.cls[mid].first_tile <= tile) a = mid;
+    if ((half ? W.cls[mid].half_first : W.cls[mid].first_tile) <= tile) a = mid;
     else b = mid - 1;
   }
   return a;
@@ -174,8 +196,9 @@ inline int plan_ring_windows(int n, int* lo, int* w) {
 // Window [lo, lo + w) of the ring mixer on n qubits: its pairs and its tile classes.
 // `target` = amplitudes per tile (per buffer); `every_state` also visits the single-row
 // classes (kw = 0, kw = w), for a pass that applies the cost unitary to every amplitude.
+// `half` (k = n / 2; not for a window of all qubits) also plans the pass over a half state.
 inline void plan_window(Window& W, int n, int k, int lo, int w, int target, const u64 (*B)[kBN],
-                        bool every_state = false) {
+                        bool every_state = false, bool half = false) {
   W.n = n;
   W.k = k;
   W.lo = lo;
@@ -188,31 +211,86 @@ inline void plan_window(Window& W, int n, int k, int lo, int w, int target, cons
   W.ncls = 0;
   W.tiles = 0;
   W.elems = 0;
+  W.half_tiles = W.half_elems = 0;
+  W.f.last = half ? B[n][k] - 1 : 0;
+  W.f.flag = nullptr;
   W.tile_elems = 0;
   for (int h = 0; h <= W.nh; ++h) {
     for (int kw = every_state ? 0 : 1; kw <= (every_state ? w : w - 1); ++kw) {
       const int kL = k - h - kw;
       if (kL < 0 || kL > lo) continue;
       Class& C = W.cls[W.ncls++];
-      C.h = h;
-      C.kw = kw;
-      C.kL = kL;
-      C.rows = (int)B[w][kw];
+      C.h = (unsigned char)h;
+      C.kw = (unsigned char)kw;
+      C.kL = (unsigned char)kL;
+      C.rows = (unsigned short)B[w][kw];
       C.len = B[lo][kL];
       C.ncols = B[W.nh][h] * C.len;
+      C.half_cols = !half ? 0 : W.nh == 0 ? B[lo - 1][kL] : B[W.nh - 1][h] * C.len;
       u64 m = 1;  // the most columns of a power of two in the target, no more than the class needs
       C.mb = 0;
       while (2 * m * (u64)C.rows <= (u64)target && 2 * m <= (u64)kMaxCols && m < C.ncols) {
         m *= 2;
         ++C.mb;
       }
-      C.m = (int)m;
+      C.m = (unsigned short)m;
       C.first_tile = W.tiles;
       W.tiles += (C.ncols + m - 1) / m;
       W.elems += C.ncols * (u64)C.rows;
+      C.half_first = W.half_tiles;
+      W.half_tiles += (C.half_cols + m - 1) / m;
+      W.half_elems += C.half_cols * (u64)C.rows;
       if (C.rows * C.m > W.tile_elems) W.tile_elems = C.rows * C.m;
     }
   }
+}
+
+// ---------------------------------------------------------------- the closing pair
+
+constexpr int kCloseBits = 10;   // most low bits: both parts are below binom(11, 5) + ... < 2^16
+constexpr int kCloseCols = 256;  // columns per tile
+constexpr int kClosePairs = 2048;
+struct Closing {
+  int n, k, lb, nh, ncls;
+  u64 tiles, half_tiles;
+  u64 pairs, half_pairs;  // visited by one pass
+  Fold f;
+  struct Cls {
+    u64 first_tile, ncols, half_first, half_cols;
+    int kl, rows, start, m;
+  } cls[kCloseBits + 1];
+};
+
+// the closing pair's classes and tiles (n >= 3, 0 < k < n).  Half states (n >= lb + 3): one of every
+// two complementary pairs, the one whose middle bits have a clear top bit.
+inline Closing plan_closing(int n, int k, const u64 (*B)[kBN], bool half = false) {
+  Closing W = {};
+  W.n = n;
+  W.k = k;
+  W.lb = std::max(0, std::min(kCloseBits, n - 2));
+  W.nh = std::max(0, n - 2 - W.lb);
+  W.f.last = half ? B[n][k] - 1 : 0;
+  int start = 0;
+  for (int kl = 0; kl <= W.lb; ++kl) {
+    const int rows = (int)B[W.lb][kl], kh = k - 1 - kl;
+    if (kh >= 0 && kh <= W.nh) {
+      Closing::Cls& C = W.cls[W.ncls++];
+      C.kl = kl;
+      C.rows = rows;
+      C.start = start;
+      C.ncols = B[W.nh][kh];
+      C.half_cols = half ? B[W.nh - 1][kh] : 0;
+      C.m = std::max(1, std::min(kCloseCols, kClosePairs / rows));
+      C.first_tile = W.tiles;
+      C.half_first = W.half_tiles;
+      W.tiles += (C.ncols + C.m - 1) / C.m;
+      W.half_tiles += (C.half_cols + C.m - 1) / C.m;
+      W.pairs += C.ncols * (u64)rows;
+      W.half_pairs += C.half_cols * (u64)rows;
+    }
+    start += rows;
+  }
+  return W;
 }
 
 }  // namespace xyw
