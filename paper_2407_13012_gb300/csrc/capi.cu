@@ -272,7 +272,7 @@ static int run_sweeps(const Ctx& c, std::vector<Sweep>& sw, const std::vector<Gr
   const int nscan = half || (fx && any_two) ? cost_scan_blocks(c.n) : 0;
   const bool scan_now = nscan > 0 && !c.bound_ready;
   // the tables ride on a scan of enough blocks: they are float64 work, which few SMs would serialise
-  const bool ride = scan_now && nscan >= 64;
+  const bool ride = scan_now && nscan >= 32;
   if (nscan > 0) {
     static_assert(kMaxScan * sizeof(unsigned long long) <= kNormPartialBytes, "the scan takes the norm partials' place");
     if (any_user_load) return QAOA_ERR_UNSUPPORTED;  // (no plan has both)

@@ -442,7 +442,7 @@ cudaError_t launch_tables(const TableArgs& t, cudaStream_t s) {
 }
 
 int cost_scan_blocks(int n) {
-  const int64_t blocks = ((1ll << n) + 8191) / 8192;
+  const int64_t blocks = ((1ll << n) + 16383) / 16384;
   return (int)std::min<int64_t>({blocks, (int64_t)num_sms(), (int64_t)kMaxScan});
 }
 

@@ -114,8 +114,8 @@ __device__ __forceinline__ uint64_t tile_base(const SweepGeom& g, int64_t tile) 
   const uint64_t highrest = (uint64_t)tile >> lowrest_bits;
   return (lowrest << g.c) | (highrest << (g.j0 + g.t - g.pair));
 }
-// What a scan of C says, read by each warp for itself: whether C(z) = C(~z), and the smallest k >= 0
-// with 2^k >= max |C|.
+// What a scan of C says, read by each warp for itself (a single entry by each thread): whether
+// C(z) = C(~z), and the smallest k >= 0 with 2^k >= max |C|.
 struct CostScan {
   bool symmetric;
   int shift;
@@ -123,12 +123,16 @@ struct CostScan {
 __device__ __forceinline__ CostScan read_scan(const unsigned long long* scan, int nscan) {
   bool asym = false;
   int k = 0;
-  for (int i = threadIdx.x & 31; i < nscan; i += 32) {
-    const unsigned long long b = scan[i];
+  auto take = [&](unsigned long long b) {
     const int ex = (int)(b >> 52) & 0x7FF;
     asym |= (b >> 63) != 0;
     if (ex != 0) k = max(k, ex - 1023 + ((b & ((1ull << 52) - 1)) != 0 ? 1 : 0));
+  };
+  if (nscan == 1) {
+    take(scan[0]);
+    return {!asym, k};
   }
+  for (int i = threadIdx.x & 31; i < nscan; i += 32) take(scan[i]);
   return {!__any_sync(0xffffffffu, asym), __reduce_max_sync(0xffffffffu, k)};
 }
 
