@@ -94,7 +94,9 @@ __device__ __forceinline__ T warp_sum8(T (&x)[8], ADD&& add) {
 // (1) one warp per leaf; a.len entries (the last leaf may be partly past the end).  Full
 // leaves of an aligned vector take 16-byte loads, all issued before the sums (complex128:
 // one amplitude per load, two independent float64 FMA chains; complex64: two amplitudes
-// per load, double-float sums in float32); other leaves go amplitude by amplitude.
+// per load, double-float sums in float32); other leaves go amplitude by amplitude.  SUBS: with the
+// running sums at the eighths.
+template <bool SUBS>
 __global__ void leaf_sum_kernel(const __grid_constant__ SampleArgs a) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -122,10 +124,12 @@ __global__ void leaf_sum_kernel(const __grid_constant__ SampleArgs a) {
           }
         }
         s = run[kSubs - 1];
-        const double t = warp_sum8(run, [](double keep, double give, int o) {
-          return keep + __shfl_xor_sync(0xffffffffu, give, o);
-        });
-        if ((lane & 3) == 0) a.sub[li * kSubs + (lane >> 2)] = t;
+        if constexpr (SUBS) {
+          const double t = warp_sum8(run, [](double keep, double give, int o) {
+            return keep + __shfl_xor_sync(0xffffffffu, give, o);
+          });
+          if ((lane & 3) == 0) a.sub[li * kSubs + (lane >> 2)] = t;
+        }
       } else {
         const float4* q = (const float4*)a.psi + (base >> 1) + lane;
         F2Sum f0, f1;
@@ -141,7 +145,7 @@ __global__ void leaf_sum_kernel(const __grid_constant__ SampleArgs a) {
             f1.add_sq(v[m].y);
             f0.add_sq(v[m].z);
             f1.add_sq(v[m].w);
-            if (m & 1) {
+            if (SUBS && (m & 1)) {
               float2& x = run[(m0 + m) >> 1];
               two_sum(f0.s, f1.s, x.x, x.y);
               x.y += f0.c + f1.c;
@@ -149,14 +153,16 @@ __global__ void leaf_sum_kernel(const __grid_constant__ SampleArgs a) {
           }
         }
         s = f0.value() + f1.value();
-        const float2 t = warp_sum8(run, [](float2 keep, float2 give, int o) {
-          const float gx = __shfl_xor_sync(0xffffffffu, give.x, o), gy = __shfl_xor_sync(0xffffffffu, give.y, o);
-          float2 r;
-          two_sum(keep.x, gx, r.x, r.y);
-          r.y += keep.y + gy;
-          return r;
-        });
-        if ((lane & 3) == 0) a.sub[li * kSubs + (lane >> 2)] = (double)t.x + (double)t.y;
+        if constexpr (SUBS) {
+          const float2 t = warp_sum8(run, [](float2 keep, float2 give, int o) {
+            const float gx = __shfl_xor_sync(0xffffffffu, give.x, o), gy = __shfl_xor_sync(0xffffffffu, give.y, o);
+            float2 r;
+            two_sum(keep.x, gx, r.x, r.y);
+            r.y += keep.y + gy;
+            return r;
+          });
+          if ((lane & 3) == 0) a.sub[li * kSubs + (lane >> 2)] = (double)t.x + (double)t.y;
+        }
       }
     } else {
       for (uint32_t k = lane; k < L && base + k < a.len; k += 32) s += prob_at(a.psi, a.dtype, base + k);
@@ -197,7 +203,11 @@ __global__ void chunk_scan_kernel(double* bsum, int64_t nchunks) {
   }
 }
 
-// (2c) exclusive scan inside each chunk; prefix[nleaf] = total
+// (2c) exclusive scan inside each chunk; prefix[nleaf] = total.  ONE: the only chunk, whose total it
+// forms itself, in chunk_sum_kernel's order (up to 2^22 amplitudes; two launches fewer, and the serial
+// scan below ends with the threads that hold leaves: n = 10, p = 2 evaluation with 4096 samples
+// 95 -> 80 us back to back).
+template <bool ONE>
 __global__ void leaf_scan_kernel(const double* __restrict__ leaf, int64_t nleaf, const double* __restrict__ bsum,
                                  double* __restrict__ prefix, int64_t nchunks) {
   __shared__ double sh[kThreads];
@@ -208,23 +218,37 @@ __global__ void leaf_scan_kernel(const double* __restrict__ leaf, int64_t nleaf,
     v[k] = (base + k < nleaf) ? leaf[base + k] : 0.0;
     s += v[k];
   }
+  double total = 0.0;
+  if constexpr (ONE) {
+    sh[threadIdx.x] = s;
+    __syncthreads();
+    for (int st = kThreads / 2; st > 0; st >>= 1) {
+      if ((int)threadIdx.x < st) sh[threadIdx.x] += sh[threadIdx.x + st];
+      __syncthreads();
+    }
+    total = sh[0];
+    __syncthreads();
+  }
   sh[threadIdx.x] = s;
   __syncthreads();
-  if (threadIdx.x == 0) {  // sequential exclusive scan of 256 thread totals
+  if (threadIdx.x == 0) {  // sequential exclusive scan of the thread totals
     double run = 0.0;
-    for (int t = 0; t < kThreads; ++t) {
+    const int64_t held = (nleaf - base + 15) / 16;
+    const int live = held < kThreads ? (int)held : kThreads;
+#pragma unroll 8
+    for (int t = 0; t < live; ++t) {
       const double x = sh[t];
       sh[t] = run;
       run += x;
     }
   }
   __syncthreads();
-  double run = bsum[blockIdx.x] + sh[threadIdx.x];
+  double run = (ONE ? 0.0 : bsum[blockIdx.x]) + sh[threadIdx.x];
   for (int k = 0; k < 16; ++k) {
     if (base + k < nleaf) prefix[base + k] = run;
     run += v[k];
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) prefix[nleaf] = bsum[nchunks];
+  if (blockIdx.x == 0 && threadIdx.x == 0) prefix[nleaf] = ONE ? total : bsum[nchunks];
 }
 
 // |psi_z|^2 in float32, to 2^-21 relative: complex128 components enter by their bits (truncated;
@@ -319,7 +343,7 @@ __global__ void draw_kernel(const __grid_constant__ SampleArgs a, const double* 
     double run = 0.0;
     uint32_t k1 = 0;  // first entry of the eighth that holds the target (0 without running sums)
     int64_t found = -1, last_nz = -1;
-    if (vec && !past_end && Lh == L) {
+    if (vec && a.sub != nullptr && !past_end && Lh == L) {
       const double r = lane < kSubs ? __ldg(a.sub + li * kSubs + lane) : 0.0;
       const unsigned le = __ballot_sync(0xffffffffu, lane < kSubs - 1 && r <= rem);
       const int j = 32 - __clz(le);  // eighths whose end the target has passed
@@ -394,6 +418,10 @@ cudaError_t launch_sample(const SampleArgs& a0, cudaStream_t s) {
   double* prefix = (double*)carve((nleaf + 1) * sizeof(double));
   double* bsum = (double*)carve((nchunks + 1) * sizeof(double));
   a.sub = (double*)carve((a.leaf_bits == 10 ? kSubs * nleaf : 0) * sizeof(double));
+  // few shots of a large state: the eighths take longer to sum and store than they save (n = 28, 1000
+  // shots: 1290 instead of 1073 us complex128, whose leaf sums are bound by the float64 pipe, 401 instead of
+  // 396 complex64; a shot that scans its leaf costs ~14 ns)
+  if (a.shots < nleaf / (a.dtype == QAOA_C64 ? 256 : 16)) a.sub = nullptr;
   a.leaf = leaf;
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
@@ -404,20 +432,27 @@ cudaError_t launch_sample(const SampleArgs& a0, cudaStream_t s) {
     const int64_t warps = nleaf;
     int64_t blocks = (warps * 32 + kThreads - 1) / kThreads;
     if (blocks > (int64_t)sms * 16) blocks = (int64_t)sms * 16;
-    leaf_sum_kernel<<<(int)blocks, kThreads, 0, s>>>(a);
+    if (a.sub != nullptr) leaf_sum_kernel<true><<<(int)blocks, kThreads, 0, s>>>(a);
+    else leaf_sum_kernel<false><<<(int)blocks, kThreads, 0, s>>>(a);
   }
   note_launch(2, s, false, (double)a.len * (a.dtype == QAOA_C128 ? 16.0 : 8.0));
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  note_launch(3, s, true);
-  chunk_sum_kernel<<<(int)nchunks, kThreads, 0, s>>>(leaf, nleaf, bsum);
-  note_launch(3, s, false);
-  note_launch(3, s, true);
-  chunk_scan_kernel<<<1, 32, 0, s>>>(bsum, nchunks);
-  note_launch(3, s, false);
-  note_launch(3, s, true);
-  leaf_scan_kernel<<<(int)nchunks, kThreads, 0, s>>>(leaf, nleaf, bsum, prefix, nchunks);
-  note_launch(3, s, false);
+  if (nchunks == 1) {
+    note_launch(3, s, true);
+    leaf_scan_kernel<true><<<1, kThreads, 0, s>>>(leaf, nleaf, bsum, prefix, nchunks);
+    note_launch(3, s, false);
+  } else {
+    note_launch(3, s, true);
+    chunk_sum_kernel<<<(int)nchunks, kThreads, 0, s>>>(leaf, nleaf, bsum);
+    note_launch(3, s, false);
+    note_launch(3, s, true);
+    chunk_scan_kernel<<<1, 32, 0, s>>>(bsum, nchunks);
+    note_launch(3, s, false);
+    note_launch(3, s, true);
+    leaf_scan_kernel<false><<<(int)nchunks, kThreads, 0, s>>>(leaf, nleaf, bsum, prefix, nchunks);
+    note_launch(3, s, false);
+  }
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (a.shots > 0) {
