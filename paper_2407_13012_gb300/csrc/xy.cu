@@ -841,7 +841,8 @@ __global__ void __launch_bounds__(kXYThreads) xy_grad_reduce_kernel(const __grid
 template <typename T>
 __global__ void __launch_bounds__(kXYThreads)
     xy_expect_kernel(const T* __restrict__ psi, const void* __restrict__ C, int cost_dtype, unsigned long long D,
-                     double* __restrict__ part) {
+                     double* __restrict__ part, const unsigned* half_flag) {
+  if (half_flag != nullptr && *half_flag == 0) D >>= 1;
   __shared__ double se[kXYThreads], sn[kXYThreads];
   double e = 0.0, nn = 0.0;
   if (std::is_same<T, float2>::value && cost_dtype == QAOA_COST_I32) {
@@ -891,7 +892,8 @@ __global__ void __launch_bounds__(kXYThreads)
 }
 
 __global__ void __launch_bounds__(kXYThreads) xy_finish_kernel(const double* __restrict__ part, int nb,
-                                                               double* __restrict__ out) {
+                                                               double* __restrict__ out, const unsigned* half_flag) {
+  const double scale = half_flag != nullptr && *half_flag == 0 ? 2.0 : 1.0;
   __shared__ double se[kXYThreads], sn[kXYThreads];
   double e = 0.0, nn = 0.0;
   for (int b = threadIdx.x; b < nb; b += kXYThreads) {
@@ -909,8 +911,8 @@ __global__ void __launch_bounds__(kXYThreads) xy_finish_kernel(const double* __r
     __syncthreads();
   }
   if (threadIdx.x == 0) {
-    out[0] = se[0];
-    out[1] = sn[0];
+    out[0] = scale * se[0];
+    out[1] = scale * sn[0];
   }
 }
 
@@ -1027,14 +1029,14 @@ bool cost_ok(const qaoa_cost_t* c) {
 
 template <typename T>
 int expectation_t(const XYShape& s, const T* psi, const qaoa_cost_t* cost, double* out, double* part,
-                  cudaStream_t st) {
-  const int nb = (int)(s.D < (unsigned long long)kXYRedBlocks * kXYThreads ? (s.D + kXYThreads - 1) / kXYThreads
-                                                                         : kXYRedBlocks);
+                  cudaStream_t st, const unsigned* half_flag = nullptr) {
+  const int most = kXYRedBlocks - (half_flag != nullptr);  // (the flag lies in the last block's slots)
+  const int nb = (int)(s.D < (unsigned long long)most * kXYThreads ? (s.D + kXYThreads - 1) / kXYThreads : most);
   note_launch(3, st, true);
-  xy_expect_kernel<T><<<nb, kXYThreads, 0, st>>>(psi, cost->C_dev, cost->dtype, s.D, part);
+  xy_expect_kernel<T><<<nb, kXYThreads, 0, st>>>(psi, cost->C_dev, cost->dtype, s.D, part, half_flag);
   note_launch(3, st, false, (double)s.D * (sizeof(T) + cost_bytes(cost->dtype)));
   note_launch(3, st, true);
-  xy_finish_kernel<<<1, kXYThreads, 0, st>>>(part, nb, out);
+  xy_finish_kernel<<<1, kXYThreads, 0, st>>>(part, nb, out, half_flag);
   note_launch(3, st, false);
   return status_of(cudaGetLastError());
 }
@@ -1055,6 +1057,8 @@ struct XYMixPlan {
 // is not symmetric pays for the read of C and the launches that return at once: n = 26, p = 1 layers 1057 ->
 // 1077 us complex128, 400 -> 431 complex64, n = 28 4033 -> 4070 and 1647 -> 1695; below n = 26 that share grows.
 constexpr int kXYHalfMinN = 26;
+// (the last slot of the expectation's partials, which half calls leave alone)
+unsigned* half_flag_at(char* ws) { return (unsigned*)((double*)ws + 2 * kXYRedBlocks - 1); }
 bool half_plan(const XYShape& s, int p, int init) {
   return init && p > 0 && s.n >= kXYHalfMinN && s.n % 2 == 0 && s.k == s.n / 2;
 }
@@ -1148,7 +1152,7 @@ int layers_t(const XYShape& s, T* psi, const qaoa_cost_t* cost, const double* ga
   const long long span = p > 0 ? table_span(cost) : 0;
   T* tab = span > 0 ? (T*)(ws + round256(2 * (size_t)kXYRedBlocks * sizeof(double))) : nullptr;
   const bool half = half_plan(s, p, init);
-  unsigned* flag = half ? (unsigned*)part : nullptr;  // (in the partials' place: they are written after its last use)
+  unsigned* flag = half ? half_flag_at(ws) : nullptr;
   if (half) {
     note_launch(3, st, true);
     cudaMemsetAsync(flag, 0, sizeof(unsigned), st);
@@ -1216,7 +1220,7 @@ int layers_t(const XYShape& s, T* psi, const qaoa_cost_t* cost, const double* ga
     xy_mirror_kernel<T><<<(unsigned)sms * 8, kXYThreads, 0, st>>>(psi, s.D, flag);
     note_launch(3, st, false, (double)s.D * sb);
   }
-  if (expect_dev != nullptr) return expectation_t<T>(s, psi, cost, expect_dev, part, st);
+  if (expect_dev != nullptr) return expectation_t<T>(s, psi, cost, expect_dev, part, st, flag);
   return status_of(cudaGetLastError());
 }
 
@@ -1246,7 +1250,7 @@ int gradient_t(const XYShape& s, T* psi, T* lam, const qaoa_cost_t* cost, const 
   const unsigned long long nch = (s.D + kXYChunk - 1) / kXYChunk;
   const unsigned gg = std::min<unsigned>(grid_for(nch, sms), kXYPartStride);
   const bool half = half_plan(s, p, 1);
-  const unsigned* flag = half ? (const unsigned*)ws : nullptr;  // set by the forward pass
+  const unsigned* flag = half ? half_flag_at(ws) : nullptr;  // set by the forward pass
   note_launch(0, st, true);
   xy_lambda_kernel<T><<<gr, kXYThreads, 0, st>>>(psi, lam, cost->C_dev, cost->dtype, s.D, part, part + kXYPartStride,
                                                  flag);
