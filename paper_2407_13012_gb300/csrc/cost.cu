@@ -21,7 +21,9 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kMaxLowBits = 12;
 
-// A block stages the weights in shared memory, builds the low-low table A and the sums
+// A block stages the weights in shared memory, builds the low-low table A (itself from tables of the two
+// six-bit halves of x and of the edges between them: with the 66 pairs summed for each of 4096 entries an
+// n = 14 vector took 38 us, with the tables 7.7) and the sums
 // b_v = sum_{u < L} w_uv of every high vertex once, then per high part h: a_u(h) for the L
 // low vertices, K(h) by one warp (a lane per high vertex), and sum_u x_u a_u(h) as two
 // 64-entry tables over the low six and the next six low bits; an element is then four
@@ -32,16 +34,39 @@ __global__ void __launch_bounds__(kThreads) cost_kernel(const __grid_constant__ 
   __shared__ long long bsum[QAOA_MAX_N];
   __shared__ long long au[kMaxLowBits];
   __shared__ long long S0[64], S1[64];
+  __shared__ long long T[8 * 64];  // edges inside x's low half; inside its high half and x_v w of edges down; a_u
   __shared__ long long Kh;
   const int n = a.n, L = a.lo_bits, tid = threadIdx.x;
   const uint32_t X = 1u << L;
-  for (int i = tid; i < n * n; i += kThreads) W[i / n][i % n] = a.wi[i / n][i % n];
+  for (int i = tid; i < QAOA_MAX_N * QAOA_MAX_N; i += kThreads) {
+    const int u = i / QAOA_MAX_N, v = i % QAOA_MAX_N;
+    W[u][v] = u < n && v < n ? a.wi[u][v] : 0;
+  }
+  __syncthreads();
+  auto w = [&](int u, int v) { return v < L ? W[u][v] : 0ll; };  // u < v
+  for (int i = tid; i < 8 * 64; i += kThreads) {
+    const int y = i & 63, row = i >> 6;
+    long long s = 0;
+    if (row < 2) {
+      const int b0 = 6 * row;
+      for (int u = 0; u < 6; ++u)
+        for (int v = u + 1; v < 6; ++v)
+          if (((y >> u) ^ (y >> v)) & 1) s += w(b0 + u, b0 + v);
+      if (row == 1)
+        for (int v = 0; v < 6; ++v)
+          if ((y >> v) & 1)
+            for (int u = 0; u < 6; ++u) s += w(u, 6 + v);
+    } else {
+      for (int v = 0; v < 6; ++v) s += (y >> v) & 1 ? -w(row - 2, 6 + v) : w(row - 2, 6 + v);
+    }
+    T[i] = s;
+  }
   __syncthreads();
   for (uint32_t x = tid; x < X; x += kThreads) {  // low-low table
-    long long s = 0;
-    for (int u = 0; u < L; ++u)
-      for (int v = u + 1; v < L; ++v)
-        if (((x >> u) ^ (x >> v)) & 1) s += W[u][v];
+    const uint32_t y = x >> 6;
+    long long s = T[x & 63] + T[64 + y];
+#pragma unroll
+    for (int u = 0; u < 6; ++u) s += (x >> u) & 1 ? T[128 + 64 * u + y] : 0ll;
     A[x] = s;
   }
   for (int v = L + tid; v < n; v += kThreads) {
