@@ -195,7 +195,7 @@ def measured_peak_hbm():
         return 6800.0, "fallback"
 
 
-SWEEP_SOURCES = ("sweep.cu", "sweeper.cuh", "tile_layout.cuh", "fixedpoint.cuh", "internal.h", "capi.cu")
+SWEEP_SOURCES = ("sweep.cu", "sweeper.cuh", "lean_kernel.cuh", "tile_layout.cuh", "fixedpoint.cuh", "internal.h", "capi.cu")
 
 
 def sweep_source_hash() -> str:
@@ -650,11 +650,12 @@ def run_ours(a):
     if tr is not None:
         traffic = tr.get("bytes_per_launch")
     # the method's least HBM traffic for the step's 3p layers: a forward layer reads and
-    # writes psi once and reads C, (2S + c) 2^n bytes; an adjoint layer does so for psi and
-    # lambda, (4S + c) 2^n (S, c: bytes per amplitude and per cost entry)
+    # writes psi once and reads C, (2S + c) bytes per amplitude; an adjoint layer does so for psi
+    # and lambda, 4S + c (S, c: bytes per amplitude and per cost entry); a cut is symmetric under
+    # flipping every qubit, so 2^(n - 1) amplitudes carry the state
     S_b = 16 if a.dtype == "c128" else 8
     c_b = 4 if integer else 8
-    min_bytes = float(2 ** a.n) * (2 * a.p * (2 * S_b + c_b) + a.p * (4 * S_b + c_b))
+    min_bytes = float(2 ** (a.n - 1)) * (2 * a.p * (2 * S_b + c_b) + a.p * (4 * S_b + c_b))
     min_gbs = min_bytes / (step_ms / 1e3) / 1e9
 
     if rank == 0:

@@ -181,7 +181,10 @@ int qaoa_cost_vector(const qaoa_graph_t* g, void* C_dev, int cost_dtype, qaoa_co
  * for l = 0..p-1: psi_z *= exp(-i gamma[l] C(z)), then RX(2 beta[l]) on every
  * qubit.  init = 1 starts from |+>^n (psi_dev is write-only then); init = 0
  * continues from the state in psi_dev.  gamma/beta are host arrays of p
- * doubles.  p = 0 with init = 1 just writes |+>^n.
+ * doubles.  p = 0 with init = 1 just writes |+>^n.  Calls from |+>^n (these, the
+ * gradients and the optimisers) read C once to see whether C(z) = C(~z) for
+ * all z (every cut); if so, larger n sweep half the state and store the other
+ * half from it.
  *  expect_dev: optional (may be NULL) device double[2] receiving
  *    [<C>, <psi|psi>] of the final state, fused into the last sweep.
  */
@@ -375,7 +378,8 @@ void qaoa_launch_count_reset(void);
  * events and writes, per class (arrays of 4, any may be NULL), the summed
  * milliseconds, the launch count and the algorithmic HBM bytes of those
  * launches (each state, lambda and cost-vector element read or written once
- * per launch), then clears them.  At most 65536 launches are recorded between
+ * per launch; half of them where a call may sweep half a state, which the
+ * device decides), then clears them.  At most 65536 launches are recorded between
  * reads; later ones are counted in *dropped but not timed.
  */
 int qaoa_timing_enable(int on);
