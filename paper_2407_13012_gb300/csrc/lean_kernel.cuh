@@ -167,6 +167,7 @@ __global__ void __launch_bounds__(CF::NT, CF::MINB) lean_kernel(const __grid_con
     s.Ps = (V*)(smem_raw + ((off + 15) & ~(size_t)15));
   }
   s.evalid = 1u << CF::B;
+  if constexpr (FX && !TWO) s.in_shift = input_shift(a.norm2_dev);
   if constexpr (FX && TWO) {
     if (a.gslot != nullptr) {
       s.lam_shift = a.gslot[blockIdx.x / a.gbpg].lam_shift;

@@ -30,11 +30,7 @@ __global__ void __launch_bounds__(CF::NT, CF::MINB) sweep_kernel(const __grid_co
   s.evalid = 1u << (g.t + g.c);
   if constexpr (FX) {
     if (a.scan != nullptr) s.lam_shift = read_scan(a.scan, a.nscan).shift;
-    if (a.norm2_dev != nullptr) {  // 2^k with |psi| / 2^k in [1, 2)
-      const unsigned long long b = (unsigned long long)__double_as_longlong(*a.norm2_dev);
-      const int ex = (int)((b >> 52) & 0x7FF);
-      s.in_shift = ex == 0 ? 0 : ((ex - 1023) >= 0 ? (ex - 1023) / 2 : -((1023 - ex + 1) / 2));
-    }
+    s.in_shift = input_shift(a.norm2_dev);
   }
   for (int64_t tile = blockIdx.x; tile < g.tiles; tile += gridDim.x) sweep_tile<CF, FX, TWO, false>(s, a, tile, Cs);
 

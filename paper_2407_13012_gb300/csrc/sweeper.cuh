@@ -136,6 +136,16 @@ __device__ __forceinline__ CostScan read_scan(const unsigned long long* scan, in
   return {!__any_sync(0xffffffffu, asym), __reduce_max_sync(0xffffffffu, k)};
 }
 
+// The scale of a user state (complex128): k with |psi| / 2^k in [1, 2), from its norm^2.  The first
+// sweep loads psi / 2^k; every sweep that gives out values of psi (its last store, <C> and the
+// norm) multiplies by 2^k again.
+__device__ __forceinline__ int input_shift(const double* norm2) {
+  if (norm2 == nullptr) return 0;
+  const unsigned long long b = (unsigned long long)__double_as_longlong(*norm2);
+  const int ex = (int)((b >> 52) & 0x7FF);
+  return ex == 0 ? 0 : ((ex - 1023) >= 0 ? (ex - 1023) / 2 : -((1023 - ex + 1) / 2));
+}
+
 // the sweep's geometry on a half state
 __device__ __forceinline__ SweepGeom half_geom(SweepGeom g) {
   g.n -= 1;
@@ -1505,7 +1515,8 @@ __device__ __forceinline__ void lean_tile(Lean<CF, FX, TWO, C>& s, const SweepAr
       if (st_fmt == 0) {
         ((V*)a.psi)[z] = v[r];
       } else if (st_fmt == 1) {
-        const double2 d = make_double2(fx_to_double(v[r].x, a.fx_shift), fx_to_double(v[r].y, a.fx_shift));
+        const int sh = a.fx_shift - s.in_shift;
+        const double2 d = make_double2(fx_to_double(v[r].x, sh), fx_to_double(v[r].y, sh));
         ((double2*)a.psi)[z] = d;
         if (mirror) ((double2*)a.psi)[zc - z] = d;
       }
