@@ -536,7 +536,9 @@ int qaoa_xy_gradient_workspace_size(int n, int k, int dtype, int p, int64_t cost
  * caller-owned), then walks the gates backwards, undoing each on both buffers
  * after taking its term.  out_dev (device, 2p + 2 doubles): [E, <psi|psi>,
  * dE/dgamma_1..p, dE/dbeta_1..p]; psi_dev ends back at the Dicke state (up to
- * rounding).  Every sum is float64 with a fixed order.  Errors as for
+ * rounding).  Every sum has a fixed order: E and the norm are float64; the other
+ * terms are exact 128-bit sums per tile (QAOA_C128) or exact float32 products in
+ * double-float sums per thread (QAOA_C64), added up in float64.  Errors as for
  * qaoa_xy_apply_layers, QAOA_ERR_WORKSPACE below
  * qaoa_xy_gradient_workspace_size.
  */

@@ -224,8 +224,10 @@ __global__ void __launch_bounds__(kXYThreads) xy_unrank_kernel(const __grid_cons
 // gate g and lambda_g = (gates after g)^dagger C psi_final, dE/dtheta_g = 2 Im <lambda_g|H_g|psi_g>
 // (Sec. II-B, IV-C); a parameter's derivative is the sum over its gates.  The pass walks the
 // gates backwards from lambda = C psi_final, undoing each on psi and lambda after taking its
-// term, so it needs the two subspace buffers only.  Every term is summed in float64 per
-// thread and per block, one partial per block in a fixed grid (deterministic).
+// term, so it needs the two subspace buffers only.  E and the norm are summed in float64 from
+// float64 terms; the gate and gamma terms are exact 128-bit sums per tile (complex128) or exact
+// float32 products in double-float sums per thread (complex64, Acc); the rest of every sum is
+// float64, one partial per block in a fixed grid (deterministic).
 
 __device__ __forceinline__ double block_sum(double v, double* red) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -238,9 +240,10 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
 }
 
 // Sums of products of a state's components.  Float32 states: the exact product (as a product
-// and its FMA residual) into a double-float sum, ~2^-44 relative, all on the float32 pipe: a
-// float64 product and sum per term (with its conversions) takes GB300's float64 pipe, two lanes
-// per SM and clock, a dozen times as long as the rest of a subspace gate.
+// and its FMA residual) into a double-float sum, all on the float32 pipe: a float64 product and sum
+// per term (with its conversions) takes GB300's float64 pipe, two lanes per SM and clock, a dozen
+// times as long as the rest of a subspace gate.  Relative error of a thread's sum of 34 squares 8e-15
+// (rms); the terms themselves carry the float32 state's 1e-8 to 1e-9.
 template <typename T>
 struct Acc {
   double s = 0.0;
@@ -258,6 +261,15 @@ struct Acc<float2> {
     s = t;
   }
   __device__ __forceinline__ void sub(float a, float b) { add(-a, b); }
+  // + c Im(conj(l) v) for a c exact in float32: l.x v.y - l.y v.x as a sum of two floats, then times c
+  __device__ __forceinline__ void add_im(float c_, float2 l, float2 v) {
+    const float p = __fmul_rn(l.x, v.y), q = __fmul_rn(l.y, v.x);
+    const float pe = __fmaf_rn(l.x, v.y, -p), qe = __fmaf_rn(l.y, v.x, -q);
+    const float h = __fsub_rn(p, q), bq = __fsub_rn(h, p);
+    const float e = __fsub_rn(__fsub_rn(p, __fsub_rn(h, bq)), __fadd_rn(q, bq));
+    add(c_, h);
+    c = __fmaf_rn(c_, __fadd_rn(e, __fsub_rn(pe, qe)), c);
+  }
   __device__ __forceinline__ double value() const { return (double)s + (double)c; }
 };
 
@@ -270,22 +282,25 @@ __global__ void __launch_bounds__(kXYThreads)
   if (half_flag != nullptr && *half_flag == 0) D >>= 1;
   __shared__ double red[kXYThreads / 32];
   using R = typename Real<T>::type;
-  Acc<T> e, nn;
+  // float64 throughout, also for float32 states: this kernel runs once per gradient.  In double-float,
+  // with C and |psi|^2 rounded to float32, E was off its own state's by 1e-9 sum|w| (n = 12) to
+  // 1e-11 (n = 26) instead of 1e-16, and the norm by 3e-15
+  double e = 0.0, nn = 0.0;
   for (unsigned long long r = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; r < D;
        r += (unsigned long long)gridDim.x * blockDim.x) {
     const T x = psi[r];
-    const R c = cost_dtype == QAOA_COST_I32 ? (R)((const int*)C)[r] : (R)((const double*)C)[r];
+    const double c = cost_dtype == QAOA_COST_I32 ? (double)((const int*)C)[r] : ((const double*)C)[r];
     T y;
-    y.x = c * x.x;
-    y.y = c * x.y;
+    y.x = (R)c * x.x;
+    y.y = (R)c * x.y;
     lam[r] = y;
-    e.add(c, x.x * x.x + x.y * x.y);
-    nn.add(x.x, x.x);
-    nn.add(x.y, x.y);
+    const double pr = (double)x.x * (double)x.x + (double)x.y * (double)x.y;
+    e += c * pr;
+    nn += pr;
   }
-  const double se = block_sum(e.value(), red);
+  const double se = block_sum(e, red);
   __syncthreads();
-  const double sn = block_sum(nn.value(), red);
+  const double sn = block_sum(nn, red);
   if (threadIdx.x == 0) {
     pe[blockIdx.x] = se;
     pn[blockIdx.x] = sn;
@@ -779,8 +794,7 @@ __global__ void __launch_bounds__(xy_window_threads(TWO), TWO ? 2 : 4)
         } else {
           T f = xy_phase_factor(ph, cf, cI);
           if (ph.cost_dtype == QAOA_COST_I32 && abs((long long)cI) <= (1 << 24)) {  // c exact in float32
-            cacc.add((float)cI * L.x, X.y);
-            cacc.sub((float)cI * L.y, X.x);
+            cacc.add_im((float)cI, L, X);
           } else {
             const double cv = ph.cost_dtype == QAOA_COST_I32 ? (double)cI : cf;
             cacc_d += cv * ((double)L.x * X.y - (double)L.y * X.x);
