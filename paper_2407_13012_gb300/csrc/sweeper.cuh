@@ -188,9 +188,8 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
 // fraction of the turn comes from the integer bits (its float64 rounding, subtraction and
 // conversion took the float64 pipe three times as long as the product that th is).
 __device__ __noinline__ float2 phase_f32_direct(double th) {
-  const int f = (int)(unsigned)(frac_turns(th) >> 32);  // signed: the turn in [-1/2, 1/2) x 2^32
   float s, c;
-  sincospif((float)f * 0x1.0p-31f, &s, &c);
+  sincospif(fx::two_turns_f32(th), &s, &c);
   if (((unsigned)__double2hiint(th) & 0x7ff00000u) == 0x7ff00000u) s = c = __int_as_float(0x7fffffff);  // no phase
   return make_float2(c, -s);
 }
