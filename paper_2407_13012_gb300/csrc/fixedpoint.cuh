@@ -266,20 +266,29 @@ QAOA_HD long long mul_unit(long long x, Limbs c) {
   return madw(a.h, c.h, madw(a.l, c.h, madw(a.h, c.l, 1ll << 31)) >> 32);
 }
 
-// Running sums of Im(conj(w) v) = w.x v.y - w.y v.x by limb weight: value = P 2^64 + M 2^32 +
-// L 2^4.  One multiply-add-wide per limb product and no carries between products (an exact
-// 128-bit product and sum per term took ~80 instructions per amplitude, this ~15); the four
-// lowest bits of w are left out of the low x low products only (2^-73 of a unit product).
+// Low x low part of w.x v.y - w.y v.x: its high word (rounded down) and its low word.  Limbs lie in
+// [-2^31, 2^31), so the difference of the two products fits 64 bits.
+QAOA_HD long long low_diff(Limbs vx, Limbs vy, Limbs wx, Limbs wy) {
+  return madw(wx.l, vy.l, 0) - madw(wy.l, vx.l, 0);
+}
+
+// Running sums of Im(conj(w) v) = w.x v.y - w.y v.x by limb weight, exact: value = P 2^64 + M 2^32 + L,
+// one multiply-add-wide per limb product and few carries (an exact 128-bit product and sum per term
+// took ~80 instructions per amplitude, this ~17).  Leaving the four lowest bits of w out of the low x
+// low products saved two of them, but those bits are all of w where amplitudes are small: the n = 20
+// gradient of costs of 1e-6 was off by 8e-9 instead of 1e-10.
 // Sums of up to 8 terms with weights 0..3 fit int64 when the 2-norms of w and of v over the
 // terms are at most 1.1 x 2^60: |h| norms are then at most 1.1 x 2^28 and each of M's two
 // halves at most that x 2^31 sqrt(2 sum of squared weights <= 48) < 2^62.
 struct ImSum {
   unsigned long long P = 0, M = 0, L = 0;
   QAOA_HD void add(Limbs vx, Limbs vy, Limbs wx, Limbs wy) {
-    const int nwyh = -wy.h, nvxh = -vx.h, wxl = wx.l >> 4, nwyl = -(wy.l >> 4);
+    const int nwyh = -wy.h, nvxh = -vx.h;
+    const long long d = low_diff(vx, vy, wx, wy);
     P = (unsigned long long)madw(nwyh, vx.h, madw(wx.h, vy.h, (long long)P));
     M = (unsigned long long)madw(wy.l, nvxh, madw(nwyh, vx.l, madw(wx.l, vy.h, madw(wx.h, vy.l, (long long)M))));
-    L = (unsigned long long)madw(nwyl, vx.l, madw(wxl, vy.l, (long long)L));
+    M += (unsigned long long)(d >> 32);
+    L += (unsigned)d;
   }
   // this += m s for a small m (modulo 2^64: intermediate sums may wrap)
   QAOA_HD void add_times(const ImSum& s, int m) {
@@ -289,20 +298,21 @@ struct ImSum {
     L += s.L * (unsigned long long)(long long)m;
   }
   QAOA_HD i128 value() const {
-    return ((i128)(long long)P << 64) + ((i128)(long long)M << 32) + ((i128)(long long)L << 4);
+    return ((i128)(long long)P << 64) + ((i128)(long long)M << 32) + (i128)(long long)L;
   }
 };
 
-// sum of c Im(conj(w) v) for integer c, |c| <= 2^28, and |components| < 2^56 (up to 8 terms):
-// the term is P 2^64 + Q 2^32 with the low products folded into Q, and each word of P and Q is
-// weighted by c with one multiply-add-wide.  value = sum >> 32.
+// sum of c Im(conj(w) v) / 2^32 for integer c, |c| <= 2^28, and |components| < 2^59 (up to 8 terms), each
+// term rounded to nearest (rounding down shifts the n = 28 gradient by 2e-12 of its size): the term
+// is P 2^64 + Q 2^32, the low products' share in Q, and each word of P and Q is weighted by c with one
+// multiply-add-wide.
 struct WeightedImSum {
   long long ph = 0, pl = 0, qh = 0, ql = 0;
   QAOA_HD void add(long long vx_, long long vy_, long long wx_, long long wy_, int c) {
     const Limbs vx = split(vx_), vy = split(vy_), wx = split(wx_), wy = split(wy_);
-    const int nwyh = -wy.h, nvxh = -vx.h, wxl = wx.l >> 4, nwyl = -(wy.l >> 4);
-    const long long Lo = madw(nwyl, vx.l, madw(wxl, vy.l, 1ll << 27)) >> 28;
-    const Limbs Q = split(madw(wy.l, nvxh, madw(nwyh, vx.l, madw(wx.l, vy.h, madw(wx.h, vy.l, Lo)))));
+    const int nwyh = -wy.h, nvxh = -vx.h;
+    const long long d = low_diff(vx, vy, wx, wy), carry = (d >> 32) + (long long)((unsigned)d >> 31);
+    const Limbs Q = split(madw(wy.l, nvxh, madw(nwyh, vx.l, madw(wx.l, vy.h, madw(wx.h, vy.l, carry)))));
     const Limbs P = split(madw(nwyh, vx.h, madw(wx.h, vy.h, 0)));
     ph = madw(P.h, c, ph);
     pl = madw(P.l, c, pl);
