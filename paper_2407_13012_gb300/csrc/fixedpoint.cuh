@@ -360,7 +360,8 @@ QAOA_HD double i128_to_double(i128 v, int s) {
   return to_double(neg ? -q : q, s - sh);
 }
 
-// round(d * 2^s) as int64 (half away from zero) for |d| 2^s < 2^62
+// round(d * 2^s) as int64 (half away from zero) for |d| 2^s <= 2^62 (a cost vector's largest entry
+// meets the bound with equality when it is a power of two)
 QAOA_HD long long from_double(double d, int s) {
   const unsigned long long bits = double_to_bits(d);
   const int ex = (int)((bits >> 52) & 0x7FF);
@@ -368,7 +369,7 @@ QAOA_HD long long from_double(double d, int s) {
   const long long m = (long long)((bits & ((1ull << 52) - 1)) | (1ull << 52));
   const int sh = ex - 1075 + s;  // value * 2^s = m * 2^sh
   long long r;
-  if (sh >= 0) r = sh >= 10 ? (m << 9) : (m << sh);  // clamp; callers stay in range
+  if (sh >= 0) r = m << (sh > 10 ? 10 : sh);  // clamp; callers stay in range
   else if (sh > -64) r = (m >> (-sh)) + ((m >> (-sh - 1)) & 1);
   else r = 0;
   return (bits >> 63) ? -r : r;
