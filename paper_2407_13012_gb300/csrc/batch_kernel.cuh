@@ -144,7 +144,10 @@ __global__ void __launch_bounds__(CF::NT, CF::MINB) batch_kernel(const __grid_co
         S s(sa, X, Cs, blk, red);
         s.Ds = dsm;
         s.evalid = 1u << (bs.g.t + bs.g.c);
-        if constexpr (FX) s.lam_shift = G.lam_shift;
+        if constexpr (FX) {
+          s.lam_shift = G.lam_shift;
+          s.c_expo = G.c_expo;
+        }
         if (lean) {
           s.wacc = wacc;
           if (staged) s.dpre = dpre;

@@ -1141,6 +1141,8 @@ int batch_layout(int dtype, int p, int ngraphs, const qaoa_graph_t* gs, const do
     int ls = 0;  // 2^lam_shift >= sum |w| >= max |C|
     while (ls < 62 && std::ldexp(1.0, ls) < sum_abs) ++ls;
     G.lam_shift = ls;
+    G.c_expo = 0;
+    if (sum_abs > 0.0) std::frexp(sum_abs, &G.c_expo);  // sum |w| < 2^c_expo
     const int64_t span = cmax[i] - cmin[i] + 1;
     G.cmin = L.cost_f64 ? 0 : (int)cmin[i];
     G.span = (!L.cost_f64 && span >= 1 && span <= QAOA_MAX_TABLE_SPAN) ? (int)span : 0;
@@ -1344,6 +1346,7 @@ int batch_run(int dtype, int p, const BatchLayout& L, double* out_dev, void* ws_
       g.d_table = fx ? (const void*)((char*)b.dtab + (size_t)k * p * 196 * sizeof(longlong2)) : nullptr;
       g.trig = b.trig + (size_t)k * 3 * p;
       g.lam_shift = G.lam_shift;
+      g.c_expo = G.c_expo;
       rows[k] = G.out;
     }
     if (cudaMemcpyAsync(ws + L.off_gslot, slots.data(), sizeof(GroupSlot) * slots.size(), cudaMemcpyHostToDevice,

@@ -67,7 +67,8 @@ struct GroupSlot {
   int64_t cmin, span;
   const void* d_table;      // fixed point: p * 14 * 14 mixer-diagonal entries
   const double* trig;       // [g2pi p | cos p | sin p]
-  int lam_shift;            // fixed point: 2^lam_shift >= max |C|
+  int lam_shift;            // fixed point: 2^lam_shift >= max |C|, lam_shift >= 0
+  int c_expo;               // the same of any sign
 };
 
 struct SweepArgs {
@@ -280,7 +281,8 @@ struct BatchGraph {
   int n, m;
   int plan;        // index into the plans
   int out;         // output row (the caller's graph index)
-  int lam_shift;   // fixed point: 2^lam_shift >= max |C|
+  int lam_shift;   // fixed point: 2^lam_shift >= max |C|, lam_shift >= 0
+  int c_expo;      // the same of any sign
   int cmin, span;  // integer cost range covered by the phase table (span 0: no table)
   int64_t state;   // element offset of psi and lambda in the state arenas
   int64_t cost;    // element offset of C in the cost arena

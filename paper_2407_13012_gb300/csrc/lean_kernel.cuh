@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(CF::NT, CF::MINB) lean_kernel(const __grid_con
     else facc[r] = make_float2(0.f, 0.f);
     if (r < kLeanAcc) ishift[r] = 0;
   }
-  const CostScan scan = a.half == 2 ? read_scan(a.scan, a.nscan) : CostScan{a.half != 0, 0};
+  const CostScan scan = a.half == 2 ? read_scan(a.scan, a.nscan) : CostScan{a.half != 0, true, 0};
   const SweepGeom g = scan.symmetric ? half_geom(a.g) : a.g;
   S s(a, X, Cs, nullptr, nullptr);
   s.wacc = wacc;
@@ -171,8 +171,9 @@ __global__ void __launch_bounds__(CF::NT, CF::MINB) lean_kernel(const __grid_con
   if constexpr (FX && TWO) {
     if (a.gslot != nullptr) {
       s.lam_shift = a.gslot[blockIdx.x / a.gbpg].lam_shift;
+      s.c_expo = a.gslot[blockIdx.x / a.gbpg].c_expo;
     } else if (a.scan != nullptr) {
-      s.lam_shift = a.half == 2 ? scan.shift : read_scan(a.scan, a.nscan).shift;
+      s.set_scan(a.half == 2 ? scan : read_scan(a.scan, a.nscan));
     }
   }
   __syncthreads();

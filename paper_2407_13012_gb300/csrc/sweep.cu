@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(CF::NT, CF::MINB) sweep_kernel(const __grid_co
   const SweepGeom& g = a.g;
   s.evalid = 1u << (g.t + g.c);
   if constexpr (FX) {
-    if (a.scan != nullptr) s.lam_shift = read_scan(a.scan, a.nscan).shift;
+    if (a.scan != nullptr) s.set_scan(read_scan(a.scan, a.nscan));
     s.in_shift = input_shift(a.norm2_dev);
   }
   for (int64_t tile = blockIdx.x; tile < g.tiles; tile += gridDim.x) sweep_tile<CF, FX, TWO, false>(s, a, tile, Cs);

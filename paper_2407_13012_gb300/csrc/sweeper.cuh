@@ -115,25 +115,31 @@ __device__ __forceinline__ uint64_t tile_base(const SweepGeom& g, int64_t tile) 
   return (lowrest << g.c) | (highrest << (g.j0 + g.t - g.pair));
 }
 // What a scan of C says, read by each warp for itself (a single entry by each thread): whether
-// C(z) = C(~z), and the smallest k >= 0 with 2^k >= max |C|.
+// C(z) = C(~z), whether every entry is finite, and the smallest k with 2^k >= max |C| (0 if C = 0).
 struct CostScan {
-  bool symmetric;
-  int shift;
+  bool symmetric, finite;
+  int expo;
+  __device__ __forceinline__ int lam_shift() const { return max(expo, 0); }
 };
 __device__ __forceinline__ CostScan read_scan(const unsigned long long* scan, int nscan) {
-  bool asym = false;
-  int k = 0;
+  bool asym = false, bad = false;
+  constexpr int kNone = -2000;  // below every exponent
+  int k = kNone;
   auto take = [&](unsigned long long b) {
     const int ex = (int)(b >> 52) & 0x7FF;
     asym |= (b >> 63) != 0;
+    bad |= ex == 0x7FF;
     if (ex != 0) k = max(k, ex - 1023 + ((b & ((1ull << 52) - 1)) != 0 ? 1 : 0));
   };
   if (nscan == 1) {
     take(scan[0]);
-    return {!asym, k};
+  } else {
+    for (int i = threadIdx.x & 31; i < nscan; i += 32) take(scan[i]);
+    asym = __any_sync(0xffffffffu, asym);
+    bad = __any_sync(0xffffffffu, bad);
+    k = __reduce_max_sync(0xffffffffu, k);
   }
-  for (int i = threadIdx.x & 31; i < nscan; i += 32) take(scan[i]);
-  return {!__any_sync(0xffffffffu, asym), __reduce_max_sync(0xffffffffu, k)};
+  return {!asym, !bad, k == kNone ? 0 : k};
 }
 
 // The scale of a user state (complex128): k with |psi| / 2^k in [1, 2), from its norm^2.  The first
@@ -258,6 +264,8 @@ struct Sweeper {
   double* red;   // reduction scratch [2][NT/32]
   int cur;       // current layout
   int lam_shift;  // lambda scale exponent (fixed point)
+  int c_expo = 0;        // fixed point, float64 costs: 2^c_expo >= max |C|
+  bool c_finite = true;  // and no entry of C is infinite or NaN
   int in_shift;   // extra input scale exponent of a user state (fixed point)
   uint32_t evalid;
   uint64_t base;
@@ -281,6 +289,11 @@ struct Sweeper {
     turns = (const longlong2*)a_.turn_table;
   }
 
+  __device__ __forceinline__ void set_scan(const CostScan& c) {
+    lam_shift = c.lam_shift();
+    c_expo = c.expo;
+    c_finite = c.finite;
+  }
   __device__ __forceinline__ uint32_t idx(int r) const { return CF::idx(cur, tid, r); }
 
   // barrier over the exchange group of a move between layouts F and T (Cfg: exchange groups).
@@ -866,19 +879,22 @@ struct Sweeper {
   __device__ __forceinline__ void op_cterm(int acc) {
     const bool f64 = a.cost_dtype == QAOA_COST_F64;
     if constexpr (FX) {
-      if (R <= 8 && f64) {
-        // C psi / 2^lam_shift rounded to the state's resolution (as lambda holds it), then exact
-        // limb sums against lambda / 2^lam_shift
+      if (R <= 8 && f64 && c_finite) {
+        // C psi / 2^c_expo in units of 2^-59 (the state's are 2^-54 on tiles of 2^12), then exact limb
+        // sums against lambda / 2^lam_shift.  (float64 terms, which non-finite costs take below, hold the
+        // float64 pipe for 64 cycles per amplitude and warp.)
+        const int up = 59 - a.fx_shift;
         fx::ImSum sw;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           const uint32_t i = idx(r);
           if (i >= evalid) continue;
-          const fx::Limbs c = fx::split(double_to_fx(cost_f(Cs, true, i), 62 - lam_shift));
-          sw.add(fx::split(fx::mul_unit(v[r].x, c)), fx::split(fx::mul_unit(v[r].y, c)), fx::split(w[r].x),
+          const fx::Limbs c = fx::split(double_to_fx(cost_f(Cs, true, i), 62 - c_expo));
+          sw.add(fx::split(fx::mul_unit((long long)((unsigned long long)v[r].x << up), c)),
+                 fx::split(fx::mul_unit((long long)((unsigned long long)v[r].y << up), c)), fx::split(w[r].x),
                  fx::split(w[r].y));
         }
-        block_add_fx(acc, sw.value(), 2 * a.fx_shift - 2 * lam_shift - 1);
+        block_add_fx(acc, sw.value(), 2 * a.fx_shift + up - lam_shift - c_expo - 1);
       } else if (R <= 8 && lam_shift <= 28) {  // |C| <= 2^28: limb sums (fx::WeightedImSum)
         fx::WeightedImSum sw;
 #pragma unroll
