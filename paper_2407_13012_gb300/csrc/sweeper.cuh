@@ -189,6 +189,12 @@ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = t;
 }
 
+// lane 0 adds the warp's sum of v to *slot (out of line: the rare form of block_add_f32)
+__device__ __noinline__ void warp_add_f64(double* slot, double v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) *slot += v;
+}
+
 // exp(-2 pi i th) in float32 for a turn count th (the path of float costs or costs outside the
 // table); kept out of line so it does not raise the register budget of the common path.  The
 // fraction of the turn comes from the integer bits (its float64 rounding, subtraction and
@@ -438,12 +444,19 @@ struct Sweeper {
     if ((tid & 31) == 0) iacc[r * (CF::NT / 32) + (tid >> 5)] += v;
     if (tid == 0) ishift[r] = shift;
   }
-  // add the block's sum of the float32 v to accumulator r
-  __device__ __forceinline__ void block_add_f32(int r, float v) {
+  // add f times the block's sum of the float32 v to accumulator r
+  __device__ __forceinline__ void block_add_f32(int r, float v, float f = 1.f) {
     if (facc == nullptr) {
-      block_add(r, (double)v, 0.0, false);
+      block_add(r, (double)f * (double)v, 0.0, false);
       return;
     }
+    // double-float keeps float32's range: sums that may pass it (states or costs of huge norm), infinities
+    // and NaN go to the float64 slots
+    if (__any_sync(0xffffffffu, !(fabsf(v) < 0x1.0p100f))) {
+      warp_add_f64(wacc + r * (CF::NT / 32) + (tid >> 5), (double)f * (double)v);
+      return;
+    }
+    v *= f;
     float c = 0.f;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -715,7 +728,7 @@ struct Sweeper {
       if (on_psi) scale_f32(v, f);
       if (TWO && on_lam) scale_f32(w, f);
     }
-    if (xt) block_add_f32(xacc, 2.f * xs);
+    if (xt) block_add_f32(xacc, xs, 2.f);
   }
 
   // ---------------------------------------------------------------- mixer, fixed point: W D W
@@ -925,7 +938,7 @@ struct Sweeper {
         if (i >= evalid) continue;
         s[r & 3] += cost32_at(f64, r) * (w[r].x * v[r].y - w[r].y * v[r].x);
       }
-      block_add_f32(acc, 2.f * ((s[0] + s[1]) + (s[2] + s[3])));
+      block_add_f32(acc, (s[0] + s[1]) + (s[2] + s[3]), 2.f);
     }
   }
 };
@@ -1375,7 +1388,7 @@ struct Lean : Sweeper<CF, FX, TWO> {
       f32_fwd<0, L>(q.tanf, q.tu, q.m * q.m, xt, xs, w2);
       scale_axis(this->v, q.f, q.real);
       if constexpr (TWO) scale_axis(this->w, q.f, q.real);
-      if (xt) this->block_add_f32(xacc, 2.f * xs);
+      if (xt) this->block_add_f32(xacc, xs, 2.f);
       if constexpr (L > 0) exb<L, 0>();
     }
   }
