@@ -159,8 +159,8 @@ __global__ void __launch_bounds__(kPrepThreads) batch_prep_kernel(const __grid_c
       double* out = (double*)b.C + G.cost;
       batch_costs<long long>(G.n, e_s, w_s, G.m, z0, W_s, tab_s, [&](uint32_t z, const long long(&s)[16]) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i)
-          if (i < live) out[z + i] = fx::to_double(s[i], shift_s);
+        for (int i = 0; i < 16; ++i)  // (to_double forms normal numbers: every entry's are down to 2^-1022)
+          if (i < live) out[z + i] = shift_s <= 1022 ? fx::to_double(s[i], shift_s) : ldexp((double)s[i], -shift_s);
       });
     } else {
       int* out = (int*)b.C + G.cost;
