@@ -378,8 +378,8 @@ void qaoa_launch_count_reset(void);
  * events and writes, per class (arrays of 4, any may be NULL), the summed
  * milliseconds, the launch count and the algorithmic HBM bytes of those
  * launches (each state, lambda and cost-vector element read or written once
- * per launch; half of them where a call may sweep half a state, which the
- * device decides), then clears them.  At most 65536 launches are recorded between
+ * per launch; where a call swept half a state, of that half and of the stores
+ * that complete it), then clears them.  At most 65536 launches are recorded between
  * reads; later ones are counted in *dropped but not timed.
  */
 int qaoa_timing_enable(int on);

@@ -26,12 +26,22 @@ constexpr int kMaxTimed = 65536;
 struct TimedLaunch {
   cudaEvent_t e0, e1;
   int kind;
-  double bytes;
+  double bytes, half_bytes;
+  int slot;
 };
 std::vector<TimedLaunch> g_timed;
 std::vector<cudaEvent_t> g_event_pool;
 int64_t g_dropped = 0;
 cudaEvent_t g_pending_begin = nullptr;
+// pinned host words, one per timed call that may sweep half a state: 0 once the device has done so
+unsigned* g_flags = nullptr;
+int g_flags_used = 0;
+
+bool timing_now(cudaStream_t s) {
+  if (!g_timing_on) return false;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  return !(cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone);  // graph capture
+}
 
 cudaEvent_t pool_event() {
   if (!g_event_pool.empty()) {
@@ -45,11 +55,18 @@ cudaEvent_t pool_event() {
 }
 }  // namespace
 
-void note_launch(int kind, cudaStream_t s, bool begin, double bytes) {
+unsigned* timing_flag(cudaStream_t s, int* slot) {
+  *slot = 0;
+  if (!timing_now(s)) return nullptr;
+  std::lock_guard<std::mutex> lk(g_timing_mu);
+  if (g_flags == nullptr || g_flags_used >= kMaxTimed) return nullptr;
+  *slot = ++g_flags_used;
+  return g_flags + (*slot - 1);
+}
+
+void note_launch(int kind, cudaStream_t s, bool begin, double bytes, double half_bytes, int slot) {
   if (begin) g_launches.fetch_add(1, std::memory_order_relaxed);
-  if (!g_timing_on) return;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone) return;  // graph capture
+  if (!timing_now(s)) return;
   std::lock_guard<std::mutex> lk(g_timing_mu);
   if (begin) {
     if ((int)g_timed.size() >= kMaxTimed) {
@@ -62,7 +79,7 @@ void note_launch(int kind, cudaStream_t s, bool begin, double bytes) {
   } else if (g_pending_begin != nullptr) {
     cudaEvent_t e1 = pool_event();
     cudaEventRecord(e1, s);
-    g_timed.push_back({g_pending_begin, e1, kind, bytes});
+    g_timed.push_back({g_pending_begin, e1, kind, bytes, half_bytes, slot});
     g_pending_begin = nullptr;
   }
 }
@@ -301,6 +318,13 @@ static int run_sweeps(const Ctx& c, std::vector<Sweep>& sw, const std::vector<Gr
     rc = cuda_status(launch_reduce(r, norm_part, norm2, c.s));
     if (rc) return rc;
   }
+  int slot = 0;  // timing: whether C was symmetric decides the bytes of the sweeps
+  if (half) {
+    if (unsigned* flag = timing_flag(c.s, &slot)) {
+      int rc = cuda_status(launch_scan_flag(scan, nscan, flag, c.s));
+      if (rc) return rc;
+    }
+  }
   const double amp0 = std::pow(2.0, -0.5 * c.n);
   const int S = fx_shift_for(tmax);
   for (const Sweep& s : sw) {
@@ -367,7 +391,9 @@ static int run_sweeps(const Ctx& c, std::vector<Sweep>& sw, const std::vector<Gr
       const double per = S_b * ((s.init ? 0 : 1) + (s.store_psi ? 1 : 0) + (s.two && s.load_lam ? 1 : 0) +
                                 (s.two && s.store_lam ? 1 : 0)) +
                          (reads_c ? cb : 0.0);
-      a.algo_bytes = per * (double)(1ull << (c.n - half));  // (only the device knows whether C is symmetric)
+      a.algo_bytes = per * (double)(1ull << c.n);
+      a.half_bytes = (per + (a.mirror ? S_b : 0.0)) * (double)(1ull << (c.n - 1));
+      a.timing_slot = slot;
     }
     a.kind = lean_kind(s, g, tile_bits, c.dtype);
     if (a.mirror) a.kind = SWEEP_LEAN_OPS;  // (the plain mixer kernels store no complements)
@@ -1563,6 +1589,9 @@ void qaoa_launch_count_reset(void) { g_launches.store(0); }
 
 int qaoa_timing_enable(int on) {
   std::lock_guard<std::mutex> lk(g_timing_mu);
+  if (on && g_flags == nullptr &&
+      cudaHostAlloc((void**)&g_flags, kMaxTimed * sizeof(unsigned), cudaHostAllocPortable) != cudaSuccess)
+    g_flags = nullptr;  // calls that may sweep half a state then count as whole
   g_timing_on = on != 0;
   return QAOA_OK;
 }
@@ -1582,12 +1611,13 @@ int qaoa_timing_read(double* ms, int64_t* launches, double* bytes, int64_t* drop
     if (t.kind >= 0 && t.kind < 4) {
       if (ms) ms[t.kind] += f;
       if (launches) launches[t.kind] += 1;
-      if (bytes) bytes[t.kind] += t.bytes;
+      if (bytes) bytes[t.kind] += t.slot > 0 && g_flags[t.slot - 1] == 0 ? t.half_bytes : t.bytes;
     }
     g_event_pool.push_back(t.e0);
     g_event_pool.push_back(t.e1);
   }
   g_timed.clear();
+  g_flags_used = 0;
   if (dropped) *dropped = g_dropped;
   g_dropped = 0;
   return rc;

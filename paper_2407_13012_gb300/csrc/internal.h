@@ -128,7 +128,9 @@ struct SweepArgs {
   int red_slot[kMaxAcc];
   double* partials;
   int grid;
-  double algo_bytes;  // HBM bytes this sweep must move (for timing reports)
+  // for timing reports: HBM bytes this sweep must move, on half the state, and the call's slot (timing_flag)
+  double algo_bytes, half_bytes;
+  int timing_slot;
   // grouped sweeps (lean kernels only): per-graph data, blocks per graph; nullptr = one graph
   const GroupSlot* gslot;
   int gbpg;
@@ -183,6 +185,8 @@ cudaError_t launch_tables(const TableArgs& t, cudaStream_t s);
 constexpr int kMaxScan = 256;
 int cost_scan_blocks(int n);
 cudaError_t launch_cost_scan(const void* C, int f64, int n, unsigned long long* scan, const TableArgs& t, cudaStream_t s);
+// *flag (host memory the device can write) = 0 if the scanned C is symmetric, else 1
+cudaError_t launch_scan_flag(const unsigned long long* scan, int nscan, unsigned* flag, cudaStream_t s);
 cudaError_t launch_norm(const void* psi, int dtype, int n, double* partials, int* nblocks, cudaStream_t s);
 cudaError_t launch_adam(double* ang, const double* g, double* state, long long* step, int p, double lr, double b1,
                         double b2, double eps, double* history, long long row0, long long max_rows, cudaStream_t s);
@@ -247,7 +251,10 @@ size_t sample_ws_bytes_len(uint64_t len);  // workspace for a vector of len entr
 
 // bookkeeping for benchmarks: call with begin = true before a launch and begin = false
 // after it; `bytes` (algorithmic HBM bytes of the launch) is read on the second call
-void note_launch(int kind, cudaStream_t s, bool begin, double bytes = 0.0);
+void note_launch(int kind, cudaStream_t s, bool begin, double bytes = 0.0, double half_bytes = 0.0, int slot = 0);
+// while launches are timed (else nullptr, *slot = 0): a host word for this call, in which the device leaves 0
+// if C was symmetric; note_launch with this slot then counts half_bytes instead of bytes
+unsigned* timing_flag(cudaStream_t s, int* slot);
 
 // ---------------------------------------------------------------- batched gradients
 //

@@ -196,6 +196,11 @@ __global__ void __launch_bounds__(1024) cost_scan_kernel(const T* __restrict__ C
   }
 }
 
+__global__ void scan_flag_kernel(const unsigned long long* __restrict__ scan, int nscan, unsigned* flag) {
+  const bool symmetric = read_scan(scan, nscan).symmetric;
+  if (threadIdx.x == 0) *flag = symmetric ? 0u : 1u;
+}
+
 // state norm^2 of a user (float64 / float32) state, for the fixed-point input scale
 __global__ void norm_kernel(const void* __restrict__ psi, int dtype, int64_t count, double* __restrict__ partials) {
   double s = 0.0;
@@ -389,7 +394,7 @@ cudaError_t launch_sweep(int dtype, bool two, const SweepArgs& a, cudaStream_t s
     if (two) launch_t<CfgF3, false, true>(a, s);
     else launch_t<CfgF1, false, false>(a, s);
   }
-  note_launch(0, s, false, a.algo_bytes);
+  note_launch(0, s, false, a.algo_bytes, a.half_bytes, a.timing_slot);
   return cudaGetLastError();
 }
 
@@ -433,6 +438,13 @@ cudaError_t launch_tables(const TableArgs& t, cudaStream_t s) {
   const int64_t blocks = std::min<int64_t>((total + 31) / 32, 4096);
   note_launch(3, s, true);
   tables_kernel<<<(int)blocks, 32, 0, s>>>(t);
+  note_launch(3, s, false);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_scan_flag(const unsigned long long* scan, int nscan, unsigned* flag, cudaStream_t s) {
+  note_launch(3, s, true);
+  scan_flag_kernel<<<1, 32, 0, s>>>(scan, nscan, flag);
   note_launch(3, s, false);
   return cudaGetLastError();
 }

@@ -1043,12 +1043,13 @@ bool cost_ok(const qaoa_cost_t* c) {
 
 template <typename T>
 int expectation_t(const XYShape& s, const T* psi, const qaoa_cost_t* cost, double* out, double* part,
-                  cudaStream_t st, const unsigned* half_flag = nullptr) {
+                  cudaStream_t st, const unsigned* half_flag = nullptr, int slot = 0) {
   const int most = kXYRedBlocks - (half_flag != nullptr);  // (the flag lies in the last block's slots)
   const int nb = (int)(s.D < (unsigned long long)most * kXYThreads ? (s.D + kXYThreads - 1) / kXYThreads : most);
   note_launch(3, st, true);
   xy_expect_kernel<T><<<nb, kXYThreads, 0, st>>>(psi, cost->C_dev, cost->dtype, s.D, part, half_flag);
-  note_launch(3, st, false, (double)s.D * (sizeof(T) + cost_bytes(cost->dtype)));
+  const double bytes = (double)s.D * (sizeof(T) + cost_bytes(cost->dtype));
+  note_launch(3, st, false, bytes, bytes / 2, slot);
   note_launch(3, st, true);
   xy_finish_kernel<<<1, kXYThreads, 0, st>>>(part, nb, out, half_flag);
   note_launch(3, st, false);
@@ -1098,7 +1099,7 @@ XYMixPlan* make_mix_plan(const XYShape& s, const unsigned* half_flag) {
 template <typename T, bool TWO, bool PH, bool FOLD>
 cudaError_t launch_window_as(const xyw::Window& W, T* psi, T* lam, typename Real<T>::type cb,
                           typename Real<T>::type sb, double* part, int part_cols, const XYPhaseArgs<T>& ph,
-                          cudaStream_t st) {
+                          cudaStream_t st, int slot) {
   static std::mutex mu;
   static unsigned long long done = 0;
   static int per_sm[64] = {};
@@ -1124,41 +1125,40 @@ cudaError_t launch_window_as(const xyw::Window& W, T* psi, T* lam, typename Real
   unsigned long long g = (unsigned long long)sm_count() * resident;
   if (TWO && g > (unsigned long long)part_cols) g = part_cols;
   const unsigned grid = (unsigned)(W.tiles < g ? W.tiles : g);
-  // (only the device knows whether C is symmetric)
-  const double elems = W.f.flag == nullptr ? (double)W.elems : W.nh == 0 && !FOLD ? 0.0 : (double)W.half_elems;
-  const double cb_bytes = PH ? elems * cost_bytes(ph.cost_dtype) : 0.0;
-  const double bytes = elems * sizeof(T) * 2 * (TWO ? 2 : 1) + cb_bytes;
+  const double each = (double)sizeof(T) * 2 * (TWO ? 2 : 1) + (PH ? cost_bytes(ph.cost_dtype) : 0.0);
+  const double whole = FOLD ? 0.0 : each * (double)W.elems;
+  const double half = !FOLD && W.nh == 0 ? 0.0 : each * (double)W.half_elems;
   note_launch(0, st, true);
   xy_window_kernel<T, TWO, PH, FOLD><<<grid, NT, smem, st>>>(W, psi, lam, cb, sb, part, part_cols, ph);
-  note_launch(0, st, false, bytes);
+  note_launch(0, st, false, whole, half, slot);
   return cudaGetLastError();
 }
 
 template <typename T, bool TWO, bool PH>
 cudaError_t launch_window(const xyw::Window& W, T* psi, T* lam, typename Real<T>::type cb,
                           typename Real<T>::type sb, double* part, int part_cols, const XYPhaseArgs<T>& ph,
-                          cudaStream_t st) {
+                          cudaStream_t st, int slot) {
   if constexpr (!PH)
     if (W.f.flag != nullptr && W.nh == 0) {
-      const cudaError_t e = launch_window_as<T, TWO, false, true>(W, psi, lam, cb, sb, part, part_cols, ph, st);
+      const cudaError_t e = launch_window_as<T, TWO, false, true>(W, psi, lam, cb, sb, part, part_cols, ph, st, slot);
       if (e != cudaSuccess) return e;
     }
-  return launch_window_as<T, TWO, PH, false>(W, psi, lam, cb, sb, part, part_cols, ph, st);
+  return launch_window_as<T, TWO, PH, false>(W, psi, lam, cb, sb, part, part_cols, ph, st, slot);
 }
 
 template <typename T, bool TWO>
 void launch_closing(const xyw::Closing& W, T* psi, T* lam, typename Real<T>::type cb, typename Real<T>::type sb,
-                    double* part, unsigned grid, cudaStream_t st) {
-  const double pairs = (double)(W.f.flag != nullptr ? W.half_pairs : W.pairs);
+                    double* part, unsigned grid, cudaStream_t st, int slot) {
+  const double each = 2.0 * sizeof(T) * (TWO ? 4 : 2);
   note_launch(0, st, true);
   if (W.f.flag != nullptr) xy_closing_kernel<T, TWO, true><<<grid, kXYThreads, 0, st>>>(W, psi, lam, cb, sb, part);
   xy_closing_kernel<T, TWO, false><<<grid, kXYThreads, 0, st>>>(W, psi, lam, cb, sb, part);
-  note_launch(0, st, false, pairs * 2 * sizeof(T) * (TWO ? 4 : 2));
+  note_launch(0, st, false, each * (double)W.pairs, each * (double)W.half_pairs, slot);
 }
 
 template <typename T>
 int layers_t(const XYShape& s, T* psi, const qaoa_cost_t* cost, const double* gamma, const double* beta, int p,
-             int init, double* expect_dev, char* ws, cudaStream_t st, bool whole = true) {
+             int init, double* expect_dev, char* ws, cudaStream_t st, bool whole = true, int* slot_out = nullptr) {
   using R = typename Real<T>::type;
   const int sms = sm_count();
   const size_t sb = sizeof(T);
@@ -1176,10 +1176,14 @@ int layers_t(const XYShape& s, T* psi, const qaoa_cost_t* cost, const double* ga
       xy_symmetry_kernel<<<(unsigned)sms * 8, kXYThreads, 0, st>>>((const unsigned*)cost->C_dev, s.D, flag);
     note_launch(3, st, false, (double)s.D * cost_bytes(cost->dtype));
   }
+  int slot = 0;  // timing: whether C was symmetric decides the bytes of the passes
+  if (half)
+    if (unsigned* word = timing_flag(st, &slot)) cudaMemcpyAsync(word, flag, sizeof(unsigned), cudaMemcpyDeviceToHost, st);
+  if (slot_out != nullptr) *slot_out = slot;
   if (init) {
     note_launch(3, st, true);
     xy_init_kernel<T><<<grid_for(s.D, sms), kXYThreads, 0, st>>>(psi, s.D, 1.0 / std::sqrt((double)s.D), flag);
-    note_launch(3, st, false, (double)s.D * sb);
+    note_launch(3, st, false, (double)s.D * sb, (double)s.D * sb / 2, slot);
   }
   if (tab != nullptr) {
     XYTableArgs ta;
@@ -1209,8 +1213,8 @@ int layers_t(const XYShape& s, T* psi, const qaoa_cost_t* cost, const double* ga
     if (mp != nullptr) {  // the cost unitary on the first window's pass, the ring mixer, the closing pair
       for (int i = 0; i < mp->nwin; ++i) {
         const cudaError_t e =
-            i == 0 ? launch_window<T, false, true>(mp->win[i], psi, nullptr, cb, snb, nullptr, 0, ph, st)
-                   : launch_window<T, false, false>(mp->win[i], psi, nullptr, cb, snb, nullptr, 0, ph, st);
+            i == 0 ? launch_window<T, false, true>(mp->win[i], psi, nullptr, cb, snb, nullptr, 0, ph, st, slot)
+                   : launch_window<T, false, false>(mp->win[i], psi, nullptr, cb, snb, nullptr, 0, ph, st, slot);
         if (e != cudaSuccess) {
           delete mp;
           return QAOA_ERR_CUDA;
@@ -1219,7 +1223,7 @@ int layers_t(const XYShape& s, T* psi, const qaoa_cost_t* cost, const double* ga
       if (mp->closing) {
         const unsigned long long most = std::min<unsigned long long>(mp->close.tiles, (unsigned)sms * 6u);
         launch_closing<T, false>(mp->close, psi, nullptr, cb, snb, nullptr,
-                                 (unsigned)std::max<unsigned long long>(1, most), st);
+                                 (unsigned)std::max<unsigned long long>(1, most), st, slot);
       }
     }
     const int rc = status_of(cudaGetLastError());
@@ -1232,9 +1236,9 @@ int layers_t(const XYShape& s, T* psi, const qaoa_cost_t* cost, const double* ga
   if (half && whole) {
     note_launch(3, st, true);
     xy_mirror_kernel<T><<<(unsigned)sms * 8, kXYThreads, 0, st>>>(psi, s.D, flag);
-    note_launch(3, st, false, (double)s.D * sb);
+    note_launch(3, st, false, 0.0, (double)s.D * sb, slot);
   }
-  if (expect_dev != nullptr) return expectation_t<T>(s, psi, cost, expect_dev, part, st, flag);
+  if (expect_dev != nullptr) return expectation_t<T>(s, psi, cost, expect_dev, part, st, flag, slot);
   return status_of(cudaGetLastError());
 }
 
@@ -1253,7 +1257,8 @@ int gradient_t(const XYShape& s, T* psi, T* lam, const qaoa_cost_t* cost, const 
   const int sms = sm_count();
   const size_t sb = sizeof(T);
   // forward pass (Dicke start, p layers) with the layer workspace at the front
-  int rc = layers_t<T>(s, psi, cost, gamma, beta, p, 1, nullptr, ws, st, false);
+  int slot = 0;
+  int rc = layers_t<T>(s, psi, cost, gamma, beta, p, 1, nullptr, ws, st, false, &slot);
   if (rc) return rc;
   const long long span = p > 0 ? table_span(cost) : 0;
   const T* tab = span > 0 ? (const T*)(ws + round256(2 * (size_t)kXYRedBlocks * sizeof(double))) : nullptr;
@@ -1268,7 +1273,8 @@ int gradient_t(const XYShape& s, T* psi, T* lam, const qaoa_cost_t* cost, const 
   note_launch(0, st, true);
   xy_lambda_kernel<T><<<gr, kXYThreads, 0, st>>>(psi, lam, cost->C_dev, cost->dtype, s.D, part, part + kXYPartStride,
                                                  flag);
-  note_launch(0, st, false, (double)s.D * (2 * sb + cost_bytes(cost->dtype)));
+  const double lbytes = (double)s.D * (2 * sb + cost_bytes(cost->dtype));
+  note_launch(0, st, false, lbytes, lbytes / 2, slot);
   // beta rows of layer l: one per window and one for the closing pair (at most np of them), every row's gg slots written
   XYMixPlan* mp = np > 0 && p > 0 ? make_mix_plan<T>(s, flag) : nullptr;
   const int brows = mp != nullptr ? mp->nwin + (mp->closing ? 1 : 0) : 0;
@@ -1278,14 +1284,15 @@ int gradient_t(const XYShape& s, T* psi, T* lam, const qaoa_cost_t* cost, const 
     double* rows = part + (size_t)(2 + p + (size_t)l * np) * kXYPartStride;
     if (mp != nullptr) {
       if (mp->closing)  // applied last in the layer, undone first
-        launch_closing<T, true>(mp->close, psi, lam, cb, snb, rows + (size_t)mp->nwin * kXYPartStride, gg, st);
+        launch_closing<T, true>(mp->close, psi, lam, cb, snb, rows + (size_t)mp->nwin * kXYPartStride, gg, st,
+                                slot);
       // the first window's pass also takes the gamma term and undoes the cost unitary
       const XYPhaseArgs<T> ph = {cost->C_dev, cost->dtype, tab ? tab + (size_t)l * span : nullptr, cost->cmin,
                                  span, gamma[l], part + (size_t)(2 + l) * kXYPartStride};
       for (int i = mp->nwin - 1; i >= 0; --i) {
         double* row = rows + (size_t)i * kXYPartStride;
-        const cudaError_t e = i == 0 ? launch_window<T, true, true>(mp->win[i], psi, lam, cb, snb, row, (int)gg, ph, st)
-                                     : launch_window<T, true, false>(mp->win[i], psi, lam, cb, snb, row, (int)gg, ph, st);
+        const cudaError_t e = i == 0 ? launch_window<T, true, true>(mp->win[i], psi, lam, cb, snb, row, (int)gg, ph, st, slot)
+                                     : launch_window<T, true, false>(mp->win[i], psi, lam, cb, snb, row, (int)gg, ph, st, slot);
         if (e != cudaSuccess) {
           delete mp;
           return QAOA_ERR_CUDA;
@@ -1307,7 +1314,7 @@ int gradient_t(const XYShape& s, T* psi, T* lam, const qaoa_cost_t* cost, const 
   if (half) {
     note_launch(3, st, true);
     xy_mirror_kernel<T><<<(unsigned)sms * 8, kXYThreads, 0, st>>>(psi, s.D, flag);
-    note_launch(3, st, false, (double)s.D * sb);
+    note_launch(3, st, false, 0.0, (double)s.D * sb, slot);
   }
   delete mp;
   XYReducePlan rp;
