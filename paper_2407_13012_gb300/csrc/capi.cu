@@ -302,7 +302,7 @@ static int run_sweeps(const Ctx& c, std::vector<Sweep>& sw, const std::vector<Gr
   if (scan_now) {
     TableArgs none;
     std::memset(&none, 0, sizeof(none));
-    int rc = cuda_status(launch_cost_scan(c.cost->C_dev, c.cost->dtype == QAOA_COST_F64, c.n, scan, ride ? t : none, c.s));
+    int rc = cuda_status(launch_cost_scan(c.cost->C_dev, c.cost->dtype == QAOA_COST_F64, c.n, any_two, scan, ride ? t : none, c.s));
     if (rc) return rc;
   }
   if (fx && any_user_load) {  // input scale from |psi|^2 of the caller's state

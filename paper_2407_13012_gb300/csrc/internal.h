@@ -184,7 +184,9 @@ cudaError_t launch_tables(const TableArgs& t, cudaStream_t s);
 // t: tables to build in the same launch (t.p = 0: none)
 constexpr int kMaxScan = 256;
 int cost_scan_blocks(int n);
-cudaError_t launch_cost_scan(const void* C, int f64, int n, unsigned long long* scan, const TableArgs& t, cudaStream_t s);
+// bound: max |C| is wanted, not only whether C is symmetric
+cudaError_t launch_cost_scan(const void* C, int f64, int n, int bound, unsigned long long* scan, const TableArgs& t,
+                             cudaStream_t s);
 // *flag (host memory the device can write) = 0 if the scanned C is symmetric, else 1
 cudaError_t launch_scan_flag(const unsigned long long* scan, int nscan, unsigned* flag, cudaStream_t s);
 cudaError_t launch_norm(const void* psi, int dtype, int n, double* partials, int* nblocks, cudaStream_t s);

@@ -165,14 +165,20 @@ __device__ __forceinline__ float2 phase_of(double theta, float2*) {
   return make_float2(cs, -sn);
 }
 
-// *asym = 1 if C[i] != C[D - 1 - i] (bitwise) for some i (cleared by the caller)
+// *asym = 1 if C[i] != C[D - 1 - i] (bitwise) for some i (cleared by the caller); a thread that has met
+// such a pair stops
 template <class C>
 __global__ void xy_symmetry_kernel(const C* __restrict__ c, unsigned long long D, unsigned* asym) {
   bool bad = false;
-#pragma unroll 4
-  for (unsigned long long r = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; r < D / 2;
-       r += (unsigned long long)gridDim.x * blockDim.x)
-    bad |= __ldg(c + r) != __ldg(c + (D - 1 - r));
+  const unsigned long long step = (unsigned long long)gridDim.x * blockDim.x;
+  for (unsigned long long r0 = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; r0 < D / 2 && !bad;
+       r0 += 4 * step) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const unsigned long long r = r0 + u * step;
+      if (r < D / 2) bad |= __ldg(c + r) != __ldg(c + (D - 1 - r));
+    }
+  }
   if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(asym, 1u);
 }
 
@@ -1070,7 +1076,7 @@ struct XYMixPlan {
 // (xy_window.cuh).  Whole -> half: n = 26, p = 1 layers 1057 -> 597 us complex128, 400 -> 280 complex64,
 // p = 4 gradient 13.9 -> 7.2 and 4.54 -> 2.53 ms; n = 30, p = 3 complex128 layers 48.0 -> 25.5 ms.  A cost that
 // is not symmetric pays for the read of C and the launches that return at once: n = 26, p = 1 layers 1057 ->
-// 1077 us complex128, 400 -> 431 complex64, n = 28 4033 -> 4070 and 1647 -> 1695; below n = 26 that share grows.
+// 1070 us complex128, 400 -> 422 complex64, n = 28 4033 -> 4030 and 1647 -> 1650; below n = 26 that share grows.
 constexpr int kXYHalfMinN = 26;
 // (the last slot of the expectation's partials, which half calls leave alone)
 unsigned* half_flag_at(char* ws) { return (unsigned*)((double*)ws + 2 * kXYRedBlocks - 1); }
