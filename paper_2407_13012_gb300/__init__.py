@@ -13,7 +13,6 @@ psi *= exp(-i gamma C) followed by RX(2 beta) on every qubit.
 from __future__ import annotations
 
 import ctypes as ct
-import functools
 from dataclasses import dataclass
 from pathlib import Path
 

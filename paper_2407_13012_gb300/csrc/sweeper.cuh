@@ -1146,7 +1146,7 @@ struct Lean : Sweeper<CF, FX, TWO> {
   // mixer diagonals of the launch's mixers, staged once in shared memory ([kLeanMix][16]),
   // or nullptr: each mixer then stages its own between block barriers
   const fx::Factor* dpre = nullptr;
-  const F32Mix* fpre = nullptr;  // float32: the mixers' coefficients, staged likewise
+  const F32Mix* fpre = nullptr;  // float32: the mixers' coefficients, always staged
 
   // group-qubit register bits of round K (relative to lo(K)), uniform
   template <int K>
@@ -1382,7 +1382,7 @@ struct Lean : Sweeper<CF, FX, TWO> {
   template <int L>
   __device__ __forceinline__ void f32_mixer(int layer, bool inverse, int xacc, int mix) {
     if constexpr (!FX) {
-      const F32Mix q = fpre != nullptr ? fpre[mix] : f32_mix(this->a, this->trig, layer, inverse, gt());
+      const F32Mix q = fpre[mix];
       const bool xt = TWO && xacc >= 0;
       float xs = 0.f, w2 = 1.f;
       f32_fwd<0, L>(q.tanf, q.tu, q.m * q.m, xt, xs, w2);
