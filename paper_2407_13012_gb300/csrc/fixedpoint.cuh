@@ -414,8 +414,9 @@ QAOA_HD float two_turns_f32(double d) {
 
 // exp(-2 pi i t / 2^64) in Q62: two 256-entry tables (tt[k] = exp(-2 pi i k / 2^8), tt[256 + k] =
 // exp(-2 pi i k / 2^16)) take the turn's nearest multiple of 2^-16, and the residual angle rho
-// (below 2^-13.3) enters as (1 - rho^2/2) - i (rho - rho^3/6), to 2^-57 (the next term is
-// rho^4/24).  The tables are 8 KB, so a sweep holds them in shared memory beside its cost tile;
+// (at most pi 2^-16 = 2^-14.35) enters as (1 - rho^2/2) - i (rho - rho^3/6), to 2^-57: rho is cut to 44
+// bits for its powers, which is 2^-58.3 of rho^2/2, and that to 2^-58; the next term, rho^4/24, is
+// 2^-62.  The tables are 8 KB, so a sweep holds them in shared memory beside its cost tile;
 // three 1024-entry tables with a first-order residual (to 2^-55) took three reads from L2 and two
 // 128-bit complex products per amplitude.
 template <class E>

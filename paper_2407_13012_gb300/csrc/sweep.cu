@@ -352,9 +352,12 @@ __global__ void expect_kernel(const void* __restrict__ psi, const void* __restri
 
 }  // namespace
 
-// complex128 sweeps of up to kSmallTileN qubits run on 512-amplitude tiles (two groups, so the
-// same number of sweeps as on 4096-amplitude tiles): they fill the chip better while the large
-// tiles of such a state are fewer than its SMs.  Measured, 4096- -> 512-amplitude tiles: n = 14, p = 4,
+// complex128 sweeps of up to kSmallTileN qubits run on 512-amplitude tiles (from n = 13 on in two groups
+// like 4096-amplitude tiles, so in as many sweeps): they fill the chip better while the large tiles of
+// such a state are fewer than its SMs.  At n = 10..12, where one 4096-amplitude tile takes the whole
+// circuit in one launch, two groups of small tiles are still faster: p = 6 layers 84 -> 62 us (n = 10) and
+// 92 -> 56 (n = 12), p = 1 33 -> 24 and 27 -> 24, p = 6 gradient 270 -> 173 and 284 -> 156.  Measured,
+// 4096- -> 512-amplitude tiles: n = 14, p = 4,
 // 50 Adam steps 12.4 -> 5.5 ms; n = 16 and 18, p = 6 gradients 353 -> 175 and 366 -> 266 us; n = 17,
 // p = 6 layers 151 -> 88 us.  n = 19 (4096- -> 1024-amplitude tiles, half states): p = 6 layers 151 -> 118 us,
 // gradient 383 -> 314 us, 50 Adam steps 12.3 -> 10.2 ms.  At n = 20 those lose: layers 151 -> 153, gradient

@@ -21,9 +21,11 @@
 //    group of t qubits uses RX(2b)^{(x)t} = H^{(x)t} D H^{(x)t} = 2^-t W D W, where W is
 //    the unnormalised Walsh-Hadamard transform on the group (exact integer add/sub
 //    butterflies) and D = diag(exp(-i b (t - 2 popcount(g)))) is one complex multiply
-//    per amplitude, rounded once.  Phase factors are Q62 fixed point.  Reductions
-//    accumulate exact int128 products per thread and per tile and are converted to
-//    float64 once per tile.
+//    per amplitude, rounded once.  Phase factors are Q62 fixed point.  Reductions are
+//    integer sums: 128-bit ones, or limb sums that give the same (fixedpoint.cuh), of products
+//    that are exact or, where an integer cost weights them, rounded at 2^32 of 2^108.  Lean kernels
+//    carry them in 128 bits through the launch, the others convert to float64 once per tile;
+//    only <C> of float64 costs is summed in float64.
 #pragma once
 
 #include "internal.h"
