@@ -99,8 +99,8 @@ def workload_name(a):
 # an amplitude of magnitude 2^-15 (n = 30) carries ~39 significant bits, not float64's 53.
 ARITHMETIC = {
     "c128": "int64 fixed point, value = integer x 2^-54 (Q54), inside each call; float64 pairs (complex128) "
-            "in memory between calls; reductions exact in int128, converted to float64",
-    "c64": "float32 (complex64 state), reductions accumulated in float64",
+            "in memory between calls; reductions as integer sums of up to 128 bits, converted to float64",
+    "c64": "float32 (complex64 state), threads' float32 sums added up in double-float and float64",
 }
 
 
@@ -195,7 +195,9 @@ def measured_peak_hbm():
         return 6800.0, "fallback"
 
 
-SWEEP_SOURCES = ("sweep.cu", "sweeper.cuh", "lean_kernel.cuh", "tile_layout.cuh", "fixedpoint.cuh", "internal.h", "capi.cu")
+SWEEP_SOURCES = ("sweep.cu", "sweeper.cuh", "lean_kernel.cuh", "lean_f1.cu", "lean_f1d.cu", "lean_f2.cu", "lean_x1.cu",
+                 "lean_x2_mix.cu", "lean_x2_ops.cu", "lean_xm.cu", "lean_xt.cu", "tile_layout.cuh", "fixedpoint.cuh",
+                 "internal.h", "capi.cu")
 
 
 def sweep_source_hash() -> str:
